@@ -105,15 +105,11 @@ enum { SMG_KRYLOV_PCG = 0, SMG_KRYLOV_FPCG = 1, SMG_KRYLOV_FGMRES = 2 };
  *                    residual is FP64-bound, and the fused pass's tile-edge
  *                    recomputation and lower occupancy cost more than the
  *                    fine-residual traffic it saves (measured on GB300).
- *  sweep_warps [0]   warps per 32-column strip of the point smoothers'
- *                    wavefront sweeps on 19/27-point levels: 1 one warp
- *                    does everything; 2 a helper warp loads the operands and
- *                    forms the early partial sums while the main warp only
- *                    finishes points (FP64 Gauss-Seidel with old values,
- *                    y extents above 384, and y extents above 256 except
- *                    for FP64 ILU(0), keep one); 0 the library's choice
- *                    (two where they apply).  Same arithmetic in the same
- *                    order either way. */
+ *  sweep_warps [0]   1: in the point smoothers' wavefront sweeps the warp that
+ *                    finishes a plane's points also forms all their terms;
+ *                    2 and 0: on FP64 19/27-point levels helper warps form
+ *                    the older terms ahead of it.  Same arithmetic in the
+ *                    same order either way. */
 typedef struct {
   int smoother, transfer, precision, krylov, restart;
   double relax_w;
@@ -156,7 +152,7 @@ int smg_vcycle(smg_t h, const double* r, double* z, void* stream);
  * after every stage, so the device time of each stage is measured without
  * host gaps.  Stage t (0 <= t < *count) ran on level levels[t]; stages[t] is
  * one of SMG_STAGE_* (PACK / UNPACK: vectors into and out of the sweeps'
- * skewed plane layout; POST_ADD: the unpack that adds the correction); ms[t]
+ * streams; POST_ADD: the unpack that adds the correction); ms[t]
  * its device time.  At most cap entries are
  * written (*count is the full number).  Synchronises the stream.  Not part
  * of the method: a measurement aid for the per-level cost of a cycle.
@@ -218,7 +214,7 @@ int smg_level_info(smg_t h, int l, int dims[3], int* nstencil, int* offsets);
  * uint16 for BF16), 4 FP32 row scale of A [n], 5 low-precision ILU factors
  * ([n][ns] like 3: lower entries scaled by 6, upper by 7), 6 FP32 row scale of
  * L [n], 7 FP32 row scale of U [n], 8 FP32 inverse diagonal [n].
- * On levels whose ILU(0) sweeps read the skewed records, 5-8 are not kept
+ * On levels whose ILU(0) sweeps read records of their own, 5-8 are not kept
  * after set-up: the first request for one of them allocates and computes
  * all four on `stream` (SMG_ENOMEM if that allocation fails).
  * Returns SMG_EINVAL if the array does not exist on that level or bytes is
@@ -253,13 +249,15 @@ enum {
 };
 int smg_level_apply(smg_t h, int l, int op, const void* x, const void* b, void* y, void* stream);
 
-/* Warps per 32-column strip of the wavefront kernel that runs the point
- * sweep `op` (SMG_OP_GS_FORWARD / GS_BACKWARD / GS_ZERO / ILU_LOWER /
- * ILU_UPPER) of level l, in the V-cycle and in smg_level_apply: 2 the two-
- * warp kernel (option sweep_warps), 1 the one-warp warp-pipelined kernel,
- * 0 another kernel (or the level has no such sweep).  Host-only: reports the
- * choice the launch makes, launches nothing.  Errors: -SMG_EINVAL for a bad
- * handle, level or op. */
+/* The number the option sweep_warps stands for on the point sweep `op`
+ * (SMG_OP_GS_FORWARD / GS_BACKWARD / GS_ZERO / ILU_LOWER / ILU_UPPER) of level
+ * l, by mask, precision and y extent: 2 on 19/27-point levels with ny <= 256
+ * (not FP64 Gauss-Seidel with old values), and for the FP64 ILU(0) solves up
+ * to ny = 384, unless the option is 1; otherwise 1; 0 where the level has no
+ * such sweep or smg_sweep_noalloc's kernel for it is another one.  The rule is
+ * that of the option's first kernels; it does not count the warps of the
+ * kernel that runs today.  Host-only: launches nothing.  Errors: -SMG_EINVAL
+ * for a bad handle, level or op. */
 int smg_level_sweep_warps(smg_t h, int l, int op);
 
 /* Number of CUDA kernels this library has enqueued since it was loaded (a
@@ -391,7 +389,8 @@ int smg_learned_loss_grad(smg_t h, const float* theta, const float* in2, const f
  *            inverse diagonal 1/a_pp), SMG_OP_ILU_LOWER (u = L^{-1} b, M the
  *            ILU(0) factors of smg_level_copy which 1, dinv unused, u may
  *            equal b), SMG_OP_ILU_UPPER (u = U^{-1} b, dinv = 1/u_pp, u may
- *            equal b).  The results equal smg_level_apply's for the same op.
+ *            equal b).  The results equal smg_level_apply's for the same op
+ *            bit for bit.
  *  dims      host int[3]; nx <= 4096 (the scratch holds 16 counters per
  *            x-plane), ny <= 1024, nz <= 4096.
  *  nstencil, offsets  host; offsets in lexicographic order (dx slowest),

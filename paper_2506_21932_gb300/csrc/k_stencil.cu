@@ -4,7 +4,6 @@
 // casts and lowering, diagonal inverses and the dense coarsest level.
 #include <algorithm>
 
-#include "ilurec.cuh"
 #include "smg_internal.cuh"
 
 namespace {
@@ -24,16 +23,14 @@ __device__ __forceinline__ void coords(long long p, const Grid& g, int& i, int& 
 
 // ---------------------------------------------------------------------------
 // SpMV / residual.  One thread per point, all stencil entries unrolled
-// (NS known at compile time), one fused multiply-add per coefficient.  With
-// skew > 0 the result goes to the point's slot in the skewed plane layout of
-// in-plane skew SB = skew (ilurec.cuh) instead of its natural index.
+// (NS known at compile time), one fused multiply-add per coefficient.
 // ---------------------------------------------------------------------------
 template <int PK, int NS>
 __global__ void __launch_bounds__(TPB) k_spmv1(Grid g, Stencil s, const typename Prec<PK>::val* __restrict__ A,
                                                const float* __restrict__ scale,
                                                const typename Prec<PK>::vec* __restrict__ x,
                                                const typename Prec<PK>::vec* __restrict__ b,
-                                               typename Prec<PK>::vec* __restrict__ y, int mode, int skew) {
+                                               typename Prec<PK>::vec* __restrict__ y, int mode) {
   using V = typename Prec<PK>::vec;
   long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= g.n) return;
@@ -50,7 +47,7 @@ __global__ void __launch_bounds__(TPB) k_spmv1(Grid g, Stencil s, const typename
   // the row scale multiplies the finished sum, rounded on its own (never
   // contracted into the subtraction below)
   if (PK == KBF) acc = __fmul_rn(scale[p], (float)acc);
-  y[skew ? skew_slot(g, skew, i, j, k) : p] = mode ? b[p] - acc : acc;
+  y[p] = mode ? b[p] - acc : acc;
 }
 
 // The same for FP32 levels, bandwidth-bound: the CTA's rows of A (one
@@ -64,7 +61,7 @@ __global__ void __launch_bounds__(TPB) k_spmv1s(Grid g, Stencil s, const typenam
                                                 const float* __restrict__ scale,
                                                 const typename Prec<PK>::vec* __restrict__ x,
                                                 const typename Prec<PK>::vec* __restrict__ b,
-                                                typename Prec<PK>::vec* __restrict__ y, int mode, int skew) {
+                                                typename Prec<PK>::vec* __restrict__ y, int mode) {
   using V = typename Prec<PK>::vec;
   using Val = typename Prec<PK>::val;
   __shared__ __align__(16) Val sa[TPB * NS];
@@ -90,7 +87,7 @@ __global__ void __launch_bounds__(TPB) k_spmv1s(Grid g, Stencil s, const typenam
   }
   // the row scale multiplies the finished sum, rounded on its own
   if (PK == KBF) acc = __fmul_rn(scale[p], (float)acc);
-  y[skew ? skew_slot(g, skew, i, j, k) : p] = mode ? b[p] - acc : acc;
+  y[p] = mode ? b[p] - acc : acc;
 }
 
 // Runtime stencil size (any mask).
@@ -99,7 +96,7 @@ __global__ void __launch_bounds__(TPB) k_spmv1_any(Grid g, Stencil s, const type
                                                    const float* __restrict__ scale,
                                                    const typename Prec<PK>::vec* __restrict__ x,
                                                    const typename Prec<PK>::vec* __restrict__ b,
-                                                   typename Prec<PK>::vec* __restrict__ y, int mode, int skew) {
+                                                   typename Prec<PK>::vec* __restrict__ y, int mode) {
   using V = typename Prec<PK>::vec;
   long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= g.n) return;
@@ -115,7 +112,7 @@ __global__ void __launch_bounds__(TPB) k_spmv1_any(Grid g, Stencil s, const type
   // the row scale multiplies the finished sum, rounded on its own (never
   // contracted into the subtraction below)
   if (PK == KBF) acc = __fmul_rn(scale[p], (float)acc);
-  y[skew ? skew_slot(g, skew, i, j, k) : p] = mode ? b[p] - acc : acc;
+  y[p] = mode ? b[p] - acc : acc;
 }
 
 // 3 unknowns per point, BxB blocks (FP64 or FP32 only).
@@ -573,99 +570,6 @@ __global__ void k_lower(Grid g, Stencil s, const double* __restrict__ A, int pk,
   for (int e = 0; e < s.ns; ++e) v[e] = __double2bfloat16(a[e] / (double)(e < s.ec ? sl : su));
 }
 
-// Sweep records (ilurec.cuh) of every point, from the FP64 ILU factors or
-// matrix, written in the skewed layout.  Values and scales equal those of
-// k_lower entry by entry (split = 1 for the ILU triangles, 0 for the matrix).
-template <typename R>
-struct RecBuf {
-  union {
-    uint4 q[R::CHUNKS];
-    unsigned char b[R::BYTES];
-  };
-};
-
-__device__ __forceinline__ void grid_ijk(const Grid& g, long long p, int& i, int& j, int& k) {
-  k = (int)(p % g.nz);
-  j = (int)((p / g.nz) % g.ny);
-  i = (int)(p / ((long long)g.ny * g.nz));
-}
-
-template <int PK, int NS>
-__global__ void k_ilu_records(Grid g, int SB, const double* __restrict__ LU, const double* __restrict__ udinv,
-                              uint4* __restrict__ Lrec, uint4* __restrict__ Urec) {
-  using Val = typename Prec<PK>::val;
-  using Vec = typename Prec<PK>::vec;
-  using RL = SweepRec<PK, NS, 0>;
-  using RU = SweepRec<PK, NS, 1>;
-  constexpr int EC = Shape<NS>::EC;
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= g.n) return;
-  const double* a = LU + p * NS;
-  RecBuf<RL> L;
-  RecBuf<RU> U;
-  for (int c = 0; c < RL::CHUNKS; ++c) L.q[c] = make_uint4(0, 0, 0, 0);
-  for (int c = 0; c < RU::CHUNKS; ++c) U.q[c] = make_uint4(0, 0, 0, 0);
-  Val* lv = (Val*)L.b;
-  Val* uv = (Val*)U.b;
-  if constexpr (PK == KBF) {
-    const float sl = row_scale(a, 0, EC), su = row_scale(a, EC + 1, NS);
-    for (int e = 0; e < EC; ++e) lv[e] = __double2bfloat16(a[e] / (double)sl);
-    for (int e = EC + 1; e < NS; ++e) uv[RU::slot(e)] = __double2bfloat16(a[e] / (double)su);
-    *(float*)(L.b + RL::S_OFF) = sl;
-    *(float*)(U.b + RU::S_OFF) = su;
-  } else {
-    for (int e = 0; e < EC; ++e) lv[e] = (Val)a[e];
-    for (int e = EC + 1; e < NS; ++e) uv[RU::slot(e)] = (Val)a[e];
-  }
-  *(Vec*)(U.b + RU::D_OFF) = (Vec)udinv[p];
-  int i, j, k;
-  grid_ijk(g, p, i, j, k);
-  const long long row = (long long)i * g.nz + skew_row(j, k, SB, g.nz);
-  for (int c = 0; c < RL::CHUNKS; ++c) Lrec[(row * RL::CHUNKS + c) * g.ny + j] = L.q[c];
-  for (int c = 0; c < RU::CHUNKS; ++c) Urec[(row * RU::CHUNKS + c) * g.ny + j] = U.q[c];
-}
-
-template <int PK, int NS>
-__global__ void k_gs_records(Grid g, int SB, const double* __restrict__ A, const double* __restrict__ dinv,
-                             uint4* __restrict__ Grec) {
-  using Val = typename Prec<PK>::val;
-  using Vec = typename Prec<PK>::vec;
-  using RG = SweepRec<PK, NS, 2>;
-  constexpr int EC = Shape<NS>::EC;
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= g.n) return;
-  const double* a = A + p * NS;
-  RecBuf<RG> G;
-  for (int c = 0; c < RG::CHUNKS; ++c) G.q[c] = make_uint4(0, 0, 0, 0);
-  Val* v = (Val*)G.b;
-  if constexpr (PK == KBF) {
-    const float sc = row_scale(a, 0, NS);
-    for (int e = 0; e < NS; ++e)
-      if (e != EC) v[e] = __double2bfloat16(a[e] / (double)sc);
-    *(float*)(G.b + RG::S_OFF) = sc;
-  } else {
-    for (int e = 0; e < NS; ++e)
-      if (e != EC) v[e] = (Val)a[e];
-  }
-  *(Vec*)(G.b + RG::D_OFF) = (Vec)dinv[p];
-  int i, j, k;
-  grid_ijk(g, p, i, j, k);
-  const long long row = (long long)i * g.nz + skew_row(j, k, SB, g.nz);
-  for (int c = 0; c < RG::CHUNKS; ++c) Grec[(row * RG::CHUNKS + c) * g.ny + j] = G.q[c];
-}
-
-// Vector between natural order and the skewed layout.
-template <typename T>
-__global__ void k_skew_copy(Grid g, int SB, int to_skew, const T* __restrict__ src, T* __restrict__ dst, int add) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= g.n) return;
-  int i, j, k;
-  grid_ijk(g, p, i, j, k);
-  const long long q = skew_slot(g, SB, i, j, k);
-  if (to_skew) dst[q] = src[p];
-  else dst[p] = add ? dst[p] + src[q] : src[q];
-}
-
 // Stencil entries reordered: out[p][e] = in[p][perm[e]] (BxB blocks).
 __global__ void k_permute(long long n, int ns, int bb, const int* __restrict__ perm, const double* __restrict__ in,
                           double* __restrict__ out) {
@@ -994,11 +898,9 @@ __global__ void k_dense_matvec(int n, const double* __restrict__ Minv, const dou
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-cudaError_t launch_spmv(const LevelView& L, const void* x, const void* b, void* y, int mode, cudaStream_t st,
-                        int skew) {
+cudaError_t launch_spmv(const LevelView& L, const void* x, const void* b, void* y, int mode, cudaStream_t st) {
   int nb = div_up(L.g.n, TPB);
   if (L.B == 3) {
-    if (skew) return cudaErrorInvalidValue;  // block levels have no skewed layout
     if (L.pk == K64)
       k_spmv3<double><<<nb, TPB, 0, st>>>(L.g, L.s, (const double*)L.A, (const double*)x, (const double*)b,
                                           (double*)y, mode);
@@ -1014,19 +916,19 @@ cudaError_t launch_spmv(const LevelView& L, const void* x, const void* b, void* 
     using Vec = typename Prec<PK>::vec;                                                                        \
     if (L.s.ns == 27 && PK == K32 && aligned16)                                                                \
       k_spmv1s<PK, 27><<<nb, TPB, 0, st>>>(L.g, L.s, (const Val*)L.A, L.scale, (const Vec*)x, (const Vec*)b,   \
-                                           (Vec*)y, mode, skew);                                               \
+                                           (Vec*)y, mode);                                               \
     else if (L.s.ns == 7 && PK == K32 && aligned16)                                                            \
       k_spmv1s<PK, 7><<<nb, TPB, 0, st>>>(L.g, L.s, (const Val*)L.A, L.scale, (const Vec*)x, (const Vec*)b,    \
-                                          (Vec*)y, mode, skew);                                                \
+                                          (Vec*)y, mode);                                                \
     else if (L.s.ns == 27)                                                                                     \
       k_spmv1<PK, 27><<<nb, TPB, 0, st>>>(L.g, L.s, (const Val*)L.A, L.scale, (const Vec*)x, (const Vec*)b,    \
-                                          (Vec*)y, mode, skew);                                                      \
+                                          (Vec*)y, mode);                                                      \
     else if (L.s.ns == 7)                                                                                      \
       k_spmv1<PK, 7><<<nb, TPB, 0, st>>>(L.g, L.s, (const Val*)L.A, L.scale, (const Vec*)x, (const Vec*)b,     \
-                                         (Vec*)y, mode, skew);                                                       \
+                                         (Vec*)y, mode);                                                       \
     else                                                                                                       \
       k_spmv1_any<PK><<<nb, TPB, 0, st>>>(L.g, L.s, (const Val*)L.A, L.scale, (const Vec*)x, (const Vec*)b,    \
-                                          (Vec*)y, mode, skew);                                                      \
+                                          (Vec*)y, mode);                                                      \
   }
   if (L.pk == K64) SPMV_CASE(K64)
   else if (L.pk == K32) SPMV_CASE(K32)
@@ -1153,51 +1055,6 @@ cudaError_t launch_check_padding(Grid g, const Stencil& s, int B, const double* 
 cudaError_t launch_lower_matrix(Grid g, const Stencil& s, const double* A, int pk, int split, void* vals, float* scale,
                                 float* scale2, cudaStream_t st) {
   k_lower<<<div_up(g.n, TPB), TPB, 0, st>>>(g, s, A, pk, split, vals, scale, scale2);
-  smg_count_launch(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_ilu_records(Grid g, int ns, int SB, int pk, const double* LU, const double* udinv, void* Lrec,
-                               void* Urec, cudaStream_t st) {
-  const int nb = div_up(g.n, TPB);
-  uint4 *l = (uint4*)Lrec, *u = (uint4*)Urec;
-#define REC_(PK, NS) k_ilu_records<PK, NS><<<nb, TPB, 0, st>>>(g, SB, LU, udinv, l, u)
-  if (ns != 7 && ns != 19 && ns != 27) return cudaErrorInvalidValue;
-  if (pk == K64) {
-    if (ns == 27) REC_(K64, 27); else if (ns == 19) REC_(K64, 19); else REC_(K64, 7);
-  } else if (pk == K32) {
-    if (ns == 27) REC_(K32, 27); else if (ns == 19) REC_(K32, 19); else REC_(K32, 7);
-  } else {
-    if (ns == 27) REC_(KBF, 27); else if (ns == 19) REC_(KBF, 19); else REC_(KBF, 7);
-  }
-#undef REC_
-  smg_count_launch(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gs_records(Grid g, int ns, int SB, int pk, const double* A, const double* dinv, void* Grec,
-                              cudaStream_t st) {
-  const int nb = div_up(g.n, TPB);
-  uint4* r = (uint4*)Grec;
-#define REC_(PK, NS) k_gs_records<PK, NS><<<nb, TPB, 0, st>>>(g, SB, A, dinv, r)
-  if (ns != 7 && ns != 19 && ns != 27) return cudaErrorInvalidValue;
-  if (pk == K64) {
-    if (ns == 27) REC_(K64, 27); else if (ns == 19) REC_(K64, 19); else REC_(K64, 7);
-  } else if (pk == K32) {
-    if (ns == 27) REC_(K32, 27); else if (ns == 19) REC_(K32, 19); else REC_(K32, 7);
-  } else {
-    if (ns == 27) REC_(KBF, 27); else if (ns == 19) REC_(KBF, 19); else REC_(KBF, 7);
-  }
-#undef REC_
-  smg_count_launch(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_skew_copy(Grid g, int SB, int vb, bool to_skew, const void* src, void* dst, bool add,
-                             cudaStream_t st) {
-  const int nb = div_up(g.n, TPB);
-  if (vb == 8) k_skew_copy<double><<<nb, TPB, 0, st>>>(g, SB, to_skew, (const double*)src, (double*)dst, add);
-  else k_skew_copy<float><<<nb, TPB, 0, st>>>(g, SB, to_skew, (const float*)src, (float*)dst, add);
   smg_count_launch(1);
   return cudaGetLastError();
 }

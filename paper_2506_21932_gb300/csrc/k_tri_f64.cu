@@ -1,0 +1,136 @@
+// Dispatch of the sheared wavefront solves (kernel in trisolve.cuh) and the
+// FP64 instantiations.
+#include <algorithm>
+#include <vector>
+
+#include "trisolve.cuh"
+
+using namespace tri;
+
+namespace {
+
+template <int NS>
+bool canonical(const Stencil& s) {
+  if (s.ns != NS) return false;
+  for (int e = 0; e < NS; ++e)
+    for (int d = 0; d < 3; ++d)
+      if (s.off[e][d] != Shape<NS>::o(e, d)) return false;
+  return true;
+}
+
+template <int NS, bool HD>
+cudaError_t go(int G, bool helpers, const TriParams& P, cudaStream_t st) {
+  // the 7-point mask has no terms older than one step to hand over
+  if constexpr (NS == 7) {
+    return launch_tri_kernel<K64, NS, HD, 4, 0, 16>(P, st);
+  } else {
+    if (G == 4)
+      return helpers ? launch_tri_kernel<K64, NS, HD, 4, 3, 8>(P, st) : launch_tri_kernel<K64, NS, HD, 4, 0, 8>(P, st);
+    return helpers ? launch_tri_kernel<K64, NS, HD, 2, 3, 16>(P, st) : launch_tri_kernel<K64, NS, HD, 2, 0, 16>(P, st);
+  }
+}
+
+}  // namespace
+
+cudaError_t tri_launch_k64(int ns, bool hd, int G, bool helpers, const TriParams& P, cudaStream_t st) {
+  if (ns == 27) return hd ? go<27, true>(G, helpers, P, st) : go<27, false>(G, helpers, P, st);
+  if (ns == 19) return hd ? go<19, true>(G, helpers, P, st) : go<19, false>(G, helpers, P, st);
+  return hd ? go<7, true>(G, helpers, P, st) : go<7, false>(G, helpers, P, st);
+}
+
+// Planes per tile.  More planes mean fewer hops between CTAs (about 2 us each)
+// and more work per SM and step.  Lower / upper solve in ms, FP64 27-point:
+//   G = 2: 0.56 / 0.59 at 128^3, 1.36 / 1.47 at 256^3
+//   G = 4: 0.62 / 0.69           1.31 / 1.44
+// (a step takes 0.34 us with 2 planes, 0.55 us with 4, where the SM's FP64
+// pipe is full; 4 pays once the tiles outnumber the SMs).  FP32 at 256^3 and
+// 384^3: 0.77 and 1.39 with 4 planes, 0.73 and 1.22 with 8; BF16 0.79 with 4,
+// 0.76 with 8 at 256^3 but 0.245 against 0.266 at 104 x 72 x 88.  The 7-point
+// mask has a short step whatever the precision.
+static int planes_per_tile(const Grid& g, int ns, int pk) {
+  if (ns == 7) return 4;
+  if (pk == K64) return (long long)g.nx * g.ny > 192 * 192 ? 4 : 2;
+  return pk == K32 ? 8 : 4;
+}
+
+TriShape tri_shape(const Grid& g, int ns, int pk) {
+  const int SB = ns == 27 ? Shape<27>::SB : ns == 19 ? Shape<19>::SB : Shape<7>::SB;
+  const int SA = ns == 27 ? Shape<27>::SA : ns == 19 ? Shape<19>::SA : Shape<7>::SA;
+  TriShape t;
+  t.ns = ns;
+  t.G = planes_per_tile(g, ns, pk);
+  t.strips = (g.nx + 31) / 32;
+  t.groups = (g.ny + 31 + t.G - 1) / t.G;
+  t.F = SB * (t.G - 1) + 31 * (SA - SB) + g.nz;
+  return t;
+}
+
+bool tri_supported(const LevelView& L) {
+  return L.B == 1 && (canonical<27>(L.s) || canonical<19>(L.s) || canonical<7>(L.s));
+}
+
+size_t tri_mail_bytes(const TriShape& t, int pk) {
+  const size_t word = pk == K64 ? 16 : 8;
+  return word * (size_t)t.strips * t.groups * t.F * (64 + std::max(0, t.G - 2));
+}
+
+size_t tri_rec_bytes(const TriShape& t, int pk, bool hd) {
+  const int ns = t.ns;
+#define RB_(PK, NS) (hd ? TriRec<PK, NS, true>::BYTES : TriRec<PK, NS, false>::BYTES)
+#define RN_(PK) (ns == 27 ? RB_(PK, 27) : ns == 19 ? RB_(PK, 19) : RB_(PK, 7))
+  const size_t b = pk == K64 ? RN_(K64) : pk == K32 ? RN_(K32) : RN_(KBF);
+#undef RN_
+#undef RB_
+  return b * (tri_slots(t) / 32);
+}
+
+int tri_tile_count(const Grid& g, const TriShape& t) {
+  int n = 0;
+  for (int w = 0; w < t.strips; ++w) n += (g.ny + std::min(32, g.nx - 32 * w) - 1 + t.G - 1) / t.G;
+  return n;
+}
+
+// Tiles by the time of their first step, 32 (SP + SL) w + SP G d, the lower
+// strip first: every tile comes after the ones it waits for.
+void tri_tile_table(const Grid& g, const TriShape& t, int* out) {
+  const int SA = t.ns == 27 ? Shape<27>::SA : t.ns == 19 ? Shape<19>::SA : Shape<7>::SA;
+  const int SB = t.ns == 27 ? Shape<27>::SB : t.ns == 19 ? Shape<19>::SB : Shape<7>::SB;
+  struct T {
+    int t0, w, d;
+  };
+  std::vector<T> v;
+  for (int w = 0; w < t.strips; ++w)
+    for (int d = 0; d < (g.ny + std::min(32, g.nx - 32 * w) - 1 + t.G - 1) / t.G; ++d)
+      v.push_back({32 * SA * w + SB * t.G * d, w, d});
+  std::sort(v.begin(), v.end(), [](const T& a, const T& b) { return a.t0 != b.t0 ? a.t0 < b.t0 : a.w < b.w; });
+  for (size_t q = 0; q < v.size(); ++q) out[q] = v[q].w << 16 | v[q].d;
+}
+
+cudaError_t launch_tri(const LevelView& L, const TriShape& t, const TriCall& c, const int* tiles, void* mail,
+                       SweepWs* ws, int* err, unsigned long long budget_ns, cudaStream_t st) {
+  TriParams P;
+  P.g = L.g;
+  P.ntiles = tri_tile_count(L.g, t);
+  P.ngrp = t.groups;
+  P.F = t.F;
+  P.tiles = tiles;
+  P.flip = c.flip;
+  P.budget_ns = budget_ns;
+  P.rec = c.rec;
+  P.b = c.b;
+  P.h = c.h;
+  P.old = c.old;
+  P.u = c.u;
+  P.emit = c.emit;
+  P.relax = c.relax;
+  P.w = c.w;
+  P.mail = mail;
+  P.ws = ws;
+  P.err = err;
+  cudaError_t e;
+  if (L.pk == K64) e = tri_launch_k64(t.ns, c.hd, t.G, c.warps != 1, P, st);
+  else if (L.pk == K32) e = tri_launch_k32(t.ns, c.hd, P, st);
+  else e = tri_launch_kbf(t.ns, c.hd, P, st);
+  if (e == cudaSuccess) smg_count_launch(1);
+  return e;
+}

@@ -10,9 +10,9 @@
 
 #include "chains.h"
 #include "cnn.cuh"
-#include "ilurec.cuh"
 #include "krylov.cuh"
 #include "smg_internal.cuh"
+#include "tri.cuh"
 
 // ---------------------------------------------------------------------------
 // error reporting
@@ -74,13 +74,17 @@ struct Level {
   SweepCfg cfg{};
   int* ilu_upd = nullptr;
   double* lf = nullptr;     // line Gauss-Seidel: per-column factors
-  // warp-pipelined sweeps (canonical masks): records of the working
-  // precision in the skewed layout (ilurec.cuh) and two skewed vectors
-  void* Lrec = nullptr;     // ILU(0) lower solve
-  void* Urec = nullptr;     // ILU(0) upper solve
-  void* Grec = nullptr;     // Gauss-Seidel
-  void* vs0 = nullptr;
-  void* vs1 = nullptr;
+  // sheared wavefront (canonical masks, tri.cuh): records of the lower and
+  // the upper solve in the working precision, the tile order, and vectors in
+  // the solves' streams (sf*: forward, sb*: backward; what a smoother lacks
+  // is null)
+  TriShape ts{};
+  void* Lrec = nullptr;
+  void* Urec = nullptr;
+  int* tiles = nullptr;
+  void* mail = nullptr;
+  void *sf0 = nullptr, *sf1 = nullptr, *sb0 = nullptr, *sb1 = nullptr;
+  void* so = nullptr;  // old iterate of weighted Gauss-Seidel
 };
 
 struct smg_ctx {
@@ -248,21 +252,48 @@ static int sweep(smg_ctx* h, Level& L, int kind, int dir, const void* b, void* u
   return SMG_OK;
 }
 
-// Levels whose sweeps run on the records and vectors of the skewed layout.
-static bool skewed(const Level& L) { return L.Lrec || L.Grec; }
+// Levels whose sweeps run as sheared wavefronts.
+static bool sheared(const Level& L) { return L.Lrec != nullptr; }
 
-// One sweep of a skewed level; b and u are skewed vectors.
-static int sweep_rec(smg_ctx* h, Level& L, int kind, int dir, const void* b, void* u, cudaStream_t st) {
-  const void* M = kind == SW_ILU_L ? L.Lrec : (kind == SW_ILU_U ? L.Urec : L.Grec);
-  SMG_CUDA_TRY(launch_sweep3(view(h, L, true), kind, dir, M, nullptr, nullptr, nullptr, h->opt.relax_w, b, u, L.ws,
-                             h->err, L.cfg, st, true));
+// One triangular solve of a sheared level: dir +1 the lower one from a
+// forward stream, -1 the upper one from a backward stream.  Gauss-Seidel
+// solves carry the diagonal and the weight (relax 1: from zero, 2: blended
+// with old); emit receives b minus the solve's own half of A u, plus addend.
+// The lower solve's results go to backward streams when flip is set.
+static int tri(smg_ctx* h, Level& L, int dir, const void* b, void* u, bool flip, cudaStream_t st, int relax = 0,
+               const void* old = nullptr, void* emit = nullptr, const void* addend = nullptr) {
+  TriCall c;
+  c.rec = dir > 0 ? L.Lrec : L.Urec;
+  c.hd = dir < 0 || h->opt.smoother == SMG_SMOOTHER_SGS;
+  c.dir = dir;
+  c.b = b;
+  c.h = addend;
+  c.old = old;
+  c.u = u;
+  c.emit = emit;
+  c.flip = flip;
+  c.relax = h->opt.relax_w != 1.0 ? relax : 0;
+  c.w = h->opt.relax_w;
+  c.warps = h->opt.sweep_warps;
+  SMG_CUDA_TRY(launch_tri(view(h, L, true), L.ts, c, L.tiles, L.mail, L.ws, h->err, L.cfg.budget_ns, st));
   return SMG_OK;
 }
 
-// Vector between natural order and the level's skewed layout.
-static int skew(smg_ctx* h, Level& L, const void* src, void* dst, bool to_skew, bool add, cudaStream_t st) {
-  SMG_CUDA_TRY(launch_skew_copy(L.g, L.cfg.SB, (int)vsize(h), to_skew, src, dst, add, st));
+// Natural order -> stream of direction dir, and back (optionally added).
+static int shear(smg_ctx* h, Level& L, int dir, const void* src, void* dst, cudaStream_t st) {
+  SMG_CUDA_TRY(launch_shear_copy(L.g, L.ts, dir, (int)vsize(h), true, src, dst, false, st));
   return SMG_OK;
+}
+static int unshear(smg_ctx* h, Level& L, int dir, const void* src, void* dst, bool add, cudaStream_t st) {
+  SMG_CUDA_TRY(launch_shear_copy(L.g, L.ts, dir, (int)vsize(h), false, src, dst, add, st));
+  return SMG_OK;
+}
+
+// The old iterate of a weighted Gauss-Seidel sweep in the stream of its
+// direction (null for weight 1, which does not read it).
+static int shear_old(smg_ctx* h, Level& L, int dir, const void* u, const void** old, cudaStream_t st) {
+  *old = L.so;
+  return L.so ? shear(h, L, dir, u, L.so, st) : SMG_OK;
 }
 
 // One line Gauss-Seidel sweep (FP64 hierarchy only).
@@ -273,16 +304,22 @@ static int lsweep(smg_ctx* h, Level& L, int kind, int dir, const void* b, void* 
 }
 
 static int smooth_pre(smg_ctx* h, Level& L, int l, const void* f, void* u, cudaStream_t st) {
-  if (skewed(L)) {
-    // f -> vs0; the first sweep writes vs1 from zero, the second updates it
-    TRY(skew(h, L, f, L.vs0, true, false, st));
+  if (sheared(L)) {
+    TRY(shear(h, L, +1, f, L.sf0, st));
     prof_mark(h, l, PM_PACK, st);
-    const bool ilu = h->opt.smoother == SMG_SMOOTHER_ILU0;
-    TRY(sweep_rec(h, L, ilu ? SW_ILU_L : SW_GS_ZERO, +1, L.vs0, L.vs1, st));
-    prof_mark(h, l, PM_PRE1, st);
-    TRY(sweep_rec(h, L, ilu ? SW_ILU_U : SW_GS_FULL, -1, ilu ? L.vs1 : L.vs0, L.vs1, st));
+    if (h->opt.smoother == SMG_SMOOTHER_ILU0) {
+      TRY(tri(h, L, +1, L.sf0, L.sb0, true, st));
+      prof_mark(h, l, PM_PRE1, st);
+      TRY(tri(h, L, -1, L.sb0, L.sb0, false, st));
+    } else {
+      // the forward sweep from zero leaves f - L u, which is the right-hand
+      // side of the backward one, in sb1
+      TRY(tri(h, L, +1, L.sf0, L.sb0, true, st, 1, nullptr, L.sb1));
+      prof_mark(h, l, PM_PRE1, st);
+      TRY(tri(h, L, -1, L.sb1, L.sb0, false, st, 2, L.sb0));
+    }
     prof_mark(h, l, PM_PRE2, st);
-    TRY(skew(h, L, L.vs1, u, false, false, st));
+    TRY(unshear(h, L, -1, L.sb0, u, false, st));
     prof_mark(h, l, PM_UNPACK, st);
     return SMG_OK;
   }
@@ -304,30 +341,30 @@ static int smooth_pre(smg_ctx* h, Level& L, int l, const void* f, void* u, cudaS
 }
 
 static int smooth_post(smg_ctx* h, Level& L, int l, const void* f, void* u, cudaStream_t st) {
-  if (skewed(L)) {
-    if (h->opt.smoother == SMG_SMOOTHER_ILU0) {
-      // u += U^-1 L^-1 (f - A u): the residual computed in natural order
-      // and written in the skewed layout, the solves on skewed vectors, the
-      // correction added while unpacking
-      SMG_CUDA_TRY(launch_spmv(view(h, L, true), u, f, L.vs0, 1, st, L.cfg.SB));
+  if (sheared(L)) {
+    const bool ilu = h->opt.smoother == SMG_SMOOTHER_ILU0;
+    if (ilu) {
+      // u += U^-1 L^-1 (f - A u), the correction added while unshearing
+      SMG_CUDA_TRY(launch_shear_residual(view(h, L, true), L.ts, u, f, L.sf0, st));
       prof_mark(h, l, PM_POST_RESID, st);
-      TRY(sweep_rec(h, L, SW_ILU_L, +1, L.vs0, L.vs1, st));
+      TRY(tri(h, L, +1, L.sf0, L.sb0, true, st));
       prof_mark(h, l, PM_POST1, st);
-      TRY(sweep_rec(h, L, SW_ILU_U, -1, L.vs1, L.vs1, st));
-      prof_mark(h, l, PM_POST2, st);
-      TRY(skew(h, L, L.vs1, u, false, true, st));
-      prof_mark(h, l, PM_POST_ADD, st);
+      TRY(tri(h, L, -1, L.sb0, L.sb0, false, st));
     } else {
-      TRY(skew(h, L, f, L.vs0, true, false, st));
-      TRY(skew(h, L, u, L.vs1, true, false, st));
-      prof_mark(h, l, PM_PACK, st);
-      TRY(sweep_rec(h, L, SW_GS_FULL, +1, L.vs0, L.vs1, st));
+      // sf1 = (upper part) u, sf0 = f - sf1; the forward sweep then leaves
+      // f - L u_new = (sf0 - L u_new) + sf1 for the backward one
+      SMG_CUDA_TRY(launch_half(view(h, L, true), +1, u, nullptr, L.t, st));
+      SMG_CUDA_TRY(launch_shear_split(L.g, L.ts, (int)vsize(h), f, L.t, L.sf0, L.sf1, st));
+      const void* old = nullptr;
+      TRY(shear_old(h, L, +1, u, &old, st));
+      prof_mark(h, l, PM_POST_RESID, st);
+      TRY(tri(h, L, +1, L.sf0, L.sb0, true, st, 2, old, L.sb1, L.sf1));
       prof_mark(h, l, PM_POST1, st);
-      TRY(sweep_rec(h, L, SW_GS_FULL, -1, L.vs0, L.vs1, st));
-      prof_mark(h, l, PM_POST2, st);
-      TRY(skew(h, L, L.vs1, u, false, false, st));
-      prof_mark(h, l, PM_UNPACK, st);
+      TRY(tri(h, L, -1, L.sb1, L.sb0, false, st, 2, L.sb0));
     }
+    prof_mark(h, l, PM_POST2, st);
+    TRY(unshear(h, L, -1, L.sb0, u, ilu, st));
+    prof_mark(h, l, ilu ? PM_POST_ADD : PM_UNPACK, st);
     return SMG_OK;
   }
   if (h->opt.smoother == SMG_SMOOTHER_LGS) {
@@ -619,27 +656,34 @@ static int setup_level_smoother(smg_ctx* h, Level& L, cudaStream_t st) {
       SMG_CUDA_TRY(launch_d2f_array(L.dinv, (float*)L.dinv32, n * B * B, st));
     }
   }
-  // point smoothers on the warp-pipelined kernel read records of the skewed
-  // layout (ilurec.cuh), on skewed vectors
+  // point smoothers on canonical masks run as sheared wavefronts on records
+  // of their own
   const bool ilu = h->opt.smoother == SMG_SMOOTHER_ILU0, sgs = h->opt.smoother == SMG_SMOOTHER_SGS;
-  const LevelView lv = view(h, L, true);
-  if (B == 1 && ((ilu && sweep3_supported(lv, SW_ILU_L)) ||
-                 (sgs && sweep3_supported(lv, SW_GS_ZERO) && sweep3_supported(lv, SW_GS_FULL)))) {
-    const size_t unit = 16 * (size_t)n;
-    if (ilu) {
-      TRY(dev_alloc(h, &L.Lrec, unit * sweep_rec_chunks(h->pk, L.s.ns, 0)));
-      TRY(dev_alloc(h, &L.Urec, unit * sweep_rec_chunks(h->pk, L.s.ns, 1)));
-      SMG_CUDA_TRY(launch_ilu_records(L.g, L.s.ns, L.cfg.SB, h->pk, L.LU, L.udinv, L.Lrec, L.Urec, st));
-    } else {
-      TRY(dev_alloc(h, &L.Grec, unit * sweep_rec_chunks(h->pk, L.s.ns, 2)));
-      SMG_CUDA_TRY(launch_gs_records(L.g, L.s.ns, L.cfg.SB, h->pk, L.A, L.dinv, L.Grec, st));
+  if ((ilu || sgs) && tri_supported(view(h, L, true))) {
+    L.ts = tri_shape(L.g, L.s.ns, h->pk);
+    const size_t sv = tri_slots(L.ts) * vsize(h);
+    TRY(dev_alloc(h, &L.Lrec, tri_rec_bytes(L.ts, h->pk, sgs)));
+    TRY(dev_alloc(h, &L.Urec, tri_rec_bytes(L.ts, h->pk, true)));
+    if (ilu) SMG_CUDA_TRY(launch_tri_records_ilu(L.g, L.ts, h->pk, L.LU, L.udinv, L.Lrec, L.Urec, st));
+    else SMG_CUDA_TRY(launch_tri_records_gs(L.g, L.ts, h->pk, L.A, L.dinv, L.Lrec, L.Urec, st));
+    TRY(dev_alloc(h, &L.mail, tri_mail_bytes(L.ts, h->pk)));
+    SMG_CUDA_TRY(cudaMemsetAsync(L.mail, 0, tri_mail_bytes(L.ts, h->pk), st));
+    TRY(dev_alloc(h, &L.sf0, sv));
+    TRY(dev_alloc(h, &L.sb0, sv));
+    if (sgs) {
+      TRY(dev_alloc(h, &L.sf1, sv));
+      TRY(dev_alloc(h, &L.sb1, sv));
+      if (h->opt.relax_w != 1.0) TRY(dev_alloc(h, &L.so, sv));
     }
-    TRY(dev_alloc(h, &L.vs0, (size_t)n * vsize(h)));
-    TRY(dev_alloc(h, &L.vs1, (size_t)n * vsize(h)));
+    std::vector<int> tiles(tri_tile_count(L.g, L.ts));
+    tri_tile_table(L.g, L.ts, tiles.data());
+    TRY(dalloc(h, &L.tiles, tiles.size()));
+    SMG_CUDA_TRY(cudaMemcpyAsync(L.tiles, tiles.data(), tiles.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+    SMG_CUDA_TRY(cudaStreamSynchronize(st));  // tiles is a host temporary
   }
   // the natural-order sweeps read the factors in the V-cycle precision; the
-  // skewed levels' records were built from the FP64 factors directly
-  if (!skewed(L)) TRY(lower_factors(h, L, st));
+  // sheared levels' records were built from the FP64 factors directly
+  if (!sheared(L)) TRY(lower_factors(h, L, st));
   return SMG_OK;
 }
 
@@ -1102,9 +1146,9 @@ extern "C" int smg_level_sweep_warps(smg_t h, int l, int op) {
   Level& L = h->L[l];
   const bool ilu_op = kind == SW_ILU_L || kind == SW_ILU_U;
   if (ilu_op != (h->opt.smoother == SMG_SMOOTHER_ILU0) || h->opt.smoother == SMG_SMOOTHER_LGS) return 0;
-  // the warp-pipelined kernels run a level's point sweeps exactly when its
-  // records are in the skewed layout
-  return skewed(L) ? sweep3_warps(view(h, L, true), kind, true, L.cfg) : 0;
+  const LevelView v = view(h, L, true);
+  if (!sheared(L) || (!ilu_op && !sweep3_supported(v, SW_GS_FULL))) return 0;
+  return sweep3_warps(v, kind, L.cfg);
 }
 
 extern "C" int smg_level_info(smg_t h, int l, int dims[3], int* nstencil, int* offsets) {
@@ -1130,7 +1174,7 @@ extern "C" int smg_level_copy(smg_t h, int l, int which, void* dst, size_t bytes
   const void* src = nullptr;
   size_t sz = 0;
   cudaStream_t st = (cudaStream_t)stream;
-  // skewed levels keep no lowered factors; they are made on first request
+  // sheared levels keep no lowered factors; they are made on first request
   if (which >= 5 && which <= 8) TRY(lower_factors(h, L, st));
   switch (which) {
     case 0: src = L.A; sz = n * L.s.ns * L.B * L.B * 8; break;
@@ -1153,6 +1197,13 @@ extern "C" int smg_level_copy(smg_t h, int l, int which, void* dst, size_t bytes
   return SMG_OK;
 }
 
+// Whether a level operation runs the sheared wavefront: on FP64 levels only
+// where smg_sweep_noalloc's natural-order kernel (sweep3.cuh) takes the same
+// sweep and forms the same sums, so the two entry points agree to the bit.
+static bool level_op_sheared(smg_ctx* h, const Level& L, int kind) {
+  return sheared(L) && (h->pk != K64 || sweep3_supported(view(h, L, true), kind));
+}
+
 extern "C" int smg_level_apply(smg_t h, int l, int op, const void* x, const void* b, void* y, void* stream) {
   if (!h || l < 0 || l >= h->nlev) return SMG_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
@@ -1170,12 +1221,21 @@ extern "C" int smg_level_apply(smg_t h, int l, int op, const void* x, const void
     case SMG_OP_GS_BACKWARD:
     case SMG_OP_GS_ZERO:
       if (!has_sm || h->opt.smoother != SMG_SMOOTHER_SGS || !x || !b) return SMG_EINVAL;
-      if (skewed(L)) {
-        TRY(skew(h, L, b, L.vs0, true, false, st));
-        if (op != SMG_OP_GS_ZERO) TRY(skew(h, L, x, L.vs1, true, false, st));
-        TRY(sweep_rec(h, L, op == SMG_OP_GS_ZERO ? SW_GS_ZERO : SW_GS_FULL, op == SMG_OP_GS_BACKWARD ? -1 : +1,
-                      L.vs0, L.vs1, st));
-        TRY(skew(h, L, L.vs1, (void*)x, false, false, st));
+      if (level_op_sheared(h, L, op == SMG_OP_GS_ZERO ? SW_GS_ZERO : SW_GS_FULL)) {
+        const int dir = op == SMG_OP_GS_BACKWARD ? -1 : +1;
+        void* in = dir > 0 ? L.sf0 : L.sb1;
+        void* out = dir > 0 ? L.sf1 : L.sb0;
+        const void* old = nullptr;
+        if (op == SMG_OP_GS_ZERO) {
+          TRY(shear(h, L, dir, b, in, st));
+        } else {
+          // b minus the half of A x that the sweep leaves old
+          SMG_CUDA_TRY(launch_half(view(h, L, true), dir, x, b, L.t, st));
+          TRY(shear(h, L, dir, L.t, in, st));
+          TRY(shear_old(h, L, dir, x, &old, st));
+        }
+        TRY(tri(h, L, dir, in, out, false, st, op == SMG_OP_GS_ZERO ? 1 : 2, old));
+        TRY(unshear(h, L, dir, out, (void*)x, false, st));
         break;
       }
       TRY(sweep(h, L, op == SMG_OP_GS_ZERO ? SW_GS_ZERO : SW_GS_FULL, op == SMG_OP_GS_BACKWARD ? -1 : +1, b,
@@ -1190,11 +1250,11 @@ extern "C" int smg_level_apply(smg_t h, int l, int op, const void* x, const void
       break;
     case SMG_OP_ILU_APPLY:
       if (!has_sm || h->opt.smoother != SMG_SMOOTHER_ILU0 || !b || !y) return SMG_EINVAL;
-      if (skewed(L)) {
-        TRY(skew(h, L, b, L.vs0, true, false, st));
-        TRY(sweep_rec(h, L, SW_ILU_L, +1, L.vs0, L.vs1, st));
-        TRY(sweep_rec(h, L, SW_ILU_U, -1, L.vs1, L.vs1, st));
-        TRY(skew(h, L, L.vs1, y, false, false, st));
+      if (level_op_sheared(h, L, SW_ILU_L)) {
+        TRY(shear(h, L, +1, b, L.sf0, st));
+        TRY(tri(h, L, +1, L.sf0, L.sb0, true, st));
+        TRY(tri(h, L, -1, L.sb0, L.sb0, false, st));
+        TRY(unshear(h, L, -1, L.sb0, y, false, st));
         break;
       }
       TRY(sweep(h, L, SW_ILU_L, +1, b, y, st));
@@ -1215,11 +1275,12 @@ extern "C" int smg_level_apply(smg_t h, int l, int op, const void* x, const void
     case SMG_OP_ILU_LOWER:
     case SMG_OP_ILU_UPPER:
       if (!has_sm || h->opt.smoother != SMG_SMOOTHER_ILU0 || !b || !y) return SMG_EINVAL;
-      if (skewed(L)) {
-        TRY(skew(h, L, b, L.vs0, true, false, st));
-        TRY(sweep_rec(h, L, op == SMG_OP_ILU_LOWER ? SW_ILU_L : SW_ILU_U, op == SMG_OP_ILU_LOWER ? +1 : -1, L.vs0,
-                      L.vs1, st));
-        TRY(skew(h, L, L.vs1, y, false, false, st));
+      if (level_op_sheared(h, L, SW_ILU_L)) {
+        const int dir = op == SMG_OP_ILU_LOWER ? +1 : -1;
+        void* v = dir > 0 ? L.sf0 : L.sb0;
+        TRY(shear(h, L, dir, b, v, st));
+        TRY(tri(h, L, dir, v, v, false, st));
+        TRY(unshear(h, L, dir, v, y, false, st));
         break;
       }
       TRY(sweep(h, L, op == SMG_OP_ILU_LOWER ? SW_ILU_L : SW_ILU_U, op == SMG_OP_ILU_LOWER ? +1 : -1, b, y, st));

@@ -48,13 +48,14 @@ struct Stencil {
 // Per-sweep device workspace for the wavefront kernels: progress of every
 // plane, a ticket that hands out planes in order, a count of finished CTAs.
 // Progress slots: one per x-plane (plane-per-CTA kernels) or one per x-plane
-// group and 32-column warp (warp-pipelined kernel): 4096 planes x 16 warps.
+// and 32-column warp (warp-pipelined kernels): 4096 planes x 16 warps.
 constexpr int kProgSlots = 4096 * 16;
 struct SweepWs {
   int ticket;
   int finished;
-  int pad[2];
-  int prog[kProgSlots];  // global time step up to which a plane (or a plane's warp) is done
+  int epoch;  // launches of the sheared wavefront on this workspace: its mailboxes' tag
+  int pad;
+  int prog[kProgSlots];  // global time step up to which a plane or a plane's warp is done
 };
 
 // Kernel-visible error word values (mirror smg_status).
@@ -147,16 +148,13 @@ struct LevelView {
   const float* scale;   // KBF row scales of A (else null)
 };
 
-// y = A x (mode 0) or y = b - A x (mode 1).
 // fc = R (b - A x) in one pass for scalar levels and the full-weighting or
 // 3d8c restriction; cudaErrorNotSupported otherwise (the caller then runs
 // launch_spmv and launch_restrict)
 cudaError_t launch_resid_restrict(const LevelView& L, int transfer, const void* x, const void* b, void* fc,
                                   cudaStream_t st);
-// y = A x (mode 0) or b - A x (mode 1); skew > 0 writes y in the skewed
-// plane layout of in-plane skew skew (scalar levels only)
-cudaError_t launch_spmv(const LevelView& L, const void* x, const void* b, void* y, int mode, cudaStream_t st,
-                        int skew = 0);
+// y = A x (mode 0) or y = b - A x (mode 1).
+cudaError_t launch_spmv(const LevelView& L, const void* x, const void* b, void* y, int mode, cudaStream_t st);
 
 // Restriction / prolongation between level (g, B) and its coarse level.
 cudaError_t launch_restrict(int transfer, Grid fine, int B, int pk, const void* rf, void* fc, cudaStream_t st);
@@ -172,7 +170,7 @@ struct SweepCfg {
   int SA, SB;  // schedule skews: global time t = SA*i + SB*j + k
   int G;       // publish progress every G steps
   unsigned long long budget_ns;
-  int warps = 0;  // warps per 32-column strip of the skewed-layout sweeps: 0 the library's choice, 1, 2
+  int warps = 0;  // option sweep_warps
 };
 cudaError_t launch_sweep(const LevelView& L, int kind, int dir, const void* M, const float* sc1, const float* sc2,
                          const void* dinv, double w, const void* b, void* u, SweepWs* ws, int* err,
@@ -185,19 +183,12 @@ cudaError_t launch_sweep2(const LevelView& L, int kind, int dir, const void* M, 
                           const void* dinv, double w, const void* b, void* u, SweepWs* ws, int* err,
                           const SweepCfg& cfg, cudaStream_t st);
 
-// Warp-pipelined variant (same masks, ny <= 512): per-warp time loops synced
-// through shared-memory counters, a communication warp for the GPU-scope
-// hand-off; returns cudaErrorNotSupported when it does not apply.  rec: M is
-// the sweep's records and b, u are vectors, all in the skewed layout of
-// ilurec.cuh (FP32 / BF16 sweeps exist only in that form); otherwise M is
-// the matrix or ILU factors [n][ns] and the vectors are in natural order.
+// Warp-pipelined variant on natural-order FP64 data (same masks, at most 12
+// warps of columns); cudaErrorNotSupported (nothing launched) otherwise.
 bool sweep3_supported(const LevelView& L, int kind);
-// Warps per 32-column strip launch_sweep3 uses for this sweep: 2 (the
-// two-warp kernel), 1 (the one-warp kernel), 0 (not supported).
-int sweep3_warps(const LevelView& L, int kind, bool rec, const SweepCfg& cfg);
-cudaError_t launch_sweep3(const LevelView& L, int kind, int dir, const void* M, const float* sc1, const float* sc2,
-                          const void* dinv, double w, const void* b, void* u, SweepWs* ws, int* err,
-                          const SweepCfg& cfg, cudaStream_t st, bool rec);
+int sweep3_warps(const LevelView& L, int kind, const SweepCfg& cfg);
+cudaError_t launch_sweep3(const LevelView& L, int kind, int dir, const void* M, const void* dinv, double w,
+                          const void* b, void* u, SweepWs* ws, int* err, const SweepCfg& cfg, cudaStream_t st);
 
 // Bounded wait on a flag nobody sets (failure-path self-test).
 cudaError_t launch_wait_selftest(const int* flag, int* err, unsigned long long budget_ns, cudaStream_t st);
