@@ -1,62 +1,110 @@
 // Line Gauss-Seidel along z (Sec. 4.4, LGS): the points of a z-column (i, j)
-// are updated together.  The column's right-hand side is b minus every
-// coupling to another column (columns earlier in the sweep already new,
-// later ones old, none of the later ones from a zero guess), and the
+// are updated together.  The column's right-hand side is its share of b minus
+// the couplings to the columns earlier in the sweep (already new), and the
 // tridiagonal system of the offsets (0,0,-1), (0,0,0), (0,0,+1) is solved
-// exactly.  Columns run in lexicographic (i, j) order (reversed for the
-// backward sweep), scheduled like the point sweeps: one x-plane per CTA at a
-// time (atomic ticket), column j of plane i after column j + 1 (or j for a
-// 7-point mask) of plane i - 1, progress published by the wavefront engine's
-// publisher / poller warps.
+// exactly.  The couplings to later columns, old in a full sweep, are taken off
+// b beforehand by a parallel kernel (k_line_half), so one sweep kernel serves
+// both kinds.  Columns run in lexicographic (i, j) order (reversed for the
+// backward sweep): one x-plane per CTA at a time (atomic ticket), column j of
+// plane i after column j + 1 (or j) of plane i - 1.
 //
-// A column is solved by four warps, one per SM sub-partition (each of which
-// issues about one FP64 warp instruction per 64 cycles on GB300).  The serial
-// Thomas recurrence of the paper would put 2 nz dependent FP64 operations on
-// the critical path, so the column is cut into 128 chunks of m rows, one per
-// thread (partition method): every thread eliminates its rows 2..m in terms
-// of its own first unknown P_c and the next chunk's first unknown P_{c+1},
-// the 128 chunk-first unknowns form a tridiagonal system solved by parallel
-// cyclic reduction through shared memory, and each thread then recovers its
-// rows.  Everything that depends only on the matrix (reciprocal pivots,
-// elimination multipliers, the reduced system's PCR multipliers) is computed
-// once at set-up, so a sweep does no division.  In exact arithmetic the
-// result is the Thomas solution; the rounding differs.  All eight compute
-// warps assemble the right-hand side and store the column; the next
-// column's matrix rows, right-hand side and factors are copied to shared
-// memory by bulk copies (one thread, mbarrier completion) while the current
-// column is worked on.
-#include <cstdint>
-#include <utility>
+// What bounds a column is a chain of dependent FP64 instructions (about 67
+// cycles each): the last three coupling terms, the tridiagonal solve, the
+// hand-over; at nz = 64 it takes 2800 cycles (waits 360, late terms and
+// elimination 790, reduction 1150, recovery 300, stores 250), at nz = 128
+// with two solving warps 3450, where one kernel with every term and every
+// row's work on it took 10000.  A sweep at 128 x 112 x 128 on 27 points takes
+// 0.90 ms (before: 2.03 from zero, 2.48 full).  So the work is split by what
+// is on that chain:
+//  * helper warps form the right-hand side up to the terms of the previous
+//    column of the same plane, a column ahead;
+//  * the solving warps (1, 2 or 4, one per SM sub-partition) add those terms
+//    and solve.  A column is cut into 32 chunks per solving warp, of m rows,
+//    one chunk per thread (partition method): every thread eliminates its rows
+//    2..m in terms of its own first unknown P_c and the next chunk's P_{c+1},
+//    the chunk-first unknowns form a tridiagonal system solved by parallel
+//    cyclic reduction, and each thread then recovers its rows.  Chunk c belongs
+//    to warp c mod warps, so all but the first reduction steps stay inside a
+//    warp (shuffles); values that cross warps go through shared memory, one
+//    barrier each.  Everything that depends only on the matrix is computed at
+//    set-up, so a sweep does no division.  In exact arithmetic the result is
+//    the Thomas solution; the rounding differs;
+//  * a loader warp polls the previous plane's mailbox (mailbox.cuh) and keeps
+//    its last columns in shared memory; a record warp fetches the columns'
+//    coefficients and factors by bulk copies.
+// Every wait is bounded; on expiry the error word is set, the CTA waits for
+// its copies in flight and leaves.
+#include <algorithm>
+#include <climits>
 
-#include "shapes.cuh"
+#include "mailbox.cuh"
 #include "smg_internal.cuh"
-#include "wavefront.cuh"
 
 namespace {
 
-constexpr int kLgsWarps = 8;                       // compute warps of a CTA
-constexpr int kLgsThreads = (kLgsWarps + 2) * 32;  // + publisher + poller
-constexpr int kLgsSolveWarps = 4;                  // warps solving a column (warps 0..3)
-constexpr int kLgsChunks = 32 * kLgsSolveWarps;    // chunks of a column, one per solving thread
-constexpr int kLgsPcr = 7;                         // PCR steps: log2(kLgsChunks)
-constexpr int kLgsMaxM = 8;                        // rows per chunk: nz <= 1024
+using tri::ld_acq_cta;
+using tri::st_rel_cta;
 
-// Column block of the line factors, in doubles, every field kLgsChunks wide:
-// for chunk rows r = 1..m-1 the fields F_W (a_r / den_r), F_INV (1 / den_r),
-// F_CP (c_r / den_r), F_G, F_H (x_r = e_r - g_r P_{c+1} - h_r P_c); then per
-// chunk C_A0, C_C0 (the couplings of its first row), C_AL + t, C_GA + t (the
-// PCR multipliers of step t, stride 2^t) and C_INVB (1 / final pivot).
+constexpr int kHelpers = 8;      // helper warps
+constexpr int kMaxM = 8;         // rows per chunk: nz <= 1024
+constexpr int kMaxStages = 4;    // columns of records in flight
+
+// Solving warps and rows per chunk of a column of nz points.
+__host__ __device__ inline int line_warps(int nz) { return nz <= 64 ? 1 : nz <= 128 ? 2 : 4; }
+__host__ __device__ inline int line_rows(int nz) { return nz <= 256 ? 2 : nz <= 512 ? 4 : 8; }
+
+// Column block of the line factors, in doubles, every field C = 32 * warps
+// wide, chunk c at (c % warps) * 32 + c / warps: for chunk rows r = 1..m-1 the
+// fields F_W (-a_r / den_r), F_INV (1 / den_r), F_CP (-c_r / den_r), F_G, F_H
+// (x_r = e_r + g_r P_{c+1} + h_r P_c); then per chunk C_A0, C_C0 (minus the
+// couplings of its first row), C_INVB (1 / final pivot), C_AL + t, C_GA + t
+// (the multipliers of reduction step t, stride 2^t).
 enum { F_W, F_INV, F_CP, F_G, F_H, F_N };
-enum { C_A0 = 0, C_C0 = 1, C_AL = 2, C_GA = 2 + kLgsPcr, C_INVB = 2 + 2 * kLgsPcr, C_N = 3 + 2 * kLgsPcr };
-__host__ __device__ inline int lgs_row(int r, int f) { return ((r - 1) * F_N + f) * kLgsChunks; }
-__host__ __device__ inline int lgs_chunk(int m, int f) { return ((m - 1) * F_N + f) * kLgsChunks; }
-
-__device__ __forceinline__ void lgs_bar() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kLgsWarps * 32) : "memory");
+enum { C_A0, C_C0, C_INVB, C_STEP };
+__host__ __device__ constexpr int row_field(int r, int f) { return (r - 1) * F_N + f; }
+__host__ __device__ constexpr int chunk_field(int m, int f) { return (m - 1) * F_N + f; }
+__host__ __device__ constexpr int step_field(int m, int t, int which) {
+  return (m - 1) * F_N + C_STEP + 2 * t + which;
 }
-// barrier of the solving warps only
-__device__ __forceinline__ void lgs_bar_solve() {
-  asm volatile("bar.sync 2, %0;" ::"n"(kLgsChunks) : "memory");
+__host__ __device__ constexpr int log2_chunks(int warps) { return warps == 1 ? 5 : warps == 2 ? 6 : 7; }
+__host__ __device__ constexpr int block_fields(int m, int warps) {
+  return (m - 1) * F_N + C_STEP + 2 * log2_chunks(warps);
+}
+
+// Stencil entries of one direction of the sweep, in sweep coordinates: early
+// ones (previous plane: column offset ec in {-1, 0, 1}) and late ones (the
+// previous column of the same plane), each with its z offset; and the later
+// columns' entries (natural offsets) of the half product.
+struct LineTerms {
+  int ne, nh, dep;  // dep: largest ec (-2 without early entries)
+  int ee[9], ec[9], ez[9];
+  int le[3];  // by z offset + 1; -1 where the mask lacks it
+  int he[12], hx[12], hy[12], hz[12];
+};
+
+LineTerms line_terms(const Stencil& s, int dir) {
+  LineTerms t{};
+  t.dep = -2;
+  t.le[0] = t.le[1] = t.le[2] = -1;
+  for (int q = 0; q < s.ns; ++q) {
+    const int e = dir > 0 ? q : s.ns - 1 - q;
+    const int dx = dir * s.off[e][0], dy = dir * s.off[e][1], dz = s.off[e][2];
+    if (dx == 0 && dy == 0) continue;
+    if (dx < 0) {
+      t.ee[t.ne] = e;
+      t.ec[t.ne] = dy;
+      t.ez[t.ne++] = dz;
+      t.dep = std::max(t.dep, dy);
+    } else if (dx == 0 && dy < 0) {
+      t.le[dz + 1] = e;
+    } else {
+      t.he[t.nh] = e;
+      t.hx[t.nh] = s.off[e][0];
+      t.hy[t.nh] = s.off[e][1];
+      t.hz[t.nh++] = dz;
+    }
+  }
+  return t;
 }
 
 struct LineIdx {
@@ -95,16 +143,17 @@ __global__ void k_lgs_pivots(Grid g, int ns, LineIdx e, const double* __restrict
   }
 }
 
-// One block of kLgsChunks threads per column, thread c = chunk c: the
-// partitioned elimination of rows c*m + 1 .. c*m + m-1 and the reduced
-// system's PCR multipliers (neighbour values through shared memory).
-__global__ void __launch_bounds__(kLgsChunks) k_lgs_factor(Grid g, int ns, LineIdx e, const double* __restrict__ A,
-                                                           double* __restrict__ Fo, int m, long long blk, int* err) {
-  __shared__ double xa[kLgsChunks], xb[kLgsChunks], xc[kLgsChunks];
+// One block per column, thread c = chunk c: the partitioned elimination of
+// rows c*m + 1 .. c*m + m-1 and the reduced system's multipliers (neighbour
+// values through shared memory).
+__global__ void __launch_bounds__(128) k_lgs_factor(Grid g, int ns, LineIdx e, const double* __restrict__ A,
+                                                    double* __restrict__ Fo, int m, int warps, int* err) {
+  __shared__ double xa[128], xb[128], xc[128];
+  const int C = 32 * warps, steps = log2_chunks(warps);
   const long long col = blockIdx.x;
   const int c = threadIdx.x;
-  double* F = Fo + col * blk;
-  double cp[kLgsMaxM], fp[kLgsMaxM];
+  double* F = Fo + col * (long long)block_fields(m, warps) * C + (c % warps) * 32 + c / warps;
+  double cp[kMaxM], fp[kMaxM];
   bool bad = false;
   for (int r = 1; r < m; ++r) {
     double a, b, cc;
@@ -114,19 +163,19 @@ __global__ void __launch_bounds__(kLgsChunks) k_lgs_factor(Grid g, int ns, LineI
     const double inv = 1.0 / den;
     cp[r] = cc * inv;
     fp[r] = (r == 1 ? a : -a * fp[r - 1]) * inv;
-    F[lgs_row(r, F_W) + c] = a * inv;
-    F[lgs_row(r, F_INV) + c] = inv;
-    F[lgs_row(r, F_CP) + c] = cp[r];
+    F[row_field(r, F_W) * C] = -a * inv;
+    F[row_field(r, F_INV) * C] = inv;
+    F[row_field(r, F_CP) * C] = -cp[r];
   }
   double gg = cp[m - 1], hh = fp[m - 1];
   const double glast = gg, hlast = hh;
-  F[lgs_row(m - 1, F_G) + c] = gg;
-  F[lgs_row(m - 1, F_H) + c] = hh;
+  F[row_field(m - 1, F_G) * C] = -gg;
+  F[row_field(m - 1, F_H) * C] = -hh;
   for (int r = m - 2; r >= 1; --r) {
     hh = fp[r] - cp[r] * hh;
     gg = -cp[r] * gg;
-    F[lgs_row(r, F_G) + c] = gg;
-    F[lgs_row(r, F_H) + c] = hh;
+    F[row_field(r, F_G) * C] = -gg;
+    F[row_field(r, F_H) * C] = -hh;
   }
   // reduced row of chunk c in P_{c-1}, P_c, P_{c+1}
   double a0, b0, c0;
@@ -138,16 +187,16 @@ __global__ void __launch_bounds__(kLgsChunks) k_lgs_factor(Grid g, int ns, LineI
   double Ar = -a0 * hl;
   double Br = b0 - a0 * gl - c0 * hh;  // hh, gg now hold h_1, g_1
   double Cr = -c0 * gg;
-  F[lgs_chunk(m, C_A0) + c] = a0;
-  F[lgs_chunk(m, C_C0) + c] = c0;
-  for (int t = 0; t < kLgsPcr; ++t) {
+  F[chunk_field(m, C_A0) * C] = -a0;
+  F[chunk_field(m, C_C0) * C] = -c0;
+  for (int t = 0; t < steps; ++t) {
     const int s = 1 << t;
     __syncthreads();
     xa[c] = Ar;
     xb[c] = Br;
     xc[c] = Cr;
     __syncthreads();
-    const bool lo = c >= s, hi = c + s < kLgsChunks;
+    const bool lo = c >= s, hi = c + s < C;
     const double Am = lo ? xa[c - s] : 0.0, Bm = lo ? xb[c - s] : 1.0, Cm = lo ? xc[c - s] : 0.0;
     const double Ap = hi ? xa[c + s] : 0.0, Bp = hi ? xb[c + s] : 1.0, Cp = hi ? xc[c + s] : 0.0;
     const double al = lo ? -Ar / Bm : 0.0, ga = hi ? -Cr / Bp : 0.0;
@@ -155,378 +204,430 @@ __global__ void __launch_bounds__(kLgsChunks) k_lgs_factor(Grid g, int ns, LineI
     Ar = al * Am;
     Cr = ga * Cp;
     Br = nB;
-    F[lgs_chunk(m, C_AL + t) + c] = al;
-    F[lgs_chunk(m, C_GA + t) + c] = ga;
+    F[step_field(m, t, 0) * C] = al;
+    F[step_field(m, t, 1) * C] = ga;
   }
   bad |= !(Br > 0.0);
-  F[lgs_chunk(m, C_INVB) + c] = 1.0 / Br;
+  F[chunk_field(m, C_INVB) * C] = 1.0 / Br;
   if (bad) atomicCAS(err, 0, SMG_EBREAKDOWN);
+}
+
+// Line records: per column (natural index) the coefficients of the early and
+// then the three late entries (zero where the mask lacks one), negated, each
+// nzp (nz rounded up to even) wide.
+__global__ void __launch_bounds__(256) k_line_records(Grid g, int ns, LineTerms T, int nzp,
+                                                      const double* __restrict__ A, double* __restrict__ rec) {
+  const long long p = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (p >= g.n) return;
+  const long long col = p / g.nz;
+  const int k = (int)(p % g.nz), n = T.ne + 3;
+  double* r = rec + col * (long long)n * nzp + k;
+  for (int q = 0; q < n; ++q) {
+    const int e = q < T.ne ? T.ee[q] : T.le[q - T.ne];
+    r[(long long)q * nzp] = e >= 0 ? -A[p * ns + e] : 0.0;
+  }
+}
+
+// y = (couplings to later columns) x, or, with c, y = that and c = b - y.
+__global__ void __launch_bounds__(256) k_line_half(Grid g, int ns, LineTerms T, const double* __restrict__ A,
+                                                   const double* __restrict__ x, const double* __restrict__ b,
+                                                   double* __restrict__ y, double* __restrict__ c) {
+  const long long p = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (p >= g.n) return;
+  const int k = (int)(p % g.nz), j = (int)((p / g.nz) % g.ny), i = (int)(p / ((long long)g.ny * g.nz));
+  const double* a = A + p * ns;
+  double acc = 0.0;
+#pragma unroll 4
+  for (int q = 0; q < T.nh; ++q) {
+    const int a0 = i + T.hx[q], a1 = j + T.hy[q], a2 = k + T.hz[q];
+    const bool in = (unsigned)a0 < (unsigned)g.nx && (unsigned)a1 < (unsigned)g.ny && (unsigned)a2 < (unsigned)g.nz;
+    const double xv = in ? x[p + ((long long)T.hx[q] * g.ny + T.hy[q]) * g.nz + T.hz[q]] : 0.0;
+    acc = fma(a[T.he[q]], xv, acc);
+  }
+  if (y) y[p] = acc;
+  if (c) c[p] = b[p] - acc;
 }
 
 struct LsParams {
   Grid g;
-  WfCtl C;
-  Stencil s;
-  const double* A;
-  const double* F;
-  const double* b;
-  double* u;
-  int m;          // rows per chunk
-  long long blk;  // doubles per column block of F
-  int dep;        // previous-plane columns a column reads beyond its own (0 or 1)
+  LineTerms T;
+  int dir, nzp, log_stages, slots;  // record stages and columns of the previous plane kept (powers of two)
+  unsigned long long budget_ns;
+  const double *rec, *F, *b, *h;
+  double *u, *emit;
+  ulonglong2* mail;
+  SweepWs* ws;
+  int* err;
 };
 
-// Bulk (TMA, non-tensor) global -> shared copies completing on an mbarrier:
-// one thread issues a column's copies, the transaction count of the barrier
-// tracks their bytes.
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Waits for the given phase of a copy barrier, bounded by budget_ns; false
-// (and DEV_ERR_TIMEOUT in *err) when the budget runs out.
-// Bound of the waits that drain a plane's bulk copies after an abort.
-constexpr unsigned long long kLgsDrainNs = 100ull * 1000 * 1000;
+struct LineShared {
+  unsigned long long full[kMaxStages];  // records landed
+  unsigned long long rhs[2];            // right-hand side of a column formed (one arrival per active helper warp)
+  int hready;                           // columns < hready of the previous plane are in the ring
+  int done;                             // columns < done are solved
+  int abort;
+  int quit;                             // the solving warps leave in this column
+  int plane;
+};
 
-__device__ __noinline__ bool mbar_wait_bounded(unsigned long long* bar, unsigned parity, unsigned long long budget_ns,
-                                               int* err) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = globaltimer_ns();
-  for (;;) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (globaltimer_ns() - t0 > budget_ns) {
-      atomicCAS(err, 0, DEV_ERR_TIMEOUT);
-      return false;
-    }
-  }
+// Shared memory, in doubles: ring of the previous plane's columns (a zero on
+// either side), two right-hand sides, exchange rows, record stages.
+__host__ __device__ inline long long line_ring(int nz, int slots) { return (long long)slots * (nz + 2) + (slots & 1); }
+__host__ __device__ inline long long line_fixed(int nz, int C, int m, int slots) {
+  return (line_ring(nz, slots) + 1) / 2 * 2 + 2LL * C * m + 6LL * C;
+}
+__host__ __device__ inline long long line_stage(int nzp, int terms, int m, int warps) {
+  return (long long)nzp * terms + (long long)block_fields(m, warps) * 32 * warps;
 }
 
-// Shared-memory carve-up (doubles): rhs and x of the current column in the
-// chunk layout (chunk L, row r at L * (m + 1) + r), two buffers of the
-// column factors, and with STAGE two buffers of the column's matrix rows
-// [nz][ns] and right-hand side [nz].
-__host__ __device__ inline long long lgs_smem_doubles(int m, long long blk, int nz, int ns, bool stage) {
-  return 2LL * kLgsChunks * (m + 1) + kLgsChunks + 2 * blk + (stage ? 2LL * ((long long)nz * ns + nz) : 0);
+// Spin until ok() or the CTA aborts; false on abort.
+template <typename Ok>
+__device__ __forceinline__ bool wait_for(LineShared& sh, Ok&& ok) {
+  bool good = true;
+  while (!ok())
+    if (ld_acq_cta(&sh.abort)) {
+      good = false;
+      break;
+    }
+  return __all_sync(0xffffffffu, good);
 }
 
-// One off-column term of a point's right-hand side for a canonical mask
-// (compile-time offsets): acc -= a_E x_{p + o_E}.  The neighbour is read
-// unconditionally at a clamped address (its own point when off the grid, the
-// term then dropped), so all loads of a point can be issued together.
-template <int NS, int KIND, int DIR, int E>
-__device__ __forceinline__ void line_term(double (&acc)[4], const double* __restrict__ arow,
-                                          const double* __restrict__ up, const double* __restrict__ xs, int kc,
-                                          int kr, int m, int mp, const int* lin, unsigned xymask, unsigned zmask) {
-  using S = Shape<NS>;
-  constexpr int dx = S::o(E, 0), dy = S::o(E, 1), dz = S::o(E, 2);
-  constexpr bool in_column = dx == 0 && dy == 0;
-  constexpr bool earlier = DIR * dx < 0 || (dx == 0 && DIR * dy < 0);
-  if constexpr (!in_column && (KIND != SW_GS_ZERO || earlier)) {
-    const bool ok = ((xymask >> ((dx + 1) * 3 + (dy + 1))) & 1u) && ((zmask >> (dz + 1)) & 1u);
-    double x;
-    if constexpr (dx == 0 && dy == -DIR) {
-      // the previous column of the sweep, still in the x buffer (chunk layout)
-      int rc = kc, rr = kr + dz;
-      if (rr < 0) { rc -= 1; rr += m; }
-      if (rr >= m) { rc += 1; rr -= m; }
-      x = xs[ok ? rc * mp + rr : kc * mp + kr];
-    } else if constexpr (dx != 0) {
-      x = __ldcg(up + (ok ? lin[E] : 0));  // other planes: other CTAs' data, through L2
-    } else {
-      x = up[ok ? lin[E] : 0];
-    }
-    acc[E & 3] = fma(-arow[E], ok ? x : 0.0, acc[E & 3]);
-  }
-}
-
-template <int NS, int KIND, int DIR, int... Es>
-__device__ __forceinline__ void line_terms(double (&acc)[4], const double* __restrict__ arow,
-                                           const double* __restrict__ up, const double* __restrict__ xs, int kc,
-                                           int kr, int m, int mp, const int* lin, unsigned xymask, unsigned zmask,
-                                           std::integer_sequence<int, Es...>) {
-  (line_term<NS, KIND, DIR, Es>(acc, arow, up, xs, kc, kr, m, mp, lin, xymask, zmask), ...);
-}
-
-// Forward and backward elimination of rows 1..m-1 of chunk c, the PCR
-// solve of the chunk-first unknowns (through xch, kLgsChunks doubles) and
-// the recovery of the rows: x (in the chunk layout) from the right-hand side
-// d (overwritten).  Called by the kLgsChunks threads of the solving warps.
-// (xch is written and read by different threads between barriers, so it
-// carries no __restrict__: its loads must not move across the barriers.)
-__device__ __forceinline__ void lgs_solve_column(double* __restrict__ d, double* __restrict__ x,
-                                                 const double* __restrict__ fc, double* xch, int m, int c) {
-  const int mp = m + 1, base = c * mp;
-  double v = 0.0;
-  for (int r0 = 1; r0 < m; r0 += 4) {
-    double dv[4], iv[4], wv[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = r0 + q;
-      if (r < m) {
-        dv[q] = d[base + r];
-        iv[q] = fc[lgs_row(r, F_INV) + c];
-        wv[q] = fc[lgs_row(r, F_W) + c];
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = r0 + q;
-      if (r < m) {
-        // dp_r = d_r / den_r - (a_r / den_r) dp_{r-1}  (no dp_0 term in row 1)
-        v = r == 1 ? dv[q] * iv[q] : fma(-wv[q], v, dv[q] * iv[q]);
-        d[base + r] = v;
-      }
-    }
-  }
-  // backward: e_r = dp_r - c'_r e_{r+1}, from e_{m-1} = dp_{m-1} (= v)
-  for (int r0 = m - 2; r0 >= 1; r0 -= 4) {
-    double dv[4], cv[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = r0 - q;
-      if (r >= 1) {
-        dv[q] = d[base + r];
-        cv[q] = fc[lgs_row(r, F_CP) + c];
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = r0 - q;
-      if (r >= 1) {
-        v = fma(-cv[q], v, dv[q]);
-        d[base + r] = v;
-      }
-    }
-  }
-  double al[kLgsPcr], ga[kLgsPcr];
-#pragma unroll
-  for (int t = 0; t < kLgsPcr; ++t) {
-    al[t] = fc[lgs_chunk(m, C_AL + t) + c];
-    ga[t] = fc[lgs_chunk(m, C_GA + t) + c];
-  }
-  const double a0 = fc[lgs_chunk(m, C_A0) + c], c0 = fc[lgs_chunk(m, C_C0) + c];
-  const double invb = fc[lgs_chunk(m, C_INVB) + c];
-  const double e1 = d[base + 1];
-  xch[c] = d[base + m - 1];  // e_{m-1}, read by the next chunk
-  lgs_bar_solve();
-  double D = fma(-c0, e1, fma(-a0, c > 0 ? xch[c - 1] : 0.0, d[base]));
-#pragma unroll
-  for (int t = 0; t < kLgsPcr; ++t) {
-    const int s = 1 << t;
-    lgs_bar_solve();  // every read of xch is done
-    xch[c] = D;
-    lgs_bar_solve();
-    const double Dm = c >= s ? xch[c - s] : 0.0, Dp = c + s < kLgsChunks ? xch[c + s] : 0.0;
-    D = fma(al[t], Dm, fma(ga[t], Dp, D));
-  }
-  const double Pv = D * invb;
-  lgs_bar_solve();
-  xch[c] = Pv;
-  lgs_bar_solve();
-  const double Pn = c + 1 < kLgsChunks ? xch[c + 1] : 0.0;
-  x[base] = Pv;
-  for (int r0 = 1; r0 < m; r0 += 4) {
-    double ev[4], gv[4], hv[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = r0 + q;
-      if (r < m) {
-        ev[q] = d[base + r];
-        gv[q] = fc[lgs_row(r, F_G) + c];
-        hv[q] = fc[lgs_row(r, F_H) + c];
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = r0 + q;
-      if (r < m) x[base + r] = fma(-gv[q], Pn, fma(-hv[q], Pv, ev[q]));
-    }
-  }
-}
-
-// STAGE: the next column's matrix rows and right-hand side are copied to
-// shared memory while the current one is solved (needs even nz, 16-byte
-// aligned A and b, and room); otherwise they are read from global memory.
-// NS = 7, 19, 27: the canonical mask of that size (compile-time offsets);
-// NS = 0: any mask, offsets read at run time.
-template <int NS, int KIND, int DIR, bool STAGE>
-__global__ void __launch_bounds__(kLgsThreads, 1) k_lsweep(LsParams P) {
-  __shared__ WfShared sh;
-  __shared__ int s_abort;
-  __shared__ __align__(8) unsigned long long s_bar[2];  // copy barriers of the two buffers
-  __shared__ int s_landed, s_broken;
-  extern __shared__ __align__(16) double lgs_sm[];
+template <int NWS, int M>
+__global__ void __launch_bounds__((NWS + kHelpers + 2 + (NWS < 4 ? 2 - NWS : 0)) * 32, 1) k_lsweep(LsParams P) {
+  constexpr int C = 32 * NWS, STEPS = log2_chunks(NWS);
+  constexpr int FIELDS = block_fields(M, NWS);
+  __shared__ LineShared sh;
+  extern __shared__ __align__(128) double sm[];
   const Grid g = P.g;
-  const int ns = P.s.ns;
-  const int m = P.m, mp = m + 1, nzp = kLgsChunks * m;
-  const long long blk = P.blk, na = (long long)g.nz * ns;
-  // shared-memory offsets (doubles): rhs and x in the chunk layout, the PCR
-  // exchange row, two factor buffers, with STAGE two buffers of matrix rows
-  // and of b
-  const int o_rhs = 0, o_x = kLgsChunks * mp, o_xch = 2 * kLgsChunks * mp;
-  const long long o_fac = o_xch + kLgsChunks, o_a = o_fac + 2 * blk, o_b = o_a + 2 * na;
-  const double* __restrict__ A = P.A;
-  const double* __restrict__ b = P.b;
-  double* u = P.u;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nz = g.nz, terms = P.T.ne + 3;
+  double* ring = sm;
+  double* rhs = sm + (line_ring(nz, P.slots) + 1) / 2 * 2;  // two of C * M, row r of chunk c at r * C + position of c
+  double* xch = rhs + 2 * C * M;                            // six rows of C
+  double* stage0 = xch + 6 * C;
+  const long long stage_len = line_stage(P.nzp, terms, M, NWS);
+  // Warp roles, so that helpers share the sub-partitions (warp % 4) without a
+  // solving warp where there are fewer than four: solvers first, then
+  //   4 solvers: 8 helpers, loader, records;
+  //   1 or 2:    (idle,) 2 helpers, loader, records, 6 helpers.
+  int helper = -1;
+  bool is_loader = false, is_record = false;
+  if (NWS == 4) {
+    if (warp >= 4 && warp < 12) helper = warp - 4;
+    is_loader = warp == 12;
+    is_record = warp == 13;
+  } else {
+    if (warp == 2 || warp == 3) helper = warp - 2;
+    if (warp >= 6) helper = warp - 4;
+    is_loader = warp == 4;
+    is_record = warp == 5;
+  }
+  const int active = min(kHelpers, (nz + 31) / 32);  // helper warps with points
+  const unsigned tag = (unsigned)P.ws->epoch + 1u;
   if (threadIdx.x == 0) {
-    mbar_init(&s_bar[0]);
-    mbar_init(&s_bar[1]);
-    s_broken = 0;
+    for (int t = 0; t < kMaxStages; ++t) tri::mbar_init(&sh.full[t], 1);
+    tri::mbar_init(&sh.rhs[0], active);
+    tri::mbar_init(&sh.rhs[1], active);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();
-  // completed phases of each buffer's barrier (the same count in every thread)
-  unsigned fills[2] = {0u, 0u};
-  wf_run(
-      sh, P.C,
-      [&](int I) {
-        const int tid = threadIdx.x, lane = tid & 31;
-        const int i = DIR > 0 ? I : g.nx - 1 - I;
-        // bulk copies of column Jn's data into buffer Jn & 1, issued by thread 0
-        // (the buffer's previous contents were last read before the barrier
-        // that precedes this call)
-        auto prefetch = [&](int Jn) {
-          if (Jn < g.ny && tid == 0 && !s_broken) {
-            const int jn = DIR > 0 ? Jn : g.ny - 1 - Jn;
-            const long long coln = (long long)i * g.ny + jn;
-            const int sel = Jn & 1;
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            const unsigned fb = (unsigned)(blk * sizeof(double));
-            const unsigned ab = STAGE ? (unsigned)(na * sizeof(double)) : 0u;
-            const unsigned bb = STAGE ? (unsigned)(g.nz * sizeof(double)) : 0u;
-            mbar_expect_tx(&s_bar[sel], fb + ab + bb);
-            bulk_copy_g2s(lgs_sm + o_fac + sel * blk, P.F + coln * blk, fb, &s_bar[sel]);
-            if (STAGE) {
-              bulk_copy_g2s(lgs_sm + o_a + sel * na, A + coln * na, ab, &s_bar[sel]);
-              bulk_copy_g2s(lgs_sm + o_b + sel * g.nz, b + coln * g.nz, bb, &s_bar[sel]);
-            }
-          }
-        };
-        if (s_broken) {
-          // a drain gave up earlier: the copy barriers' phases are unknown, so
-          // this CTA issues no more copies and releases its planes at once
-          if (tid == 0) {
-            wf_st_rel_cta(&sh.abort_flag, 1);
-            wf_st_rel_cta(&sh.wdone[0], kWfDone);
-          }
-          return;
+  const unsigned stages = 1u << P.log_stages;
+  unsigned base = 0;  // columns of the planes before this one (every plane has ny)
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      sh.plane = atomicAdd(&P.ws->ticket, 1);
+      sh.hready = 0;
+      sh.done = 0;
+      sh.abort = 0;
+      sh.quit = INT_MAX;
+    }
+    for (int t = threadIdx.x; t < P.slots * (nz + 2); t += blockDim.x) ring[t] = 0.0;
+    for (int t = threadIdx.x; t < 2 * C * M; t += blockDim.x) rhs[t] = 0.0;  // rows beyond nz stay zero
+    __syncthreads();
+    const int I = sh.plane;
+    if (I >= g.nx) break;
+    const int i = P.dir > 0 ? I : g.nx - 1 - I;
+    auto column = [&](int J) { return (long long)i * g.ny + (P.dir > 0 ? J : g.ny - 1 - J); };
+    auto stage = [&](int J) { return stage0 + (long long)((base + J) & (stages - 1)) * stage_len; };
+    auto landed = [&](int J) {
+      const unsigned f = base + J;
+      return tri::mbar_test(&sh.full[f & (stages - 1)], (f >> P.log_stages) & 1u);
+    };
+
+    if (warp < NWS) {
+      // ---- solving warps: chunk c = lane * NWS + warp
+      const int c = lane * NWS + warp, pos = warp * 32 + lane;
+      const int k0 = c * M;
+      auto bar = [&]() {
+        if (NWS > 1) asm volatile("bar.sync 2, %0;" ::"n"(C) : "memory");
+        else __syncwarp();
+      };
+      // value of chunk c + d (0 beyond the ends), exchange row q
+      auto position = [&](int cc) { return (cc % NWS) * 32 + cc / NWS; };
+      auto from_low = [&](double v, int q) {  // chunk c - 1
+        if (NWS == 1) {
+          const double o = __shfl_up_sync(0xffffffffu, v, 1);
+          return c > 0 ? o : 0.0;
         }
-        prefetch(0);
-        int have_left = kWfDone, have_up = INT_MIN;
-        for (int J = 0; J < g.ny; ++J) {
-          const int j = DIR > 0 ? J : g.ny - 1 - J;
-          const int sel = J & 1;
-          prefetch(J + 1);
-          if (tid < 32) {
-            const int ab = wf_wait(sh, P.C, 0, J, min(J + 1 + P.dep, g.ny), have_left, have_up, lane);
-            // column J's copies have landed (thread 0 waits, whether or not
-            // the dependency wait gave up; the barrier below hands the data on
-            // to the other threads)
-            if (lane == 0) {
-              const bool landed = mbar_wait_bounded(&s_bar[sel], fills[sel] & 1u, P.C.budget_ns, P.C.err);
-              s_landed = landed;
-              s_abort = ab || !landed;
+        xch[q * C + pos] = v;
+        bar();
+        return c > 0 ? xch[q * C + position(c - 1)] : 0.0;
+      };
+      auto from_high = [&](double v, int q) {  // chunk c + 1
+        if (NWS == 1) {
+          const double o = __shfl_down_sync(0xffffffffu, v, 1);
+          return c + 1 < C ? o : 0.0;
+        }
+        xch[q * C + pos] = v;
+        bar();
+        return c + 1 < C ? xch[q * C + position(c + 1)] : 0.0;
+      };
+      double x[M], xlo = 0.0, xhi = 0.0;  // the previous column's rows, and the rows below and above them
+#pragma unroll
+      for (int r = 0; r < M; ++r) x[r] = 0.0;
+      for (int J = 0; J < g.ny; ++J) {
+        const long long col = column(J);
+        double hv[M];
+#pragma unroll
+        for (int r = 0; r < M; ++r) hv[r] = (P.h && k0 + r < nz) ? P.h[col * nz + k0 + r] : 0.0;
+        // Warp 0 waits for the right-hand side (which the helpers form once the
+        // records are there), the others for warp 0.  If it gives up it says so
+        // before the barrier, and every solving warp leaves at the end of this
+        // column (whose work is then harmless).
+        const double* rec = stage(J);
+        const double* F = rec + P.nzp * terms + pos;
+        const double* rr = rhs + ((base + J) & 1) * (C * M) + pos;
+        if (warp == 0) {
+          const bool ok =
+              wait_for(sh, [&] { return tri::mbar_test(&sh.rhs[(base + J) & 1], ((base + J) >> 1) & 1u); });
+          if (!ok && lane == 0) sh.quit = J;
+          __syncwarp();
+        }
+        bar();
+        double d[M], lc[3][M];
+#pragma unroll
+        for (int r = 0; r < M; ++r) d[r] = rr[r * C];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+          for (int r = 0; r < M; ++r) lc[q][r] = k0 + r < nz ? rec[(P.T.ne + q) * P.nzp + k0 + r] : 0.0;
+        double al[STEPS], ga[STEPS];
+#pragma unroll
+        for (int t = 0; t < STEPS; ++t) {
+          al[t] = F[step_field(M, t, 0) * C];
+          ga[t] = F[step_field(M, t, 1) * C];
+        }
+        const double a0 = F[chunk_field(M, C_A0) * C], c0 = F[chunk_field(M, C_C0) * C];
+        const double invb = F[chunk_field(M, C_INVB) * C];
+        // the previous column's terms, rows 1.. first (their elimination follows)
+        if (J > 0) {
+#pragma unroll
+          for (int rr2 = 1; rr2 <= M; ++rr2) {
+            const int r = rr2 % M;
+            if (P.T.le[0] >= 0) d[r] = fma(lc[0][r], r > 0 ? x[r > 0 ? r - 1 : 0] : xlo, d[r]);
+            if (P.T.le[1] >= 0) d[r] = fma(lc[1][r], x[r], d[r]);
+            if (P.T.le[2] >= 0) d[r] = fma(lc[2][r], r + 1 < M ? x[r + 1 < M ? r + 1 : r] : xhi, d[r]);
+          }
+        }
+        double em[M];
+#pragma unroll
+        for (int r = 0; r < M; ++r) em[r] = d[r];
+        // rows 1..M-1 in terms of P_c and P_{c+1}: d_r becomes e_r
+#pragma unroll
+        for (int r = 1; r < M; ++r) {
+          const double iv = F[row_field(r, F_INV) * C];
+          d[r] = r == 1 ? d[r] * iv : fma(F[row_field(r, F_W) * C], d[r - 1], d[r] * iv);
+        }
+#pragma unroll
+        for (int r = M - 2; r >= 1; --r) d[r] = fma(F[row_field(r, F_CP) * C], d[r + 1], d[r]);
+        const double elow = from_low(d[M - 1], 0);
+        double D = fma(c0, d[1], fma(a0, elow, d[0]));
+#pragma unroll
+        for (int t = 0; t < STEPS; ++t) {
+          const int s = 1 << t;
+          double Dm, Dp;
+          if (s < NWS) {  // the neighbours are in other warps
+            const int q = 1 + t;
+            xch[q * C + pos] = D;
+            bar();
+            Dm = c >= s ? xch[q * C + position(c >= s ? c - s : 0)] : 0.0;
+            Dp = c + s < C ? xch[q * C + position(c + s < C ? c + s : 0)] : 0.0;
+          } else {
+            Dm = __shfl_up_sync(0xffffffffu, D, s / NWS);
+            Dp = __shfl_down_sync(0xffffffffu, D, s / NWS);
+            Dm = c >= s ? Dm : 0.0;
+            Dp = c + s < C ? Dp : 0.0;
+          }
+          D = fma(al[t], Dm, fma(ga[t], Dp, D));
+        }
+        const double Pv = D * invb;
+        const double Pn = from_high(Pv, 3);
+        x[0] = Pv;
+#pragma unroll
+        for (int r = 1; r < M; ++r)
+          x[r] = fma(F[row_field(r, F_G) * C], Pn, fma(F[row_field(r, F_H) * C], Pv, d[r]));
+        ulonglong2* mb = P.mail + ((long long)I * g.ny + J) * nz;
+#pragma unroll
+        for (int r = 0; r < M; ++r)
+          if (k0 + r < nz) tri::Mail<double>::put(mb + k0 + r, x[r], tag);
+        xhi = Pn;
+        xlo = from_low(x[M - 1], 4);
+#pragma unroll
+        for (int r = 0; r < M; ++r)
+          if (k0 + r < nz) {
+            P.u[col * nz + k0 + r] = x[r];
+            if (P.emit) P.emit[col * nz + k0 + r] = em[r] + hv[r];
+          }
+        bar();  // every solving warp is past its reads of this column's records
+        // no release: what the readers of done reuse has been read, not written
+        if (threadIdx.x == 0) tri::st_relaxed_cta(&sh.done, J + 1);
+        if (sh.quit <= J) break;
+      }
+    } else if (helper >= 0 && helper < active) {
+      // ---- helper warps: the right-hand side but for the previous column's
+      // terms, one point per thread (and 256 points further)
+      for (int J = 0; J < g.ny; ++J) {
+        const long long col = column(J);
+        double bv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int k = helper * 32 + lane + 256 * q;
+          bv[q] = k < nz ? P.b[col * nz + k] : 0.0;
+        }
+        const int need = I == 0 || P.T.ne == 0 ? 0 : min(J + 1 + P.T.dep, g.ny);
+        const bool ok = wait_for(sh, [&] {
+          return ld_acq_cta(&sh.hready) >= need && ld_acq_cta(&sh.done) >= J - 1 && landed(J);
+        });
+        if (!ok) break;
+        const double* rec = stage(J);
+        double* out = rhs + ((base + J) & 1) * (C * M);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int k = helper * 32 + lane + 256 * q;
+          if (256 * q >= C * M) break;
+          if (k < C * M) {
+            double acc = bv[q];
+            if (k < nz && I > 0) {
+#pragma unroll
+              for (int e = 0; e < 9; ++e) {
+                if (e >= P.T.ne) break;
+                const int Jn = J + P.T.ec[e];
+                if ((unsigned)Jn >= (unsigned)g.ny) continue;
+                acc = fma(rec[(long long)e * P.nzp + k], ring[(Jn & (P.slots - 1)) * (nz + 2) + 1 + k + P.T.ez[e]], acc);
+              }
+            }
+            const int cc = k / M;
+            out[(k - cc * M) * C + (cc % NWS) * 32 + cc / NWS] = acc;
+          }
+        }
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tri::smem_u32(&sh.rhs[(base + J) & 1])) : "memory");
+      }
+    } else if (is_loader) {
+      // ---- loader warp: the previous plane's columns, in order
+      unsigned long long t_wait = 0;
+      unsigned iter = 0;
+      bool stop = I == 0 || P.T.ne == 0;
+      for (int J = 0; J < g.ny && !stop; ++J) {
+        const ulonglong2* mb = P.mail + ((long long)(I - 1) * g.ny + J) * nz;
+        double* dst = ring + (J & (P.slots - 1)) * (nz + 2) + 1;
+        for (int kb = 0; kb < nz && !stop;) {
+          // the slot's previous column is no longer read; up to four points a lane at once
+          bool room = true;
+          if (kb == 0) room = __shfl_sync(0xffffffffu, ld_acq_cta(&sh.done), 0) + P.slots - 2 >= J;
+          bool all = room;
+          if (room) {
+            ulonglong2 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const int k = kb + 32 * q + lane;
+              v[q] = tri::Mail<double>::value(0.0, tag);
+              if (k < nz) v[q] = tri::Mail<double>::get(mb + k);
+            }
+            bool ok = true;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) ok = ok && tri::Mail<double>::ok(v[q], tag);
+            all = __all_sync(0xffffffffu, ok);
+            if (all) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int k = kb + 32 * q + lane;
+                if (k < nz) dst[k] = tri::Mail<double>::val(v[q]);
+              }
+              kb += 128;
+              t_wait = 0;
             }
           }
-          lgs_bar();
-          if (s_abort) {
-            // drain every copy issued before leaving the plane: column J's if
-            // its wait gave up, column J + 1's always.  The drain bound does
-            // not depend on the wait budget (a copy lands in microseconds).
-            if (tid == 0) {
-              bool ok = s_landed || mbar_wait_bounded(&s_bar[sel], fills[sel] & 1u, kLgsDrainNs, P.C.err);
-              if (J + 1 < g.ny) {
-                const int s1 = (J + 1) & 1;
-                ok = mbar_wait_bounded(&s_bar[s1], fills[s1] & 1u, kLgsDrainNs, P.C.err) && ok;
+          if (!all) {
+            bool s = false;
+            if (lane == 0) {
+              if (room) {
+                // bounded: the previous plane must make progress within the budget
+                const unsigned long long now = globaltimer_ns();
+                if (t_wait == 0) t_wait = now;
+                else if (now - t_wait > P.budget_ns) {
+                  atomicCAS(P.err, 0, DEV_ERR_TIMEOUT);
+                  s = true;
+                }
               }
-              if (!ok) s_broken = 1;
+              if ((++iter & 63u) == 0) s = s || ld_relaxed(P.err) != 0;
+              s = s || ld_acq_cta(&sh.abort) != 0;
+              if (s) st_rel_cta(&sh.abort, 1);
             }
-            ++fills[sel];
-            if (J + 1 < g.ny) ++fills[(J + 1) & 1];
-            lgs_bar();
+            stop = __shfl_sync(0xffffffffu, s, 0);
+            if (!room) __nanosleep(100);
+          }
+        }
+        if (!stop) {
+          __syncwarp();
+          if (lane == 0) st_rel_cta(&sh.hready, J + 1);
+        }
+      }
+    } else if (is_record && lane == 0) {
+      // ---- record warp, one lane
+      int issued = 0;
+      bool stop = false;
+      for (int J = 0; J < g.ny && !stop; ++J) {
+        while (ld_acq_cta(&sh.done) + (int)stages <= J) {
+          if (ld_acq_cta(&sh.abort)) {
+            stop = true;
             break;
           }
-          ++fills[sel];
-          unsigned xymask = 0;
-#pragma unroll
-          for (int a = -1; a <= 1; ++a)
-#pragma unroll
-            for (int c = -1; c <= 1; ++c)
-              if ((unsigned)(i + a) < (unsigned)g.nx && (unsigned)(j + c) < (unsigned)g.ny)
-                xymask |= 1u << ((a + 1) * 3 + (c + 1));
-          const long long colbase = ((long long)i * g.ny + j) * g.nz;
-          const long long oa = o_a + sel * na, ob = o_b + sel * g.nz;
-          // right-hand side: b minus the couplings to other columns; the
-          // previous column of the sweep is still in the x buffer
-          for (int k = tid; k < nzp; k += kLgsWarps * 32) {
-            double acc[4] = {0.0, 0.0, 0.0, 0.0};
-            const int kc = k / m, kr = k - kc * m;
-            if (k < g.nz) {
-              const long long p = colbase + k;
-              acc[0] = STAGE ? lgs_sm[ob + k] : b[p];
-              const unsigned zmask = (k > 0 ? 1u : 0u) | 2u | (k + 1 < g.nz ? 4u : 0u);
-              if constexpr (NS > 0) {
-                const double* arow = STAGE ? lgs_sm + oa + (long long)k * NS : A + p * NS;
-                line_terms<NS, KIND, DIR>(acc, arow, u + p, lgs_sm + o_x, kc, kr, m, mp, P.s.lin, xymask, zmask,
-                                          std::make_integer_sequence<int, NS>{});
-              } else {
-#pragma unroll 1
-              for (int e = 0; e < ns; ++e) {
-                const int dx = P.s.off[e][0], dy = P.s.off[e][1], dz = P.s.off[e][2];
-                if (dx == 0 && dy == 0) continue;
-                if (KIND == SW_GS_ZERO && !(DIR * dx < 0 || (dx == 0 && DIR * dy < 0))) continue;
-                if (!((xymask >> ((dx + 1) * 3 + (dy + 1))) & 1u) || !((zmask >> (dz + 1)) & 1u)) continue;
-                double x;
-                if (dx == 0 && dy == -DIR) {
-                  // row k + dz of the chunk layout: same chunk unless it crosses an edge
-                  int rc = kc, rr = kr + dz;
-                  if (rr < 0) { rc -= 1; rr += m; }
-                  if (rr >= m) { rc += 1; rr -= m; }
-                  x = lgs_sm[o_x + rc * mp + rr];
-                } else if (dx != 0) {
-                  x = __ldcg(u + p + P.s.lin[e]);  // other planes: other CTAs' data, through L2
-                } else {
-                  x = u[p + P.s.lin[e]];
-                }
-                const double a = STAGE ? lgs_sm[oa + (long long)k * ns + e] : __ldg(A + p * ns + e);
-                acc[e & 3] = fma(-a, x, acc[e & 3]);
-              }
-              }
-            }
-            lgs_sm[o_rhs + kc * mp + kr] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-          }
-          lgs_bar();
-          if (tid < kLgsChunks)
-            lgs_solve_column(lgs_sm + o_rhs, lgs_sm + o_x, lgs_sm + o_fac + sel * blk, lgs_sm + o_xch, m, tid);
-          lgs_bar();
-          for (int k = tid; k < g.nz; k += kLgsWarps * 32) {
-            const int kc = k / m;
-            u[colbase + k] = lgs_sm[o_x + kc * mp + (k - kc * m)];
-          }
-          lgs_bar();  // the column's stores precede the release below
-          if (tid == 0) wf_st_rel_cta(&sh.wdone[0], J + 1);
+          __nanosleep(20);
         }
-        if (tid == 0) wf_st_rel_cta(&sh.wdone[0], kWfDone);
-      },
-      kLgsWarps);
+        if (stop) break;
+        const long long col = column(J);
+        unsigned long long* bar = &sh.full[(base + J) & (stages - 1)];
+        double* st = stage(J);
+        const unsigned rb = (unsigned)(P.nzp * terms * sizeof(double)), fb = (unsigned)(FIELDS * C * sizeof(double));
+        tri::mbar_expect_tx(bar, rb + fb);
+        if (rb) tri::bulk_copy_g2s(st, P.rec + col * (long long)(P.nzp * terms), rb, bar);
+        tri::bulk_copy_g2s(st + (long long)P.nzp * terms, P.F + col * (long long)(FIELDS * C), fb, bar);
+        issued = J + 1;
+      }
+      // every copy has landed before the plane is left
+      for (int J = max(0, issued - (int)stages); J < issued; ++J) {
+        const unsigned long long t0 = globaltimer_ns();
+        while (!landed(J))
+          if (globaltimer_ns() - t0 > tri::kCopyWaitNs) break;
+      }
+    }
+    base += (unsigned)g.ny;
+    __syncthreads();
+    if (sh.abort) break;
+  }
+  if (threadIdx.x == 0) {
+    __threadfence();
+    sh.plane = (atomicAdd(&P.ws->finished, 1) == (int)gridDim.x - 1);
+  }
+  __syncthreads();
+  if (sh.plane && threadIdx.x == 0) {
+    P.ws->ticket = 0;
+    P.ws->epoch = (int)tag;
+    __threadfence();
+    P.ws->finished = 0;
+  }
 }
 
 LineIdx line_idx(const Stencil& s) {
@@ -540,98 +641,90 @@ LineIdx line_idx(const Stencil& s) {
   return e;
 }
 
-constexpr size_t kLgsMaxSmem = 200 * 1024;
+constexpr long long kLineSmem = 216 * 1024;
 
-template <int NS>
-bool canonical_mask(const Stencil& s) {
-  if (s.ns != NS) return false;
-  for (int e = 0; e < NS; ++e)
-    for (int d = 0; d < 3; ++d)
-      if (s.off[e][d] != Shape<NS>::o(e, d)) return false;
-  return true;
-}
-
-template <int NSMAX, bool STAGE>
-cudaError_t launch_ns(int kind, int dir, const LsParams& P, int grid, size_t smem, cudaStream_t st) {
-  auto go = [&](auto kern) {
-    cudaError_t a = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (a != cudaSuccess) return a;
-    kern<<<grid, kLgsThreads, smem, st>>>(P);
-    return cudaGetLastError();
-  };
-  if (kind == SW_GS_ZERO)
-    return dir > 0 ? go(k_lsweep<NSMAX, SW_GS_ZERO, 1, STAGE>) : go(k_lsweep<NSMAX, SW_GS_ZERO, -1, STAGE>);
-  return dir > 0 ? go(k_lsweep<NSMAX, SW_GS_FULL, 1, STAGE>) : go(k_lsweep<NSMAX, SW_GS_FULL, -1, STAGE>);
-}
-
-template <int NSMAX>
-cudaError_t launch_stage(bool stage, int kind, int dir, const LsParams& P, int grid, size_t smem, cudaStream_t st) {
-  return stage ? launch_ns<NSMAX, true>(kind, dir, P, grid, smem, st)
-               : launch_ns<NSMAX, false>(kind, dir, P, grid, smem, st);
-}
-
-}  // namespace
-
-int lgs_chunk_rows(int nz) {
-  const int m = (nz + kLgsChunks - 1) / kLgsChunks;
-  return m < 2 ? 2 : m;
-}
-
-long long lgs_block_doubles(int nz) { return (long long)((lgs_chunk_rows(nz) - 1) * F_N + C_N) * kLgsChunks; }
-
-bool lgs_supported(const Grid& g, const Stencil& s) {
-  const LineIdx e = line_idx(s);
-  return e.diag >= 0 && lgs_chunk_rows(g.nz) <= kLgsMaxM && (size_t)g.nx <= (size_t)kProgSlots;
-}
-
-cudaError_t launch_lgs_setup(const Grid& g, const Stencil& s, const double* A, double* F, int* err,
-                             cudaStream_t st) {
-  if (!lgs_supported(g, s)) return cudaErrorNotSupported;
-  const LineIdx e = line_idx(s);
-  const long long ncol = (long long)g.nx * g.ny;
-  k_lgs_pivots<<<div_up(ncol, 128), 128, 0, st>>>(g, s.ns, e, A, err);
-  cudaError_t r = cudaGetLastError();
-  if (r != cudaSuccess) return r;
-  k_lgs_factor<<<(unsigned)ncol, kLgsChunks, 0, st>>>(g, s.ns, e, A, F, lgs_chunk_rows(g.nz),
-                                                       lgs_block_doubles(g.nz), err);
-  smg_count_launch(2);
+template <int NWS, int M>
+cudaError_t launch_line(LsParams P, int grid, cudaStream_t st) {
+  const int terms = P.T.ne + 3;
+  const long long per = line_stage(P.nzp, terms, M, NWS) * 8;
+  P.slots = P.g.nz <= 512 ? 8 : 4;
+  const long long fixed = line_fixed(P.g.nz, 32 * NWS, M, P.slots) * 8;
+  const long long fit = (kLineSmem - fixed) / per;
+  P.log_stages = fit >= kMaxStages ? 2 : fit >= 2 ? 1 : 0;
+  const size_t smem = (size_t)(fixed + (per << P.log_stages));
+  auto kern = k_lsweep<NWS, M>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, (NWS + kHelpers + 2 + (NWS < 4 ? 2 - NWS : 0)) * 32, smem, st>>>(P);
   return cudaGetLastError();
 }
 
-cudaError_t launch_lsweep(const Grid& g, const Stencil& s, int kind, int dir, const double* A, const double* F,
-                          const double* b, double* u, SweepWs* ws, int* err, unsigned long long budget_ns,
-                          cudaStream_t st) {
-  if (!lgs_supported(g, s) || (kind != SW_GS_ZERO && kind != SW_GS_FULL)) return cudaErrorNotSupported;
+int padded(int nz) { return nz + (nz & 1); }
+
+}  // namespace
+
+long long lgs_block_doubles(int nz) {
+  const int w = line_warps(nz);
+  return (long long)block_fields(line_rows(nz), w) * 32 * w;
+}
+
+bool lgs_supported(const Grid& g, const Stencil& s) { return line_idx(s).diag >= 0 && g.nz <= 1024; }
+
+long long lgs_record_doubles(const Grid& g, const Stencil& s, int dir) {
+  const LineTerms T = line_terms(s, dir);
+  return (long long)g.nx * g.ny * (T.ne + 3) * padded(g.nz);
+}
+
+cudaError_t launch_lgs_setup(const Grid& g, const Stencil& s, const double* A, double* F, double* recf, double* recb,
+                             int* err, cudaStream_t st) {
+  if (!lgs_supported(g, s)) return cudaErrorNotSupported;
+  const LineIdx e = line_idx(s);
+  const long long ncol = (long long)g.nx * g.ny;
+  const int warps = line_warps(g.nz);
+  k_lgs_pivots<<<div_up(ncol, 128), 128, 0, st>>>(g, s.ns, e, A, err);
+  k_lgs_factor<<<(unsigned)ncol, 32 * warps, 0, st>>>(g, s.ns, e, A, F, line_rows(g.nz), warps, err);
+  k_line_records<<<div_up(g.n, 256), 256, 0, st>>>(g, s.ns, line_terms(s, +1), padded(g.nz), A, recf);
+  k_line_records<<<div_up(g.n, 256), 256, 0, st>>>(g, s.ns, line_terms(s, -1), padded(g.nz), A, recb);
+  smg_count_launch(4);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_line_half(const Grid& g, const Stencil& s, int dir, const double* A, const double* x,
+                             const double* b, double* y, double* c, cudaStream_t st) {
+  k_line_half<<<div_up(g.n, 256), 256, 0, st>>>(g, s.ns, line_terms(s, dir), A, x, b, y, c);
+  smg_count_launch(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_lsweep(const Grid& g, const Stencil& s, int dir, const double* rec, const double* F,
+                          const double* b, const double* h, double* u, double* emit, void* mail, SweepWs* ws, int* err,
+                          unsigned long long budget_ns, cudaStream_t st) {
+  if (!lgs_supported(g, s)) return cudaErrorNotSupported;
   int dev = 0, nsm = 0;
   cudaError_t r = cudaGetDevice(&dev);
   if (r == cudaSuccess) r = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (r != cudaSuccess) return r;
   LsParams P;
   P.g = g;
-  P.C = WfCtl{g.nx, 1, 0, 0, budget_ns, ws, err};
-  P.s = s;
-  P.A = A;
+  P.T = line_terms(s, dir);
+  P.dir = dir;
+  P.nzp = padded(g.nz);
+  P.budget_ns = budget_ns;
+  P.rec = rec;
   P.F = F;
   P.b = b;
+  P.h = h;
   P.u = u;
-  P.m = lgs_chunk_rows(g.nz);
-  P.blk = lgs_block_doubles(g.nz);
-  // previous-plane columns read beyond the current one, in sweep order
-  P.dep = 0;
-  for (int t = 0; t < s.ns; ++t)
-    if (dir * s.off[t][0] == -1) P.dep = std::max(P.dep, dir * s.off[t][1]);
-  // stage the matrix rows and right-hand side of the next column in shared
-  // memory when the 16-byte copies line up and both buffers fit
-  const bool stage = g.nz % 2 == 0 && ((uintptr_t)A % 16) == 0 && ((uintptr_t)b % 16) == 0 &&
-                     lgs_smem_doubles(P.m, P.blk, g.nz, s.ns, true) * sizeof(double) <= kLgsMaxSmem;
-  // one CTA per SM: the reservation exceeds half of the SM's shared memory
-  const size_t smem =
-      std::max(kWfOneCtaPerSmSmem, (size_t)lgs_smem_doubles(P.m, P.blk, g.nz, s.ns, stage) * sizeof(double));
-  const int grid = std::min(g.nx, nsm);
-  if (canonical_mask<7>(s)) r = launch_stage<7>(stage, kind, dir, P, grid, smem, st);
-  else if (canonical_mask<19>(s)) r = launch_stage<19>(stage, kind, dir, P, grid, smem, st);
-  else if (canonical_mask<27>(s)) r = launch_stage<27>(stage, kind, dir, P, grid, smem, st);
-  else r = launch_stage<0>(stage, kind, dir, P, grid, smem, st);
+  P.emit = emit;
+  P.mail = (ulonglong2*)mail;
+  P.ws = ws;
+  P.err = err;
+  const int grid = std::min(g.nx, nsm), warps = line_warps(g.nz), m = line_rows(g.nz);
+  if (warps == 1) r = launch_line<1, 2>(P, grid, st);
+  else if (warps == 2) r = launch_line<2, 2>(P, grid, st);
+  else if (m == 2) r = launch_line<4, 2>(P, grid, st);
+  else if (m == 4) r = launch_line<4, 4>(P, grid, st);
+  else r = launch_line<4, 8>(P, grid, st);
   smg_count_launch(1);
   return r;
 }

@@ -73,7 +73,10 @@ struct Level {
   SweepWs* ws = nullptr;
   SweepCfg cfg{};
   int* ilu_upd = nullptr;
-  double* lf = nullptr;     // line Gauss-Seidel: per-column factors
+  // line Gauss-Seidel: per-column factors, the sweeps' records, the mailbox
+  // and two vectors
+  double *lf = nullptr, *lrecf = nullptr, *lrecb = nullptr, *lh = nullptr, *lc = nullptr;
+  void* lmail = nullptr;
   // sheared wavefront (canonical masks, tri.cuh): records of the lower and
   // the upper solve in the working precision, the tile order, and vectors in
   // the solves' streams (sf*: forward, sb*: backward; what a smoother lacks
@@ -296,9 +299,12 @@ static int shear_old(smg_ctx* h, Level& L, int dir, const void* u, const void** 
   return L.so ? shear(h, L, dir, u, L.so, st) : SMG_OK;
 }
 
-// One line Gauss-Seidel sweep (FP64 hierarchy only).
-static int lsweep(smg_ctx* h, Level& L, int kind, int dir, const void* b, void* u, cudaStream_t st) {
-  SMG_CUDA_TRY(launch_lsweep(L.g, L.s, kind, dir, L.A, L.lf, (const double*)b, (double*)u, L.ws, h->err,
+// One line Gauss-Seidel sweep (FP64 hierarchy only): b without the couplings
+// to later columns; emit receives b - (earlier columns) u + addend.
+static int lsweep(smg_ctx* h, Level& L, int dir, const void* b, void* u, void* emit, const void* addend,
+                  cudaStream_t st) {
+  SMG_CUDA_TRY(launch_lsweep(L.g, L.s, dir, dir > 0 ? L.lrecf : L.lrecb, L.lf, (const double*)b,
+                             (const double*)addend, (double*)u, (double*)emit, L.lmail, L.ws, h->err,
                              L.cfg.budget_ns, st));
   return SMG_OK;
 }
@@ -324,9 +330,11 @@ static int smooth_pre(smg_ctx* h, Level& L, int l, const void* f, void* u, cudaS
     return SMG_OK;
   }
   if (h->opt.smoother == SMG_SMOOTHER_LGS) {
-    TRY(lsweep(h, L, SW_GS_ZERO, +1, f, u, st));
+    // the forward sweep from zero leaves f - (earlier columns) u, the backward
+    // one's right-hand side, in t
+    TRY(lsweep(h, L, +1, f, u, L.t, nullptr, st));
     prof_mark(h, l, PM_PRE1, st);
-    TRY(lsweep(h, L, SW_GS_FULL, -1, f, u, st));
+    TRY(lsweep(h, L, -1, L.t, u, nullptr, nullptr, st));
   } else if (h->opt.smoother == SMG_SMOOTHER_SGS) {
     TRY(sweep(h, L, SW_GS_ZERO, +1, f, u, st));
     prof_mark(h, l, PM_PRE1, st);
@@ -368,9 +376,11 @@ static int smooth_post(smg_ctx* h, Level& L, int l, const void* f, void* u, cuda
     return SMG_OK;
   }
   if (h->opt.smoother == SMG_SMOOTHER_LGS) {
-    TRY(lsweep(h, L, SW_GS_FULL, +1, f, u, st));
+    SMG_CUDA_TRY(launch_line_half(L.g, L.s, +1, L.A, (const double*)u, (const double*)f, L.lh, L.lc, st));
+    prof_mark(h, l, PM_POST_RESID, st);
+    TRY(lsweep(h, L, +1, L.lc, u, L.t, L.lh, st));
     prof_mark(h, l, PM_POST1, st);
-    TRY(lsweep(h, L, SW_GS_FULL, -1, f, u, st));
+    TRY(lsweep(h, L, -1, L.t, u, nullptr, nullptr, st));
     prof_mark(h, l, PM_POST2, st);
   } else if (h->opt.smoother == SMG_SMOOTHER_SGS) {
     TRY(sweep(h, L, SW_GS_FULL, +1, f, u, st));
@@ -622,7 +632,13 @@ static int setup_level_smoother(smg_ctx* h, Level& L, cudaStream_t st) {
   if (h->opt.smoother == SMG_SMOOTHER_LGS) {
     if (!lgs_supported(L.g, L.s)) return SMG_EINVAL;
     TRY(dalloc(h, &L.lf, (long long)L.g.nx * L.g.ny * lgs_block_doubles(L.g.nz)));
-    SMG_CUDA_TRY(launch_lgs_setup(L.g, L.s, L.A, L.lf, h->err, st));
+    TRY(dalloc(h, &L.lrecf, lgs_record_doubles(L.g, L.s, +1)));
+    TRY(dalloc(h, &L.lrecb, lgs_record_doubles(L.g, L.s, -1)));
+    TRY(dev_alloc(h, &L.lmail, 16 * (size_t)n));
+    SMG_CUDA_TRY(cudaMemsetAsync(L.lmail, 0, 16 * (size_t)n, st));
+    TRY(dalloc(h, &L.lh, n));
+    TRY(dalloc(h, &L.lc, n));
+    SMG_CUDA_TRY(launch_lgs_setup(L.g, L.s, L.A, L.lf, L.lrecf, L.lrecb, h->err, st));
   } else if (h->opt.smoother == SMG_SMOOTHER_SGS) {
     TRY(dalloc(h, &L.dinv, n * B * B));
     SMG_CUDA_TRY(launch_diag_inverse(L.g, L.s, B, L.A, L.dinv, h->err, st));
@@ -1245,8 +1261,15 @@ extern "C" int smg_level_apply(smg_t h, int l, int op, const void* x, const void
     case SMG_OP_LGS_BACKWARD:
     case SMG_OP_LGS_ZERO:
       if (!has_sm || h->opt.smoother != SMG_SMOOTHER_LGS || !x || !b) return SMG_EINVAL;
-      TRY(lsweep(h, L, op == SMG_OP_LGS_ZERO ? SW_GS_ZERO : SW_GS_FULL, op == SMG_OP_LGS_BACKWARD ? -1 : +1, b,
-                 (void*)x, st));
+      {
+        const int dir = op == SMG_OP_LGS_BACKWARD ? -1 : +1;
+        const void* rhs = b;
+        if (op != SMG_OP_LGS_ZERO) {
+          SMG_CUDA_TRY(launch_line_half(L.g, L.s, dir, L.A, (const double*)x, (const double*)b, nullptr, L.lc, st));
+          rhs = L.lc;
+        }
+        TRY(lsweep(h, L, dir, rhs, (void*)x, nullptr, nullptr, st));
+      }
       break;
     case SMG_OP_ILU_APPLY:
       if (!has_sm || h->opt.smoother != SMG_SMOOTHER_ILU0 || !b || !y) return SMG_EINVAL;

@@ -209,22 +209,28 @@ cudaError_t launch_ilu_factor3(Grid g, const Stencil& s, double* LU, double* udi
 cudaError_t launch_ilu_factor(Grid g, const Stencil& s, const double* A, double* LU, double* udinv,
                               const int* upd, int nupd, SweepWs* ws, int* err, const SweepCfg& cfg, cudaStream_t st);
 
-// Line Gauss-Seidel along z (FP64, one unknown per point).  A column of nz
-// points is solved by four warps in 128 chunks of lgs_chunk_rows(nz) rows;
-// its matrix-only factors take lgs_block_doubles(nz) doubles per column,
-// columns in (i, j) order.  lgs_supported: the mask holds the centre and
-// nz <= 1024.
-int lgs_chunk_rows(int nz);
+// Line Gauss-Seidel along z (FP64, one unknown per point; any mask that holds
+// the centre, nz <= 1024).  The matrix-only factors of a column take
+// lgs_block_doubles(nz) doubles, columns in (i, j) order; the coefficients a
+// sweep of direction dir reads, lgs_record_doubles in all.
 long long lgs_block_doubles(int nz);
+long long lgs_record_doubles(const Grid& g, const Stencil& s, int dir);
 bool lgs_supported(const Grid& g, const Stencil& s);
 // Checks every column's Thomas pivots (SMG_EBREAKDOWN in *err unless all are
-// positive) and writes the factors F of every column.
-cudaError_t launch_lgs_setup(const Grid& g, const Stencil& s, const double* A, double* F, int* err, cudaStream_t st);
-// One forward (dir = +1) or backward (dir = -1) line sweep in place on u,
-// kind SW_GS_FULL, or SW_GS_ZERO (the later columns are left out).
-cudaError_t launch_lsweep(const Grid& g, const Stencil& s, int kind, int dir, const double* A, const double* F,
-                          const double* b, double* u, SweepWs* ws, int* err, unsigned long long budget_ns,
-                          cudaStream_t st);
+// positive) and writes the factors F of every column and both directions'
+// records.
+cudaError_t launch_lgs_setup(const Grid& g, const Stencil& s, const double* A, double* F, double* recf, double* recb,
+                             int* err, cudaStream_t st);
+// y = the couplings to the columns later in a sweep of direction dir, times
+// x, and c = b - y (either may be null).
+cudaError_t launch_line_half(const Grid& g, const Stencil& s, int dir, const double* A, const double* x,
+                             const double* b, double* y, double* c, cudaStream_t st);
+// u = the solution, column after column, of (lines + earlier columns) u = b;
+// emit (if not null) = b - (earlier columns) u + h (h may be null).  mail:
+// 16 bytes per point, zeroed once, shared by a level's sweeps.
+cudaError_t launch_lsweep(const Grid& g, const Stencil& s, int dir, const double* rec, const double* F,
+                          const double* b, const double* h, double* u, double* emit, void* mail, SweepWs* ws, int* err,
+                          unsigned long long budget_ns, cudaStream_t st);
 
 // Inverse diagonal (scalar 1/a_pp, or 3x3 block inverse); sets *err to
 // SMG_EBREAKDOWN on a zero pivot.

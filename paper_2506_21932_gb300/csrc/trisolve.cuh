@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "mailbox.cuh"
 #include "tri.cuh"
 
 namespace tri {
@@ -48,38 +49,7 @@ constexpr int kRecAhead = kAhead + 1;  // and loads its coefficients one step be
 constexpr int kOldest = 7;            // largest age of an operand
 constexpr int kDone = INT_MAX / 2;
 constexpr int kLanes = 33;            // ring row: lane -1 and the strip's 32
-constexpr unsigned long long kCopyWaitNs = 100ull * 1000 * 1000;  // bound on a copy in flight
 
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ int ld_acq_cta(const int* p) {
-  int v;
-  asm volatile("ld.acquire.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_rel_cta(int* p, int v) {
-  asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
-}
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
 // The step barrier: barrier 1 of N threads.
 template <int N>
 __device__ __forceinline__ void step_barrier() {
@@ -124,49 +94,6 @@ struct TriShared {
   int abort;                    // a wait ran out (or another CTA's did)
   int quit;                     // the warps of the step barrier leave in this step
   int tile;
-};
-
-// Mailbox words.  FP64: {tag | low half, tag | high half}; FP32: tag | value.
-template <typename V> struct Mail;
-template <> struct Mail<double> {
-  using word = ulonglong2;
-  static __device__ __forceinline__ void put(word* p, double v, unsigned tag) {
-    const unsigned long long t = (unsigned long long)tag << 32;
-    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(t | (unsigned)__double2loint(v)),
-                 "l"(t | (unsigned)__double2hiint(v))
-                 : "memory");
-  }
-  static __device__ __forceinline__ word get(const word* p) {
-    word w;
-    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.x), "=l"(w.y) : "l"(p) : "memory");
-    return w;
-  }
-  static __device__ __forceinline__ word value(double v, unsigned tag) {
-    const unsigned long long t = (unsigned long long)tag << 32;
-    return make_ulonglong2(t | (unsigned)__double2loint(v), t | (unsigned)__double2hiint(v));
-  }
-  static __device__ __forceinline__ bool ok(const word& w, unsigned tag) {
-    return (unsigned)(w.x >> 32) == tag && (unsigned)(w.y >> 32) == tag;
-  }
-  static __device__ __forceinline__ double val(const word& w) {
-    return __hiloint2double((int)(unsigned)w.y, (int)(unsigned)w.x);
-  }
-};
-template <> struct Mail<float> {
-  using word = unsigned long long;
-  static __device__ __forceinline__ void put(word* p, float v, unsigned tag) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(value(v, tag)) : "memory");
-  }
-  static __device__ __forceinline__ word get(const word* p) {
-    word w;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-    return w;
-  }
-  static __device__ __forceinline__ word value(float v, unsigned tag) {
-    return (unsigned long long)tag << 32 | __float_as_uint(v);
-  }
-  static __device__ __forceinline__ bool ok(const word& w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
-  static __device__ __forceinline__ float val(const word& w) { return __uint_as_float((unsigned)w); }
 };
 
 template <int G, int H>
