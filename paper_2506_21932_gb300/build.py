@@ -20,7 +20,7 @@ BUILD = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ARCH + ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 SOURCES = ["smg_api.cu", "k_stencil.cu", "k_sweep.cu", "k_sweep2.cu", "k_sweep3.cu", "k_tri_f64.cu", "k_tri_f32.cu", "k_tri_bf16.cu",
-           "k_shear.cu", "k_dense.cu", "k_ilu3.cu", "k_bsweep3.cu", "k_lsweep.cu", "k_setup.cu", "k_krylov.cu",
+           "k_shear.cu", "k_btri.cu", "k_dense.cu", "k_ilu3.cu", "k_bsweep3.cu", "k_lsweep.cu", "k_setup.cu", "k_krylov.cu",
            "k_cnn.cu", "cnn_api.cu", "noalloc.cu", "chains.cpp"]
 
 

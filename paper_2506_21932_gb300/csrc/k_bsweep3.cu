@@ -1,6 +1,6 @@
 // Point-block Gauss-Seidel (three coupled unknowns per point, Sec. 4.4
-// formulas with 3x3 blocks) for the canonical 7/19/27-point masks, on the
-// per-warp wavefront engine (wavefront.cuh):
+// formulas with 3x3 blocks) for the canonical 19/27-point masks (7-point:
+// k_btri.cu), on the per-warp wavefront engine (wavefront.cuh):
 //   u_p = D_p^{-1} (b_p - sum_{e != centre} A_pe u_{p+o_e}),
 // lower neighbours already updated, upper ones old (GS_FULL), or only the
 // lower ones from u = 0 (GS_ZERO).  Point (i,j,k) runs at t = SA*i + SB*j + k
@@ -156,8 +156,8 @@ cudaError_t launch_ns(int kind, int dir, BSweepParams& P, int grid, int nthr, cu
 cudaError_t launch_bsweep3(const LevelView& L, int kind, int dir, const void* M, const void* dinv, double w,
                            const void* b, void* u, SweepWs* ws, int* err, const SweepCfg& cfg, cudaStream_t st) {
   if (L.B != 3 || L.pk == KBF || (kind != SW_GS_ZERO && kind != SW_GS_FULL)) return cudaErrorNotSupported;
-  const bool c7 = canonical_mask<7>(L.s), c19 = canonical_mask<19>(L.s), c27 = canonical_mask<27>(L.s);
-  if (!(c7 || c19 || c27)) return cudaErrorNotSupported;
+  const bool c19 = canonical_mask<19>(L.s), c27 = canonical_mask<27>(L.s);
+  if (!(c19 || c27)) return cudaErrorNotSupported;
   int grid = 0, nthr = 0;
   cudaError_t e = wf_launch_shape(L.g, &grid, &nthr);
   if (e != cudaSuccess) return e;
@@ -171,12 +171,10 @@ cudaError_t launch_bsweep3(const LevelView& L, int kind, int dir, const void* M,
   P.u = u;
   for (int t = 0; t < 27; ++t) P.lin[t] = L.s.lin[t];
   if (L.pk == K64) {
-    if (c7) e = launch_ns<double, 7>(kind, dir, P, grid, nthr, st);
-    else if (c19) e = launch_ns<double, 19>(kind, dir, P, grid, nthr, st);
+    if (c19) e = launch_ns<double, 19>(kind, dir, P, grid, nthr, st);
     else e = launch_ns<double, 27>(kind, dir, P, grid, nthr, st);
   } else {
-    if (c7) e = launch_ns<float, 7>(kind, dir, P, grid, nthr, st);
-    else if (c19) e = launch_ns<float, 19>(kind, dir, P, grid, nthr, st);
+    if (c19) e = launch_ns<float, 19>(kind, dir, P, grid, nthr, st);
     else e = launch_ns<float, 27>(kind, dir, P, grid, nthr, st);
   }
   smg_count_launch(1);

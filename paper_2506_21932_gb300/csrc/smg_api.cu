@@ -278,17 +278,29 @@ static int tri(smg_ctx* h, Level& L, int dir, const void* b, void* u, bool flip,
   c.relax = h->opt.relax_w != 1.0 ? relax : 0;
   c.w = h->opt.relax_w;
   c.warps = h->opt.sweep_warps;
-  SMG_CUDA_TRY(launch_tri(view(h, L, true), L.ts, c, L.tiles, L.mail, L.ws, h->err, L.cfg.budget_ns, st));
+  SMG_CUDA_TRY((L.B == 3 ? launch_btri : launch_tri)(view(h, L, true), L.ts, c, L.tiles, L.mail, L.ws, h->err,
+                                                     L.cfg.budget_ns, st));
   return SMG_OK;
 }
 
 // Natural order -> stream of direction dir, and back (optionally added).
 static int shear(smg_ctx* h, Level& L, int dir, const void* src, void* dst, cudaStream_t st) {
-  SMG_CUDA_TRY(launch_shear_copy(L.g, L.ts, dir, (int)vsize(h), true, src, dst, false, st));
+  if (L.B == 3) SMG_CUDA_TRY(launch_btri_copy(L.g, L.ts, dir, h->pk, true, src, nullptr, dst, st));
+  else SMG_CUDA_TRY(launch_shear_copy(L.g, L.ts, dir, (int)vsize(h), true, src, dst, false, st));
   return SMG_OK;
 }
 static int unshear(smg_ctx* h, Level& L, int dir, const void* src, void* dst, bool add, cudaStream_t st) {
-  SMG_CUDA_TRY(launch_shear_copy(L.g, L.ts, dir, (int)vsize(h), false, src, dst, add, st));
+  if (L.B == 3) SMG_CUDA_TRY(launch_btri_copy(L.g, L.ts, dir, h->pk, false, src, nullptr, dst, st));
+  else SMG_CUDA_TRY(launch_shear_copy(L.g, L.ts, dir, (int)vsize(h), false, src, dst, add, st));
+  return SMG_OK;
+}
+static const void* block_dinv(const smg_ctx* h, const Level& L) { return h->pk == K64 ? (const void*)L.dinv : L.dinv32; }
+
+// Right-hand side of a Gauss-Seidel sweep from zero: blocks are solved with
+// the diagonal applied beforehand.
+static int shear_rhs(smg_ctx* h, Level& L, int dir, const void* b, void* dst, cudaStream_t st) {
+  if (L.B != 3) return shear(h, L, dir, b, dst, st);
+  SMG_CUDA_TRY(launch_btri_copy(L.g, L.ts, dir, h->pk, true, b, block_dinv(h, L), dst, st));
   return SMG_OK;
 }
 
@@ -311,9 +323,14 @@ static int lsweep(smg_ctx* h, Level& L, int dir, const void* b, void* u, void* e
 
 static int smooth_pre(smg_ctx* h, Level& L, int l, const void* f, void* u, cudaStream_t st) {
   if (sheared(L)) {
-    TRY(shear(h, L, +1, f, L.sf0, st));
+    TRY(shear_rhs(h, L, +1, f, L.sf0, st));
     prof_mark(h, l, PM_PACK, st);
     if (h->opt.smoother == SMG_SMOOTHER_ILU0) {
+      TRY(tri(h, L, +1, L.sf0, L.sb0, true, st));
+      prof_mark(h, l, PM_PRE1, st);
+      TRY(tri(h, L, -1, L.sb0, L.sb0, false, st));
+    } else if (L.B == 3 && h->opt.relax_w == 1.0) {
+      // D^-1 (f - L u) is u itself
       TRY(tri(h, L, +1, L.sf0, L.sb0, true, st));
       prof_mark(h, l, PM_PRE1, st);
       TRY(tri(h, L, -1, L.sb0, L.sb0, false, st));
@@ -361,8 +378,12 @@ static int smooth_post(smg_ctx* h, Level& L, int l, const void* f, void* u, cuda
     } else {
       // sf1 = (upper part) u, sf0 = f - sf1; the forward sweep then leaves
       // f - L u_new = (sf0 - L u_new) + sf1 for the backward one
-      SMG_CUDA_TRY(launch_half(view(h, L, true), +1, u, nullptr, L.t, st));
-      SMG_CUDA_TRY(launch_shear_split(L.g, L.ts, (int)vsize(h), f, L.t, L.sf0, L.sf1, st));
+      if (L.B == 3) {
+        SMG_CUDA_TRY(launch_btri_half(view(h, L, true), L.ts, +1, block_dinv(h, L), u, f, L.sf0, L.sf1, st));
+      } else {
+        SMG_CUDA_TRY(launch_half(view(h, L, true), +1, u, nullptr, L.t, st));
+        SMG_CUDA_TRY(launch_shear_split(L.g, L.ts, (int)vsize(h), f, L.t, L.sf0, L.sf1, st));
+      }
       const void* old = nullptr;
       TRY(shear_old(h, L, +1, u, &old, st));
       prof_mark(h, l, PM_POST_RESID, st);
@@ -675,15 +696,18 @@ static int setup_level_smoother(smg_ctx* h, Level& L, cudaStream_t st) {
   // point smoothers on canonical masks run as sheared wavefronts on records
   // of their own
   const bool ilu = h->opt.smoother == SMG_SMOOTHER_ILU0, sgs = h->opt.smoother == SMG_SMOOTHER_SGS;
-  if ((ilu || sgs) && tri_supported(view(h, L, true))) {
-    L.ts = tri_shape(L.g, L.s.ns, h->pk);
-    const size_t sv = tri_slots(L.ts) * vsize(h);
-    TRY(dev_alloc(h, &L.Lrec, tri_rec_bytes(L.ts, h->pk, sgs)));
-    TRY(dev_alloc(h, &L.Urec, tri_rec_bytes(L.ts, h->pk, true)));
-    if (ilu) SMG_CUDA_TRY(launch_tri_records_ilu(L.g, L.ts, h->pk, L.LU, L.udinv, L.Lrec, L.Urec, st));
+  const bool blk = sgs && btri_supported(view(h, L, true));
+  if (blk || ((ilu || sgs) && tri_supported(view(h, L, true)))) {
+    L.ts = blk ? btri_shape(L.g, h->pk) : tri_shape(L.g, L.s.ns, h->pk);
+    const size_t sv = tri_slots(L.ts) * L.B * vsize(h);
+    const size_t mail = blk ? btri_mail_bytes(L.ts, h->pk) : tri_mail_bytes(L.ts, h->pk);
+    TRY(dev_alloc(h, &L.Lrec, blk ? btri_rec_bytes(L.ts, h->pk) : tri_rec_bytes(L.ts, h->pk, sgs)));
+    TRY(dev_alloc(h, &L.Urec, blk ? btri_rec_bytes(L.ts, h->pk) : tri_rec_bytes(L.ts, h->pk, true)));
+    if (blk) SMG_CUDA_TRY(launch_btri_records(L.g, L.ts, h->pk, L.A, L.dinv, L.Lrec, L.Urec, st));
+    else if (ilu) SMG_CUDA_TRY(launch_tri_records_ilu(L.g, L.ts, h->pk, L.LU, L.udinv, L.Lrec, L.Urec, st));
     else SMG_CUDA_TRY(launch_tri_records_gs(L.g, L.ts, h->pk, L.A, L.dinv, L.Lrec, L.Urec, st));
-    TRY(dev_alloc(h, &L.mail, tri_mail_bytes(L.ts, h->pk)));
-    SMG_CUDA_TRY(cudaMemsetAsync(L.mail, 0, tri_mail_bytes(L.ts, h->pk), st));
+    TRY(dev_alloc(h, &L.mail, mail));
+    SMG_CUDA_TRY(cudaMemsetAsync(L.mail, 0, mail, st));
     TRY(dev_alloc(h, &L.sf0, sv));
     TRY(dev_alloc(h, &L.sb0, sv));
     if (sgs) {
@@ -1216,7 +1240,7 @@ extern "C" int smg_level_copy(smg_t h, int l, int which, void* dst, size_t bytes
 // where smg_sweep_noalloc's natural-order kernel (sweep3.cuh) takes the same
 // sweep and forms the same sums, so the two entry points agree to the bit.
 static bool level_op_sheared(smg_ctx* h, const Level& L, int kind) {
-  return sheared(L) && (h->pk != K64 || sweep3_supported(view(h, L, true), kind));
+  return sheared(L) && (h->pk != K64 || L.B == 3 || sweep3_supported(view(h, L, true), kind));
 }
 
 extern "C" int smg_level_apply(smg_t h, int l, int op, const void* x, const void* b, void* y, void* stream) {
@@ -1242,7 +1266,10 @@ extern "C" int smg_level_apply(smg_t h, int l, int op, const void* x, const void
         void* out = dir > 0 ? L.sf1 : L.sb0;
         const void* old = nullptr;
         if (op == SMG_OP_GS_ZERO) {
-          TRY(shear(h, L, dir, b, in, st));
+          TRY(shear_rhs(h, L, dir, b, in, st));
+        } else if (L.B == 3) {
+          SMG_CUDA_TRY(launch_btri_half(view(h, L, true), L.ts, dir, block_dinv(h, L), x, b, in, nullptr, st));
+          TRY(shear_old(h, L, dir, x, &old, st));
         } else {
           // b minus the half of A x that the sweep leaves old
           SMG_CUDA_TRY(launch_half(view(h, L, true), dir, x, b, L.t, st));

@@ -113,3 +113,25 @@ cudaError_t launch_half(const LevelView& L, int part, const void* x, const void*
 // Forward streams d0 = f - h, d1 = h from natural f, h.
 cudaError_t launch_shear_split(const Grid& g, const TriShape& t, int vb, const void* f, const void* h, void* d0,
                                void* d1, cudaStream_t st);
+
+// ---- three unknowns per point (k_btri.cu): 7-point mask, FP64 and FP32 ----------
+// The same streams with three values per slot, [slot / 32][unknown][lane], and
+// records of -D^-1 A for the lower blocks; the solves are for D^-1 b.
+bool btri_supported(const LevelView& L);
+TriShape btri_shape(const Grid& g, int pk);
+size_t btri_rec_bytes(const TriShape& t, int pk);
+size_t btri_mail_bytes(const TriShape& t, int pk);
+cudaError_t launch_btri(const LevelView& L, const TriShape& t, const TriCall& c, const int* tiles, void* mail,
+                        SweepWs* ws, int* err, unsigned long long budget_ns, cudaStream_t st);
+// Records of both solves from A [n][7][3][3] and D^-1 [n][3][3] in FP64.
+cudaError_t launch_btri_records(const Grid& g, const TriShape& t, int pk, const double* A, const double* dinv,
+                                void* Lrec, void* Urec, cudaStream_t st);
+// Vector [n][3] between natural order and a stream, times D^-1 where dinv is
+// given (into the stream only).
+cudaError_t launch_btri_copy(const Grid& g, const TriShape& t, int dir, int pk, bool to_stream, const void* src,
+                             const void* dinv, void* dst, cudaStream_t st);
+// What a sweep of direction dir leaves old: h = D^-1 (blocks after the centre
+// in sweep order) x; streams c = D^-1 b - h and h (may be null), x and b in
+// natural order.
+cudaError_t launch_btri_half(const LevelView& L, const TriShape& t, int dir, const void* dinv, const void* x,
+                             const void* b, void* c, void* h, cudaStream_t st);
