@@ -222,7 +222,8 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       int ask = 1;
       if (!__any_sync(0xffffffffu, okc)) tau = Te;
       while (tau < Te) {
-        const int n = min(min(ld_acq_cta(&sh.done) + kRing - 1, Te) - tau, ask);
+        // lane 0's view for all: the votes below need every lane
+        const int n = __shfl_sync(0xffffffffu, min(min(ld_acq_cta(&sh.done) + kRing - 1, Te) - tau, ask), 0);
         int got = 0;
         if (n > 0) {
           typename ML::word val[kBatch][3];

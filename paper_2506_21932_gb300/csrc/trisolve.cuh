@@ -403,7 +403,8 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       int ask = 1;  // one step while waiting for the first, a batch once they come
       if (!__any_sync(0xffffffffu, okc)) tau = Te;
       while (tau < Te) {
-        const int n = min(min(ld_acq_cta(&sh.done) + kRing - 4, Te) - tau, ask);
+        // lane 0's view for all: the votes below need every lane
+        const int n = __shfl_sync(0xffffffffu, min(min(ld_acq_cta(&sh.done) + kRing - 4, Te) - tau, ask), 0);
         int got = 0;
         if (n > 0) {
           typename ML::word val[kBatch];
