@@ -7,15 +7,16 @@
 // dependent instructions and a second barrier on it.  Every neighbour is one
 // step old (T = P + K): a plane has one warp per unknown, nine FMAs each.
 //
-// What bounds it: the chain of planes, a step and 1/G of a hop between CTAs
-// (about 2 us) each.  A step is the nine dependent FMAs of a warp and the
-// barrier; FP64 issues one warp instruction per 64 cycles on a sub-partition,
-// so two warps of one sub-partition take 1,150 cycles.  Lower / upper solve at
-// 128 x 128 x 64 in ms:
+// What bounds it: the chain of planes, a step and 1/G of a hop between tiles
+// each (0.45 us inside a cluster, 1.1 between clusters).  A step is the nine
+// dependent FMAs of a warp and the barrier; FP64 issues one warp instruction
+// per 64 cycles on a sub-partition, so two warps of one sub-partition take
+// 1,150 cycles.  Lower / upper solve at 128 x 128 x 64 in ms, without clusters:
 //   FP64  G = 2: 0.414 / 0.412   G = 4: 0.462 / 0.463
 //   FP32  G = 2: 0.265 / 0.262   G = 4: 0.203 / 0.201   G = 8: 0.224 / 0.226
-// (one x-plane per CTA, operands read in the step that uses them: a V-cycle
-// with 16 solves took 15.4 ms, now 3.6).
+// and in clusters of 8: FP64 0.291 / 0.291, FP32 0.147 / 0.146.  (One x-plane
+// per CTA, operands read in the step that uses them: a V-cycle with 16 solves
+// took 15.4 ms, now 2.8.)
 #include <algorithm>
 #include <climits>
 
@@ -27,6 +28,7 @@ using namespace tri;
 namespace {
 
 constexpr int kRing = 8;    // time slots of the value ring
+constexpr int kMail = 8;    // time slots of the mailbox in shared memory
 constexpr int kLanes = 33;  // ring row: lane -1 and the strip's 32
 constexpr int kStages = 8;  // record stages
 constexpr int kDone = INT_MAX / 2;
@@ -39,7 +41,7 @@ __host__ __device__ constexpr int entries_of(int G) { return 32 + G - 1; }
 
 struct BtriParams {
   Grid g;
-  int ntiles, ngrp, F;
+  int nunits, ngrp, F;
   const int* tiles;
   int flip, relax;
   unsigned long long budget_ns;
@@ -54,12 +56,17 @@ struct BtriParams {
 struct BtriShared {
   unsigned long long full[kStages];
   int hready[2];  // plane p0 - 1, the lane left of the strip
-  int rready, done, abort, quit, tile;
+  int taken;      // the next tile has taken every time < taken of the last plane
+  int rready, done, abort, tile;
 };
 
 template <typename V>
 __host__ __device__ constexpr size_t ring_bytes(int G) {
   return (sizeof(V) * 3 * (G + 1) * kRing * kLanes + 127) / 128 * 128;
+}
+template <typename V>
+__host__ __device__ constexpr size_t mail_bytes() {
+  return sizeof(typename Mail<V>::word) * 3 * kMail * 32;
 }
 template <typename V>
 __host__ __device__ constexpr unsigned stage_size(int G, int nvec) {
@@ -73,7 +80,9 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ BtriShared sh;
   V* ring = reinterpret_cast<V*>(dyn);  // [unknown][plane + 1][time][lane + 1]
-  char* stages = reinterpret_cast<char*>(dyn) + ring_bytes<V>(G);
+  // the last plane of the tile below, where the same cluster has it: [time][unknown][lane]
+  typename ML::word* own_mail = reinterpret_cast<typename ML::word*>(dyn + ring_bytes<V>(G));
+  char* stages = reinterpret_cast<char*>(dyn) + ring_bytes<V>(G) + mail_bytes<V>();
   const int nvec = 1 + (P.h != nullptr) + (P.relax == 2);
   const int hoff = G * 96, ooff = (1 + (P.h != nullptr)) * G * 96;
   const unsigned stage_bytes = stage_size<V>(G, nvec);
@@ -100,25 +109,36 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   unsigned base = 0;  // stage fills of the tiles before this one
+  const int rank = cluster_rank(), csize = cluster_size();
+  if (threadIdx.x == 0) sh.abort = 0;
   for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const int t = atomicAdd(&P.ws->ticket, 1);
-      sh.tile = t < P.ntiles ? P.tiles[t] : -1;
+    cluster_sync();
+    // the first CTA claims a unit for all, or ends the launch for all
+    if (rank == 0 && threadIdx.x == 0) {
+      bool stop = false;
+      for (int r = 0; r < csize; ++r) stop = stop || ld_peer(peer_addr(&sh.abort, r)) != 0;
+      const int t = stop ? P.nunits : atomicAdd(&P.ws->ticket, 1);
+      const int unit = t < P.nunits ? P.tiles[t] : -1;
+      for (int r = 0; r < csize; ++r) st_peer(peer_addr(&sh.tile, r), unit);
     }
-    __syncthreads();
-    if (sh.tile < 0) break;
-    const int w = sh.tile >> 16, dg = sh.tile & 0xffff;
+    cluster_sync();
+    const int tile = sh.tile;
+    if (tile < 0) break;
+    const int w = tile >> 16, dg = (tile & 0xffff) + rank;
+    const int ntile = (g.ny + min(32, g.nx - 32 * w) - 1 + G - 1) / G;  // tiles of the strip
+    const bool below = rank > 0, above = rank + 1 < csize && dg + 1 < ntile;  // neighbours in the cluster
     const int p0 = 32 * w + G * dg, T0 = p0, Te = p0 + G - 1 + g.nz - 1;
     for (int t = threadIdx.x; t < 3 * (G + 1) * kRing * kLanes; t += blockDim.x) ring[t] = V(0);
+    for (int t = threadIdx.x; t < 3 * kMail * 32; t += blockDim.x) own_mail[t] = ML::value(V(0), 0);  // tags: time + 1
     if (threadIdx.x == 0) {
       sh.hready[0] = sh.hready[1] = T0 - 1;
       sh.rready = T0;
       sh.done = T0 - 1;
       sh.abort = 0;
-      sh.quit = INT_MAX;
+      sh.taken = T0;
     }
-    __syncthreads();
+    cluster_sync();
+    if (dg >= ntile) continue;  // a unit may end early
     const int I = 32 * w + lane;
     if (warp < NC) {
       // ---- compute warps: unknown q of plane pl
@@ -130,7 +150,10 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
         return reinterpret_cast<const V*>(stage(T)) + G * 32 * kTerms + which + pl * 96 + q * 32 + lane;
       };
       long long at = colok ? column(I, p) + (long long)dstep * (T0 - 1) + 32 * q : 0;
-      const bool post = pl == G - 1 || lane == 31;
+      // every lane of the last plane, lane 31 of the others; inside the cluster
+      // the next tile's own mailbox
+      const bool near = above && pl == G - 1, post = (pl == G - 1 && !above) || lane == 31;
+      const unsigned peer = near ? peer_addr(own_mail + q * 32 + lane, rank + 1) : 0u;
       typename ML::word* mb = mail + (((long long)(w * P.ngrp + dg) * P.F - T0) * kEntries +
                                       (pl == G - 1 ? lane : 32 + pl)) * 3 + q;
       const V wv = (V)P.w;
@@ -147,9 +170,8 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       };
       const int Tb = T0 - 1;
       fetch(Tb);
-      for (int T = Tb;; ++T) {
+      for (int T = Tb; T <= Te; ++T) {
         asm volatile("bar.sync 1, %0;" ::"n"((NC + 1) * 32) : "memory");
-        if (T > Te) break;
         const int K = T - p;
         const bool ok = colok && K >= 0 && K < g.nz;
         const int s = ((T - 1) & (kRing - 1)) * kLanes;
@@ -167,37 +189,31 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
         if (P.relax) r = P.relax == 1 ? wv * r : fma(wv, r, (V(1) - wv) * *vec_of(T, ooff));
         own[q * CS + (T & (kRing - 1)) * kLanes] = ok ? r : V(0);
         if (ok) {
+          if (near)
+            ML::put_peer(peer + (T & (kMail - 1)) * (96 * (unsigned)sizeof(typename ML::word)), r, (unsigned)T + 1u);
           if (post) ML::put(mb + (long long)T * (3 * kEntries), r, tag);
           u[at] = r;
           if (ev) ev[at] = P.h ? a + *vec_of(T, hoff) : a;
         }
         at += dstep;
         fetch(T + 1);
-        if (sh.quit <= T) break;
       }
     } else if (warp == NC) {
-      // ---- sync warp
-      int hh = T0 - 1, rr = T0;
-      for (int T = T0 - 1; T <= Te + 1; ++T) {
-        bool ok = true;
-        if (T <= Te) {
-          const int need = min(T + 1, Te);
-          while (hh < T || rr <= need) {
-            hh = min(ld_acq_cta(&sh.hready[0]), ld_acq_cta(&sh.hready[1]));
-            rr = ld_acq_cta(&sh.rready);
-            if (hh >= T && rr > need) break;
-            if (ld_acq_cta(&sh.abort)) {
-              ok = false;
-              break;
-            }
-          }
+      // ---- sync warp (as in trisolve.cuh)
+      const int* word = lane < 2 ? &sh.hready[lane] : lane == 2 ? &sh.rready : &sh.taken;
+      const int ahead = lane < 2 ? 0 : lane == 2 ? 2 : above && lane == 3 ? 1 - kMail : -kDone;
+      const int most = lane == 2 ? Te + 1 : INT_MAX;
+      bool drain = false;
+      for (int T = T0 - 1; T <= Te; ++T) {
+        const int need = min(T + ahead, most);
+        unsigned iter = 0;
+        while (!drain && !__all_sync(0xffffffffu, ld_acq_cta(word) >= need)) {
+          if ((++iter & 31u) != 0) continue;
+          if ((iter & 1023u) == 0 && lane == 0 && ld_relaxed(P.err) != 0) st_relaxed_cta(&sh.abort, 1);
+          drain = __any_sync(0xffffffffu, ld_acq_cta(&sh.abort) != 0);
         }
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok && lane == 0) sh.quit = T;
-        __syncwarp();
         asm volatile("bar.sync 1, %0;" ::"n"((NC + 1) * 32) : "memory");
-        if (!ok) break;
-        if (lane == 0) st_rel_cta(&sh.done, T);
+        if (lane == 0) st_relaxed_cta(&sh.done, T);
       }
     } else if (warp < NC + 3) {
       // ---- loader warps: plane p0 - 1 (a column per lane); the column left of
@@ -221,7 +237,48 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       unsigned iter = 0;
       int ask = 1;
       if (!__any_sync(0xffffffffu, okc)) tau = Te;
-      while (tau < Te) {
+      const bool near = c == 0 && below;
+      const unsigned taken = near ? peer_addr(&sh.taken, rank - 1) : 0u;
+      unsigned long long t_near = 0;
+      while (near && tau < Te) {
+        const unsigned t1 = (unsigned)tau + 1u;
+        typename ML::word v[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          v[r] = ML::value(V(0), t1);
+          if (tau >= t_lo && tau < t_hi) v[r] = ML::get_own(own_mail + ((tau & (kMail - 1)) * 3 + r) * 32 + lane);
+        }
+        // one vote on all: a lane may see a later step than its neighbour
+        if (__all_sync(0xffffffffu, ML::ok(v[0], t1) && ML::ok(v[1], t1) && ML::ok(v[2], t1) &&
+                                        tau < ld_acq_cta(&sh.done) + kRing - 1)) {
+#pragma unroll
+          for (int r = 0; r < 3; ++r) dst[r * CS + (tau & (kRing - 1)) * kLanes] = ML::val(v[r]);
+          ++tau;
+          __syncwarp();
+          if (lane == 0) {
+            st_rel_cta(&sh.hready[c], tau);
+            if ((tau & 1) == 0) st_peer(taken, tau);
+          }
+          iter = 0;
+          continue;
+        }
+        if ((++iter & 255u) != 0) continue;
+        bool stop = false;
+        if (lane == 0) {
+          const unsigned long long now = globaltimer_ns();
+          if (iter == 256u) t_near = now;
+          else if (now - t_near > P.budget_ns) {
+            atomicCAS(P.err, 0, DEV_ERR_TIMEOUT);
+            stop = true;
+          }
+          stop = stop || ld_relaxed(P.err) != 0 || ld_acq_cta(&sh.abort) != 0;
+        }
+        if (__shfl_sync(0xffffffffu, stop, 0)) {
+          if (lane == 0) st_rel_cta(&sh.abort, 1);
+          break;
+        }
+      }
+      while (!near && tau < Te) {
         // lane 0's view for all: the votes below need every lane
         const int n = __shfl_sync(0xffffffffu, min(min(ld_acq_cta(&sh.done) + kRing - 1, Te) - tau, ask), 0);
         int got = 0;
@@ -274,7 +331,10 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
         if (ask == 1) __nanosleep(100);
         else if (n <= 0) __nanosleep(40);
       }
-      if (tau >= Te && lane == 0) st_rel_cta(&sh.hready[c], kDone);
+      if (tau >= Te && lane == 0) {
+        st_rel_cta(&sh.hready[c], kDone);
+        if (near) st_peer(taken, kDone);
+      }
     } else if (warp == NC + 3) {
       // ---- record warp, one lane
       if (lane == 0) {
@@ -345,8 +405,6 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       }
     }
     base += (unsigned)(Te - T0 + 1);
-    __syncthreads();
-    if (sh.abort) break;
   }
   if (threadIdx.x == 0) {
     __threadfence();
@@ -518,19 +576,11 @@ __global__ void __launch_bounds__(256) k_bhalf(BLine ln, const V* __restrict__ A
 BLine line_of(const Grid& g, const TriShape& t, int dir) { return BLine{g, t.G, t.F, t.groups, dir, 0, 0}; }
 
 template <typename V>
-cudaError_t go(const BtriParams& P, cudaStream_t st) {
+cudaError_t go(int CL, const BtriParams& P, cudaStream_t st) {
   constexpr int G = kPlanes<V>;
   const int nvec = 1 + (P.h != nullptr) + (P.relax == 2);
-  const size_t smem = ring_bytes<V>(G) + (size_t)kStages * stage_size<V>(G, nvec);
-  auto kern = k_btri<V>;
-  int dev = 0, nsm = 0, per = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads_of(G), smem);
-  if (e != cudaSuccess) return e;
-  kern<<<std::min(P.ntiles, nsm * std::max(1, per)), threads_of(G), smem, st>>>(P);
-  return cudaGetLastError();
+  const size_t smem = ring_bytes<V>(G) + mail_bytes<V>() + (size_t)kStages * stage_size<V>(G, nvec);
+  return launch_clusters(k_btri<V>, CL, P.nunits, threads_of(G), smem, P, st);
 }
 
 }  // namespace
@@ -550,6 +600,7 @@ TriShape btri_shape(const Grid& g, int pk) {
   t.strips = (g.nx + 31) / 32;
   t.groups = (g.ny + 31 + t.G - 1) / t.G;
   t.F = t.G - 1 + g.nz;
+  t.CL = tri_cluster(t, g, pk);
   return t;
 }
 
@@ -600,7 +651,7 @@ cudaError_t launch_btri(const LevelView& L, const TriShape& t, const TriCall& c,
                         SweepWs* ws, int* err, unsigned long long budget_ns, cudaStream_t st) {
   BtriParams P;
   P.g = L.g;
-  P.ntiles = tri_tile_count(L.g, t);
+  P.nunits = tri_unit_count(L.g, t);
   P.ngrp = t.groups;
   P.F = t.F;
   P.tiles = tiles;
@@ -617,7 +668,7 @@ cudaError_t launch_btri(const LevelView& L, const TriShape& t, const TriCall& c,
   P.mail = mail;
   P.ws = ws;
   P.err = err;
-  const cudaError_t e = L.pk == K64 ? go<double>(P, st) : go<float>(P, st);
+  const cudaError_t e = L.pk == K64 ? go<double>(t.CL, P, st) : go<float>(t.CL, P, st);
   if (e == cudaSuccess) smg_count_launch(1);
   return e;
 }

@@ -6,14 +6,14 @@ using namespace tri;
 namespace {
 
 template <int NS, bool HD>
-cudaError_t go(const TriParams& P, cudaStream_t st) {
-  return launch_tri_kernel<KBF, NS, HD, 4, 0, 16>(P, st);
+cudaError_t go(const TriShape& t, const TriParams& P, cudaStream_t st) {
+  return launch_tri_kernel<KBF, NS, HD, 4, 0, 16>(t.CL, P, st);
 }
 
 }  // namespace
 
-cudaError_t tri_launch_kbf(int ns, bool hd, const TriParams& P, cudaStream_t st) {
-  if (ns == 27) return hd ? go<27, true>(P, st) : go<27, false>(P, st);
-  if (ns == 19) return hd ? go<19, true>(P, st) : go<19, false>(P, st);
-  return hd ? go<7, true>(P, st) : go<7, false>(P, st);
+cudaError_t tri_launch_kbf(int ns, bool hd, const TriShape& t, const TriParams& P, cudaStream_t st) {
+  if (ns == 27) return hd ? go<27, true>(t, P, st) : go<27, false>(t, P, st);
+  if (ns == 19) return hd ? go<19, true>(t, P, st) : go<19, false>(t, P, st);
+  return hd ? go<7, true>(t, P, st) : go<7, false>(t, P, st);
 }

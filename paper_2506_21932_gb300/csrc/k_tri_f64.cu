@@ -19,38 +19,59 @@ bool canonical(const Stencil& s) {
 }
 
 template <int NS, bool HD>
-cudaError_t go(int G, bool helpers, const TriParams& P, cudaStream_t st) {
+cudaError_t go(const TriShape& t, bool helpers, const TriParams& P, cudaStream_t st) {
   // the 7-point mask has no terms older than one step to hand over
   if constexpr (NS == 7) {
-    return launch_tri_kernel<K64, NS, HD, 4, 0, 16>(P, st);
+    return launch_tri_kernel<K64, NS, HD, 4, 0, 16>(t.CL, P, st);
   } else {
-    if (G == 4)
-      return helpers ? launch_tri_kernel<K64, NS, HD, 4, 3, 8>(P, st) : launch_tri_kernel<K64, NS, HD, 4, 0, 8>(P, st);
-    return helpers ? launch_tri_kernel<K64, NS, HD, 2, 3, 16>(P, st) : launch_tri_kernel<K64, NS, HD, 2, 0, 16>(P, st);
+    if (t.G == 4)
+      return helpers ? launch_tri_kernel<K64, NS, HD, 4, 3, 10>(t.CL, P, st)
+                     : launch_tri_kernel<K64, NS, HD, 4, 0, 10>(t.CL, P, st);
+    return helpers ? launch_tri_kernel<K64, NS, HD, 2, 3, 16>(t.CL, P, st)
+                   : launch_tri_kernel<K64, NS, HD, 2, 0, 16>(t.CL, P, st);
   }
 }
 
 }  // namespace
 
-cudaError_t tri_launch_k64(int ns, bool hd, int G, bool helpers, const TriParams& P, cudaStream_t st) {
-  if (ns == 27) return hd ? go<27, true>(G, helpers, P, st) : go<27, false>(G, helpers, P, st);
-  if (ns == 19) return hd ? go<19, true>(G, helpers, P, st) : go<19, false>(G, helpers, P, st);
-  return hd ? go<7, true>(G, helpers, P, st) : go<7, false>(G, helpers, P, st);
+cudaError_t tri_launch_k64(int ns, bool hd, const TriShape& t, bool helpers, const TriParams& P, cudaStream_t st) {
+  if (ns == 27) return hd ? go<27, true>(t, helpers, P, st) : go<27, false>(t, helpers, P, st);
+  if (ns == 19) return hd ? go<19, true>(t, helpers, P, st) : go<19, false>(t, helpers, P, st);
+  return hd ? go<7, true>(t, helpers, P, st) : go<7, false>(t, helpers, P, st);
 }
 
-// Planes per tile.  More planes mean fewer hops between CTAs (about 2 us each)
-// and more work per SM and step.  Lower / upper solve in ms, FP64 27-point:
-//   G = 2: 0.56 / 0.59 at 128^3, 1.36 / 1.47 at 256^3
-//   G = 4: 0.62 / 0.69           1.31 / 1.44
-// (a step takes 0.34 us with 2 planes, 0.55 us with 4, where the SM's FP64
-// pipe is full; 4 pays once the tiles outnumber the SMs).  FP32 at 256^3 and
-// 384^3: 0.77 and 1.39 with 4 planes, 0.73 and 1.22 with 8; BF16 0.79 with 4,
-// 0.76 with 8 at 256^3 but 0.245 against 0.266 at 104 x 72 x 88.  The 7-point
-// mask has a short step whatever the precision.
+// Planes per tile.  More planes mean fewer hops between tiles and more work per
+// SM, but a longer step.  Lower / upper solve in ms, FP64 27-point:
+//   G = 2: 0.44 / 0.47 at 128^3, 1.34 / 1.52 at 256^3
+//   G = 4: 0.62 / 0.69           1.13 / 1.22
+// (four planes fill the SM's FP64 pipe; they pay once the tiles outnumber the
+// SMs), FP32 27-point with 4 and 8 planes: 0.23 and 0.26 at 128^3, 0.53 and 0.58
+// at 256^3, 1.09 and 1.03 at 384^3.  BF16: 4 against 8 0.245 and 0.266 at
+// 104 x 72 x 88.  The 7-point mask has a short step whatever the precision.
 static int planes_per_tile(const Grid& g, int ns, int pk) {
+  const long long plane = (long long)g.nx * g.ny;
   if (ns == 7) return 4;
-  if (pk == K64) return (long long)g.nx * g.ny > 192 * 192 ? 4 : 2;
-  return pk == K32 ? 8 : 4;
+  if (pk == K64) return plane > 192 * 192 ? 4 : 2;
+  return pk == K32 && plane > 320 * 320 ? 8 : 4;
+}
+
+static int strip_tiles(const Grid& g, const TriShape& t, int w) {
+  return (g.ny + std::min(32, g.nx - 32 * w) - 1 + t.G - 1) / t.G;
+}
+
+// Tiles per cluster (a divisor of 32 / G).  A hop inside a cluster takes 0.45
+// us, between clusters 1.1, but clusters of eight leave some SMs idle, which
+// costs more once there are several tiles per SM.  Lower solve in ms with 2, 4,
+// 8 tiles per cluster:
+//   BF16 27-point 192^3 (336 tiles) 0.489 0.428 0.405    384^3 (1248) 1.09 0.96
+//   FP64  7-point 128^3 (160)       0.204 0.179 0.167    256^3 (576)  0.68 0.68 0.80
+//   FP64 27-point 128^3 (320)       0.497 0.452 0.438    192^3 (672)  0.84 0.82 0.90
+//                 320^3 (880)       1.75  1.82           384^3 (1248) 2.56 2.70 3.53
+int tri_cluster(const TriShape& t, const Grid& g, int pk) {
+  int n = 0;
+  for (int w = 0; w < t.strips; ++w) n += strip_tiles(g, t, w);
+  const int c = n <= 340 ? 8 : pk == K64 && t.ns != 7 && t.G == 4 && n > 600 ? 2 : 4;
+  return std::min(c, 32 / t.G);
 }
 
 TriShape tri_shape(const Grid& g, int ns, int pk) {
@@ -62,6 +83,7 @@ TriShape tri_shape(const Grid& g, int ns, int pk) {
   t.strips = (g.nx + 31) / 32;
   t.groups = (g.ny + 31 + t.G - 1) / t.G;
   t.F = SB * (t.G - 1) + 31 * (SA - SB) + g.nz;
+  t.CL = tri_cluster(t, g, pk);
   return t;
 }
 
@@ -84,15 +106,16 @@ size_t tri_rec_bytes(const TriShape& t, int pk, bool hd) {
   return b * (tri_slots(t) / 32);
 }
 
-int tri_tile_count(const Grid& g, const TriShape& t) {
+int tri_unit_count(const Grid& g, const TriShape& t) {
   int n = 0;
-  for (int w = 0; w < t.strips; ++w) n += (g.ny + std::min(32, g.nx - 32 * w) - 1 + t.G - 1) / t.G;
+  for (int w = 0; w < t.strips; ++w) n += (strip_tiles(g, t, w) + t.CL - 1) / t.CL;
   return n;
 }
 
-// Tiles by the time of their first step, 32 (SP + SL) w + SP G d, the lower
-// strip first: every tile comes after the ones it waits for.
-void tri_tile_table(const Grid& g, const TriShape& t, int* out) {
+// Units by the time of their first step, 32 (SP + SL) w + SP G d, the lower
+// strip first: every unit comes after the ones its tiles wait for (CL divides
+// 32 / G, so what a unit reads of the strip on its left is in two units).
+void tri_unit_table(const Grid& g, const TriShape& t, int* out) {
   const int SA = t.ns == 27 ? Shape<27>::SA : t.ns == 19 ? Shape<19>::SA : Shape<7>::SA;
   const int SB = t.ns == 27 ? Shape<27>::SB : t.ns == 19 ? Shape<19>::SB : Shape<7>::SB;
   struct T {
@@ -100,8 +123,7 @@ void tri_tile_table(const Grid& g, const TriShape& t, int* out) {
   };
   std::vector<T> v;
   for (int w = 0; w < t.strips; ++w)
-    for (int d = 0; d < (g.ny + std::min(32, g.nx - 32 * w) - 1 + t.G - 1) / t.G; ++d)
-      v.push_back({32 * SA * w + SB * t.G * d, w, d});
+    for (int d = 0; d < strip_tiles(g, t, w); d += t.CL) v.push_back({32 * SA * w + SB * t.G * d, w, d});
   std::sort(v.begin(), v.end(), [](const T& a, const T& b) { return a.t0 != b.t0 ? a.t0 < b.t0 : a.w < b.w; });
   for (size_t q = 0; q < v.size(); ++q) out[q] = v[q].w << 16 | v[q].d;
 }
@@ -110,7 +132,7 @@ cudaError_t launch_tri(const LevelView& L, const TriShape& t, const TriCall& c, 
                        SweepWs* ws, int* err, unsigned long long budget_ns, cudaStream_t st) {
   TriParams P;
   P.g = L.g;
-  P.ntiles = tri_tile_count(L.g, t);
+  P.nunits = tri_unit_count(L.g, t);
   P.ngrp = t.groups;
   P.F = t.F;
   P.tiles = tiles;
@@ -128,9 +150,9 @@ cudaError_t launch_tri(const LevelView& L, const TriShape& t, const TriCall& c, 
   P.ws = ws;
   P.err = err;
   cudaError_t e;
-  if (L.pk == K64) e = tri_launch_k64(t.ns, c.hd, t.G, c.warps != 1, P, st);
-  else if (L.pk == K32) e = tri_launch_k32(t.ns, c.hd, P, st);
-  else e = tri_launch_kbf(t.ns, c.hd, P, st);
+  if (L.pk == K64) e = tri_launch_k64(t.ns, c.hd, t, c.warps != 1, P, st);
+  else if (L.pk == K32) e = tri_launch_k32(t.ns, c.hd, t, P, st);
+  else e = tri_launch_kbf(t.ns, c.hd, t, P, st);
   if (e == cudaSuccess) smg_count_launch(1);
   return e;
 }

@@ -1,6 +1,8 @@
 // What the wavefront kernels with mailboxes share: shared-memory counters,
 // mbarriers with bulk copies, and the mailbox words themselves.
 #pragma once
+#include <algorithm>
+
 #include "smg_internal.cuh"
 
 namespace tri {
@@ -51,7 +53,43 @@ __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, unsign
                : "memory");
 }
 
-// Mailbox words.  FP64: {tag | low half, tag | high half}; FP32: tag | value.
+// ---- thread-block clusters -------------------------------------------------
+__device__ __forceinline__ int cluster_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ int cluster_size() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// Address of p's counterpart in the shared memory of CTA rank of the cluster.
+__device__ __forceinline__ unsigned peer_addr(const void* p, int rank) {
+  unsigned a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void st_peer(unsigned a, int v) {
+  asm volatile("st.relaxed.cluster.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_peer(unsigned a) {
+  int v;
+  asm volatile("ld.relaxed.cluster.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+// A word of this CTA's shared memory that a peer writes.
+__device__ __forceinline__ int ld_own(const int* p) {
+  int v;
+  asm volatile("ld.relaxed.cluster.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+
+// Mailbox words, in global memory (put, get) or in the shared memory of the
+// reader (put_peer, get_own).  FP64: {tag | low half, tag | high half}; FP32: tag | value.
 template <typename V> struct Mail;
 template <> struct Mail<double> {
   using word = ulonglong2;
@@ -64,6 +102,18 @@ template <> struct Mail<double> {
   static __device__ __forceinline__ word get(const word* p) {
     word w;
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.x), "=l"(w.y) : "l"(p) : "memory");
+    return w;
+  }
+  static __device__ __forceinline__ void put_peer(unsigned a, double v, unsigned tag) {
+    const word w = value(v, tag);
+    asm volatile("st.relaxed.cluster.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(a), "l"(w.x), "l"(w.y) : "memory");
+  }
+  static __device__ __forceinline__ word get_own(const word* p) {
+    word w;
+    asm volatile("ld.relaxed.cluster.shared::cta.v2.u64 {%0, %1}, [%2];"
+                 : "=l"(w.x), "=l"(w.y)
+                 : "r"(smem_u32(p))
+                 : "memory");
     return w;
   }
   static __device__ __forceinline__ word value(double v, unsigned tag) {
@@ -87,11 +137,45 @@ template <> struct Mail<float> {
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
     return w;
   }
+  static __device__ __forceinline__ void put_peer(unsigned a, float v, unsigned tag) {
+    asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(value(v, tag)) : "memory");
+  }
+  static __device__ __forceinline__ word get_own(const word* p) {
+    word w;
+    asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(w) : "r"(smem_u32(p)) : "memory");
+    return w;
+  }
   static __device__ __forceinline__ word value(float v, unsigned tag) {
     return (unsigned long long)tag << 32 | __float_as_uint(v);
   }
   static __device__ __forceinline__ bool ok(const word& w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
   static __device__ __forceinline__ float val(const word& w) { return __uint_as_float((unsigned)w); }
 };
+
+// Launch in clusters of CL CTAs, one per unit of CL tiles but no more than are
+// resident at once.
+template <typename Kern, typename Params>
+cudaError_t launch_clusters(Kern kern, int CL, int nunits, int threads, size_t smem, const Params& P,
+                            cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = CL;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CL);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+  if (e != cudaSuccess) return e;
+  cfg.gridDim = dim3(CL * std::min(nunits, std::max(1, n)));
+  e = cudaLaunchKernelEx(&cfg, kern, P);
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
 
 }  // namespace tri

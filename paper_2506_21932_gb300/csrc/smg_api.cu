@@ -715,8 +715,8 @@ static int setup_level_smoother(smg_ctx* h, Level& L, cudaStream_t st) {
       TRY(dev_alloc(h, &L.sb1, sv));
       if (h->opt.relax_w != 1.0) TRY(dev_alloc(h, &L.so, sv));
     }
-    std::vector<int> tiles(tri_tile_count(L.g, L.ts));
-    tri_tile_table(L.g, L.ts, tiles.data());
+    std::vector<int> tiles(tri_unit_count(L.g, L.ts));
+    tri_unit_table(L.g, L.ts, tiles.data());
     TRY(dalloc(h, &L.tiles, tiles.size()));
     SMG_CUDA_TRY(cudaMemcpyAsync(L.tiles, tiles.data(), tiles.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     SMG_CUDA_TRY(cudaStreamSynchronize(st));  // tiles is a host temporary

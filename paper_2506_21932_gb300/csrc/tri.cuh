@@ -53,9 +53,11 @@ struct TriRec {
 // Shape of a level's streams.
 struct TriShape {
   int ns, G;              // mask, planes per tile
+  int CL;                 // consecutive tiles of a strip taken by one cluster
   int strips, groups, F;  // strips of I, groups of planes per strip, steps per tile
 };
 TriShape tri_shape(const Grid& g, int ns, int pk);
+int tri_cluster(const TriShape& t, const Grid& g, int pk);  // CL of a shape
 
 // Slots of a stream (values of one vector).
 inline size_t tri_slots(const TriShape& t) { return (size_t)t.strips * t.groups * t.F * t.G * 32; }
@@ -68,9 +70,10 @@ size_t tri_rec_bytes(const TriShape& t, int pk, bool hd);
 // a canonical 7/19/27-point mask.
 bool tri_supported(const LevelView& L);
 
-// Tile order of a level: tri_tile_count() entries strip << 16 | group.
-int tri_tile_count(const Grid& g, const TriShape& t);
-void tri_tile_table(const Grid& g, const TriShape& t, int* out);
+// Order in which the units of CL tiles are claimed: tri_unit_count() entries
+// strip << 16 | first group.
+int tri_unit_count(const Grid& g, const TriShape& t);
+void tri_unit_table(const Grid& g, const TriShape& t, int* out);
 
 struct TriCall {
   const void* rec;       // records of this solve

@@ -8,12 +8,22 @@
 // constant (plane, time, lane) offset away.  Two planes below the tile and
 // the lane left of the strip belong to other CTAs.
 //
-// Hand-over between CTAs: every point that another tile reads is also written
-// to its tile's mailbox as 64-bit words that carry half of the value (FP64)
-// or all of it (FP32) beside the launch's tag, so the word itself says whether
-// it is there: the reader polls the words it needs, without flags or fences,
-// and a hop costs about one trip to L2 and back.  Tags are the number of the
-// launch on this workspace; nothing is reset between launches.
+// What bounds a solve on all but the largest grids is the chain of time steps
+// plus one hop per tile; a step is the barrier, three dependent multiply-adds
+// and a warp's instructions one after another (27-point: 0.38 us FP64 with 2
+// planes, 0.25 FP32, 0.20 BF16; 7-point 0.27 / 0.20), so whatever else a step
+// needs is moved to other warps.  On the largest FP64 grids the FP64 pipe is
+// full (384^3: 2.45 ms a solve, 1.56 ms of multiply-adds).
+//
+// Hand-over between CTAs: every point that another tile reads is written as
+// 64-bit words that carry half of the value (FP64) or all of it (FP32) beside a
+// tag, so the word itself says whether it is there: the reader polls the words
+// it needs, without flags or fences.  CL consecutive tiles of a strip form a
+// cluster: there the words go to a mailbox of kMail time steps in the reader's
+// shared memory (tag: time + 1; the reader tells how far it has taken them) and
+// a hop takes 0.45 us.  The tiles between clusters and the strip on the right
+// read words in global memory (tag: number of the launch on this workspace, so
+// nothing is reset between launches), 1.1 us a hop.
 //
 // Warps of a CTA:
 //  * G main warps finish the points of their plane: the terms one step old
@@ -26,14 +36,15 @@
 //    step in a row.  The sums keep one order with and without helpers.
 //    Coefficients of the next step are loaded before the barrier that opens it;
 //  * the sync warp joins the step barrier once the halo and the records of
-//    the next step are there;
+//    the next step are there and the next tile has room;
 //  * three loader warps (one per plane below the tile, one for the lane left
 //    of the strip) poll the mailboxes and fill the ring, the record warp issues
-//    one bulk copy per step and array into a ring of stages, the tracker warp
-//    waits for them in order: these run ahead of the steps.
-// Tiles are claimed by a ticket in the order of their first time step, so a
-// CTA only waits for tiles that running CTAs own.  Every wait is bounded; on
-// expiry the error word is set and every CTA drains its copies and leaves.
+//    one bulk copy per array and chunk of steps into a ring of stages, the
+//    tracker warp waits for them in order: these run ahead of the steps.
+// Units of CL tiles are claimed by a ticket in the order of their first time
+// step, so a cluster only waits for tiles that running clusters own.  Every
+// wait is bounded; on expiry the error word is set, the steps of the tile run
+// through without waiting, and every CTA drains its copies and leaves.
 #pragma once
 #include <algorithm>
 #include <climits>
@@ -48,6 +59,7 @@ constexpr int kAhead = 3;             // the oldest-terms stage works kAhead ste
 constexpr int kRecAhead = kAhead + 1;  // and loads its coefficients one step before that
 constexpr int kOldest = 7;            // largest age of an operand
 constexpr int kDone = INT_MAX / 2;
+constexpr int kMail = 16;             // time slots of the mailbox in shared memory
 constexpr int kLanes = 33;            // ring row: lane -1 and the strip's 32
 
 // The step barrier: barrier 1 of N threads.
@@ -73,8 +85,9 @@ __host__ __device__ constexpr int stage_of(int e) {
 
 struct TriParams {
   Grid g;
-  int ntiles, ngrp, F;  // tiles; groups of planes per strip; steps per tile
-  const int* tiles;     // strip << 16 | group, in the order they are claimed
+  int nstg;             // record stages (steps)
+  int nunits, ngrp, F;  // units of CL tiles; groups of planes per strip; steps per tile
+  const int* tiles;     // strip << 16 | first group of a unit, in the order they are claimed
   int flip;
   unsigned long long budget_ns;
   const void *rec, *b, *h, *old;
@@ -87,12 +100,12 @@ struct TriParams {
 };
 
 struct TriShared {
-  unsigned long long full[16];  // stage barriers
+  unsigned long long full[8];   // barriers of the chunks of stages
+  int taken[2];                 // per plane that the next tile reads: it has taken every time < taken
   int hready[3];                // per loader: its halo values of every time < hready are in the ring
   int rready;                   // records and vectors of every time < rready are in their stages
   int done;                     // every step < done is finished
   int abort;                    // a wait ran out (or another CTA's did)
-  int quit;                     // the warps of the step barrier leave in this step
   int tile;
 };
 
@@ -100,6 +113,11 @@ template <int G, int H>
 __host__ __device__ constexpr int tri_threads() {
   return (G * (H + 1) + 6) * 32;
 }
+// Steps per bulk copy: a copy takes the record warp about 200 cycles to issue,
+// more than half a step of the fast kernels for the two or three of a step.
+template <int NSTG>
+constexpr int kChunk = NSTG >= 16 ? 4 : 2;
+
 template <int PK, int NS, bool HD, int G, int H>
 struct TriSmem {
   using V = typename Prec<PK>::vec;
@@ -107,7 +125,9 @@ struct TriSmem {
   static constexpr size_t ring = sizeof(V) * (G + 2) * kRing * kLanes;
   static constexpr size_t hand = H ? sizeof(V) * 3 * 2 * G * 32 : 0;
   __host__ __device__ static constexpr size_t stage(int nvec) { return (size_t)G * (RB + nvec * 32 * sizeof(V)); }
-  static constexpr size_t head = (ring + hand + 127) / 128 * 128;
+  // the last two planes of the tile below, where the same cluster has it
+  static constexpr size_t mail = sizeof(typename Mail<V>::word) * 2 * kMail * 32;
+  static constexpr size_t head = (mail + ring + hand + 127) / 128 * 128;
 };
 
 // Terms of a stage in the order they are added: sweep order, but where both
@@ -135,16 +155,16 @@ struct Terms {
   using V = typename Prec<PK>::vec;
   static constexpr int N = nterms<NS>(STG);
   V c[N ? N : 1];
-  // coefficients from a record (stored negated where the sum starts from b)
-  __device__ __forceinline__ void load(const char* rec, int lane) {
+  // coefficients from the lane's column of a record (stored negated where the sum starts from b)
+  __device__ __forceinline__ void load(const char* rec) {
 #pragma unroll
     for (int t = 0; t < N; ++t) {
       const int e = term<NS>(STG, t);
       if constexpr (PK == KBF) {
-        const unsigned wd = reinterpret_cast<const unsigned*>(rec)[(e >> 1) * 32 + lane];
+        const unsigned wd = reinterpret_cast<const unsigned*>(rec)[(e >> 1) * 32];
         c[t] = __bfloat162float(__ushort_as_bfloat16((unsigned short)((e & 1) ? (wd >> 16) : (wd & 0xffffu))));
       } else {
-        c[t] = reinterpret_cast<const V*>(rec)[e * 32 + lane];
+        c[t] = reinterpret_cast<const V*>(rec)[e * 32];
       }
     }
   }
@@ -182,18 +202,19 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
   constexpr int ME = 64 + (G > 2 ? G - 2 : 0);  // mailbox entries of a step: the last two planes, lane 31 of the others
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ TriShared sh;
-  V* ring = reinterpret_cast<V*>(dyn);
-  V* hand = reinterpret_cast<V*>(dyn + SM::ring);
-  // a stage: the records of G planes, then rows of G x 32 vector values: the
-  // right-hand side, h, the old iterate
-  const int nvec = 1 + (P.h != nullptr) + (P.relax == 2);
-  const int hoff = G * 32, ooff = (1 + (P.h != nullptr)) * G * 32;
-  const unsigned stage_bytes = (unsigned)SM::stage(nvec);
+  typename ML::word* own_mail = reinterpret_cast<typename ML::word*>(dyn);  // [plane][time][lane]
+  V* ring = reinterpret_cast<V*>(dyn + SM::mail);
+  V* hand = reinterpret_cast<V*>(dyn + SM::mail + SM::ring);
+  // stages: the records of G planes per step, then G x 32 vector values per
+  // step: the right-hand side, h, the old iterate
+  constexpr int C = kChunk<NSTG>;
+  const int nstg = P.nstg, nch = nstg / C, nvec = 1 + (P.h != nullptr) + (P.relax == 2);
+  const int hoff = nstg * G * 32, ooff = (1 + (P.h != nullptr)) * nstg * G * 32;
   char* stages = reinterpret_cast<char*>(dyn) + SM::head;
+  V* const vecs = reinterpret_cast<V*>(stages + nstg * (G * R::BYTES));
 
   const Grid g = P.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nstrip = (g.nx + 31) >> 5;
   V* u = (V*)P.u;
   V* ev = (V*)P.emit;
   // Slot of point (I, p, time T) in the result's stream: column(I, p) + dstep * T.
@@ -209,34 +230,46 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
     return (((long long)(cw * P.ngrp + cd) * P.F + SP * cg + SL * cl + k0) * G + cg) * 32 + cl;
   };
   if (threadIdx.x == 0) {
-    for (int t = 0; t < NSTG; ++t) mbar_init(&sh.full[t], 1);
+    for (int t = 0; t < nch; ++t) mbar_init(&sh.full[t], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   typename ML::word* mail = (typename ML::word*)P.mail;
   const unsigned tag = (unsigned)P.ws->epoch + 1u;
-  unsigned base = 0;  // stage fills of the tiles before this one
+  unsigned base = 0;  // chunk fills of the tiles before this one
+  const int rank = cluster_rank(), csize = cluster_size();
+  if (threadIdx.x == 0) sh.abort = 0;
   for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const int t = atomicAdd(&P.ws->ticket, 1);
-      sh.tile = t < P.ntiles ? P.tiles[t] : -1;
+    cluster_sync();
+    // the first CTA claims a unit for all, or ends the launch for all
+    if (rank == 0 && threadIdx.x == 0) {
+      bool stop = false;
+      for (int r = 0; r < csize; ++r) stop = stop || ld_peer(peer_addr(&sh.abort, r)) != 0;
+      const int t = stop ? P.nunits : atomicAdd(&P.ws->ticket, 1);
+      const int unit = t < P.nunits ? P.tiles[t] : -1;
+      for (int r = 0; r < csize; ++r) st_peer(peer_addr(&sh.tile, r), unit);
     }
-    __syncthreads();
+    cluster_sync();
     const int tile = sh.tile;
     if (tile < 0) break;
-    const int w = tile >> 16, dg = tile & 0xffff;
+    const int w = tile >> 16, dg = (tile & 0xffff) + rank;
+    const int ntile = (g.ny + min(32, g.nx - 32 * w) - 1 + G - 1) / G;  // tiles of the strip
+    const bool live = dg < ntile;                                      // a unit may end early
+    const bool below = rank > 0, above = rank + 1 < csize && dg + 1 < ntile;  // neighbours in the cluster
     const int p0 = 32 * w + G * dg;  // first plane
     const int T0 = SP * p0 + SL * 32 * w;
     const int Te = SP * (p0 + G - 1) + SL * min(32 * w + 31, g.nx - 1) + g.nz - 1;
     for (int t = threadIdx.x; t < (G + 2) * kRing * kLanes; t += blockDim.x) ring[t] = V(0);
+    // tags in it are times + 1
+    for (int t = threadIdx.x; t < 2 * kMail * 32; t += blockDim.x) own_mail[t] = ML::value(V(0), 0);
     if (threadIdx.x == 0) {
+      sh.taken[0] = sh.taken[1] = T0;
       sh.hready[0] = sh.hready[1] = sh.hready[2] = T0 - kOldest;
       sh.rready = T0;
       sh.done = T0 - kRecAhead;
       sh.abort = 0;
-      sh.quit = INT_MAX;
     }
-    __syncthreads();
+    cluster_sync();
+    if (!live) continue;
     const int I = 32 * w + lane;
 
     if (warp < NC) {
@@ -248,134 +281,168 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       } else {
         role = warp / G;
         pl = warp % G;
-        // two planes: spread the 4 + 5 + 3 + 2 FP64 instructions of a plane's
-        // warps so that every sub-partition (warp % 4) gets 7
-        if (G == 2 && role >= 2) pl = 1 - pl;
+        // two planes: the sub-partition (warp % 4) of a main warp gets the
+        // shortest helper too (4 + 2 FP64 instructions), the others share one (5 + 3)
+        if (G == 2 && role >= 2) role = 5 - role;
+        // (four planes: every sub-partition has all four kinds)
       }
       const int p = p0 + pl, J = p - I;
       const bool colok = I < g.nx && J >= 0 && J < g.ny;
-      const int koff = SP * p + SL * I;
       const V* rb = ring + pl * (kRing * kLanes) + lane + 1;
       V* own = ring + (pl + 2) * (kRing * kLanes) + lane + 1;
-      auto rec_of = [&](int T) { return stages + ((unsigned)(base + T - T0) % NSTG) * stage_bytes + pl * R::BYTES; };
-      auto vec_of = [&](int T, int which) {
-        return reinterpret_cast<const V*>(stages + ((unsigned)(base + T - T0) % NSTG) * stage_bytes + G * R::BYTES) +
-               which + pl * 32 + lane;
+      // stage of time T >= T0 - nstg and the one after it; the lane's column of
+      // the record and its vector values there
+      const int slot0 = (int)(base % (unsigned)nch) * C;
+      auto stage_of_time = [&](int T) {
+        const int t = slot0 + T - T0;
+        return t < 0 ? t + nstg : t < nstg ? t : t - nstg;
       };
+      auto next = [&](int q) { return q + 1 == nstg ? 0 : q + 1; };
+      const char* const recl = stages + pl * R::BYTES + lane * (int)sizeof(V);
+      const V* const vecl = vecs + pl * 32 + lane;
+      auto rec = [&](int q) { return recl + q * (G * R::BYTES); };
+      auto vec = [&](int q, int which) { return vecl[q * (G * 32) + which]; };
       // hand-over cells of stage pair sp: [sp][time & 1][plane][lane]
       auto cell = [&](int sp, int T) -> V& { return hand[((sp * 2 + (T & 1)) * G + pl) * 32 + lane]; };
-      long long at = colok ? column(I, p) + (long long)dstep * (T0 - kRecAhead) : 0;
       const V wv = (V)P.w;
-      // mailbox entry of this lane: every lane of the last two planes, lane 31 of the others
-      const bool post = pl >= G - 2 || lane == 31;
-      typename ML::word* mb = mail + ((long long)(w * P.ngrp + dg) * P.F - T0) * ME +
-                              (pl >= G - 2 ? (pl - (G - 2)) * 32 + lane : 64 + pl);
-      // opens step T; false after the last step.  The sync warp leaves at the
-      // barrier of step quit; a warp reads that at the end of a step, off the
-      // critical path (the step in between only does harmless work), and
-      // leaves once it has passed that barrier too.
-      auto open = [&](int T) {
-        step_barrier<(NC + 1) * 32>();
-        return T <= Te;
+      // The main warp's chain has to get into the FP64 pipe before the helpers of
+      // its sub-partition: with two planes the one there waits for it (128^3: 0.45
+      // to 0.41 ms a solve), with four, where a turn would come too late for
+      // three, they hold back by about the chain's first product (256^3: 1.21 to 1.14).
+      constexpr bool kTurn = H && G == 2;
+      auto hold = [&] {
+        if (G == 4) __nanosleep(100);
       };
-      auto start = [&](int T) { return PK == KBF ? V(0) : *vec_of(T, 0); };
+      auto start = [&](int q) { return PK == KBF ? V(0) : vec(q, 0); };
       // first step: its last loads are the first ones of a record that exists
       const int Tb = T0 - kRecAhead;
       if (role == 0) {
+        const int koff = SP * p + SL * I;
+        const unsigned nk = colok ? (unsigned)g.nz : 0u;
+        // the lane's results, mailbox entry (every lane of the last two planes,
+        // lane 31 of the others; inside the cluster the next tile's own mailbox)
+        const long long at = colok ? column(I, p) + (long long)dstep * Tb : 0;
+        V* up = u + at;
+        V* ep = ev + at;
+        const bool near = above && pl >= G - 2, post = (pl >= G - 2 && !above) || lane == 31;
+        const unsigned peer = near ? peer_addr(own_mail + (pl - (G - 2)) * (kMail * 32) + lane, rank + 1) : 0u;
+        typename ML::word* mb = mail + ((long long)(w * P.ngrp + dg) * P.F + (Tb - T0)) * ME +
+                                (pl >= G - 2 ? (pl - (G - 2)) * 32 + lane : 64 + pl);
         // H == 0: c1, c2, c3 are the partial sums of T + 1, T + 2, T + 3 before this step's share
+        constexpr bool kOlder = H == 0 && nterms<NS>(0) + nterms<NS>(1) + nterms<NS>(2) > 0;
         Terms<PK, NS, 3> k3;
         Terms<PK, NS, 2> k2;
         Terms<PK, NS, 1> k1;
         Terms<PK, NS, 0> k0;
         V d = V(0), c1 = V(0), c2 = V(0), c3 = V(0), b3 = V(0);
-        auto fetch = [&](int T) {  // operands of step T that do not depend on the step before
-          k3.load(rec_of(T), lane);
-          if (HD) d = reinterpret_cast<const V*>(rec_of(T) + R::D_OFF)[lane];
-          if (H == 0) {
-            k2.load(rec_of(T + 1), lane);
-            k1.load(rec_of(T + 2), lane);
-            k0.load(rec_of(T + 3), lane);
-            b3 = start(T + 3);
+        // stages of T, T + 1, .. T + 4
+        int q0 = stage_of_time(Tb - 1), q1 = next(q0), q2 = next(q1), q3 = next(q2), q4 = next(q3);
+        auto fetch = [&]() {  // operands of step T + 1 that do not depend on step T
+          k3.load(rec(q1));
+          if (HD) d = reinterpret_cast<const V*>(rec(q1) + R::D_OFF)[0];
+          if (kOlder) {
+            k2.load(rec(q2));
+            k1.load(rec(q3));
+            k0.load(rec(q4));
+            b3 = start(q4);
+          } else if (H == 0) {
+            c1 = start(q1);
           }
+          q0 = q1;
+          q1 = q2;
+          q2 = q3;
+          q3 = q4;
+          q4 = next(q4);
         };
-        fetch(Tb);
-        for (int T = Tb; open(T); ++T) {
-          const int K = T - koff;
-          const bool ok = colok && K >= 0 && K < g.nz;
+        fetch();
+        for (int T = Tb; T <= Te; ++T) {
+          step_barrier<(NC + 1) * 32>();
+          const bool ok = (unsigned)(T - koff) < nk;
           V a = k3.add(H ? cell(2, T) : c1, rb, T);
           if (PK == KBF) {
-            a = mul_rn(V(reinterpret_cast<const float*>(rec_of(T) + R::S_OFF)[lane]), a);
-            a = *vec_of(T, 0) - a;
+            a = mul_rn(V(reinterpret_cast<const float*>(rec(q0) + R::S_OFF)[0]), a);
+            a = vec(q0, 0) - a;
           }
           V r = a;
           if (HD) r = a * d;
-          if (P.relax) r = P.relax == 1 ? wv * r : fma(wv, r, mul_rn(V(1) - wv, *vec_of(T, ooff)));
+          if (P.relax) r = P.relax == 1 ? wv * r : fma(wv, r, mul_rn(V(1) - wv, vec(q0, ooff)));
           own[(T & (kRing - 1)) * kLanes] = ok ? r : V(0);
+          if (kTurn) asm volatile("bar.arrive 2, %0;" ::"n"(G * 64) : "memory");
           if (ok) {
-            if (post) ML::put(mb + (long long)T * ME, r, tag);
-            u[at] = r;
-            if (ev) ev[at] = P.h ? a + *vec_of(T, hoff) : a;
+            if (near)
+              ML::put_peer(peer + (T & (kMail - 1)) * (32 * (unsigned)sizeof(typename ML::word)), r, (unsigned)T + 1u);
+            if (post) ML::put(mb, r, tag);
+            *up = r;
+            if (ev) *ep = P.h ? a + vec(q0, hoff) : a;
           }
-          at += dstep;
-          if (H == 0) {
+          up += dstep;
+          ep += dstep;
+          mb += ME;
+          if (kOlder) {
             c1 = k2.add(c2, rb, T + 1);
             c2 = k1.add(c3, rb, T + 2);
             c3 = k0.add(b3, rb, T + 3);
           }
-          fetch(T + 1);
-          if (sh.quit <= T) break;
+          fetch();
         }
       } else if (role == 1) {
         Terms<PK, NS, 0> k;
-        k.load(rec_of(Tb + 3), lane);
-        V b3 = start(Tb + 3);
-        for (int T = Tb; open(T); ++T) {
+        int q = stage_of_time(Tb + 3);
+        k.load(rec(q));
+        V b3 = start(q);
+        for (int T = Tb; T <= Te; ++T) {
+          step_barrier<(NC + 1) * 32>();
+          hold();
           cell(0, T + 3) = k.add(b3, rb, T + 3);
-          k.load(rec_of(T + 4), lane);
-          b3 = start(T + 4);
-          if (sh.quit <= T) break;
+          q = next(q);
+          k.load(rec(q));
+          b3 = start(q);
         }
       } else if (role == 2) {
         Terms<PK, NS, 1> k;
-        k.load(rec_of(Tb + 2), lane);
-        for (int T = Tb; open(T); ++T) {
+        int q = stage_of_time(Tb + 2);
+        k.load(rec(q));
+        for (int T = Tb; T <= Te; ++T) {
+          step_barrier<(NC + 1) * 32>();
+          hold();
           cell(1, T + 2) = k.add(cell(0, T + 2), rb, T + 2);
-          k.load(rec_of(T + 3), lane);
-          if (sh.quit <= T) break;
+          q = next(q);
+          k.load(rec(q));
         }
       } else {
         Terms<PK, NS, 2> k;
-        k.load(rec_of(Tb + 1), lane);
-        for (int T = Tb; open(T); ++T) {
+        int q = stage_of_time(Tb + 1);
+        k.load(rec(q));
+        for (int T = Tb; T <= Te; ++T) {
+          step_barrier<(NC + 1) * 32>();
+          hold();
+          if (kTurn) asm volatile("bar.sync 2, %0;" ::"n"(G * 64) : "memory");
           cell(2, T + 1) = k.add(cell(1, T + 1), rb, T + 1);
-          k.load(rec_of(T + 2), lane);
-          if (sh.quit <= T) break;
+          q = next(q);
+          k.load(rec(q));
         }
       }
     } else if (warp == NC) {
-      // ---- sync warp
-      int hh = T0 - kOldest, rr = T0;
-      for (int T = T0 - kRecAhead; T <= Te + 1; ++T) {
-        bool ok = true;
-        if (T <= Te) {
-          // halo values up to time T - 1, records up to the one loaded in this step
-          const int need = min(T + kRecAhead, Te);
-          while (hh < T || rr <= need) {
-            hh = min(min(ld_acq_cta(&sh.hready[0]), ld_acq_cta(&sh.hready[1])), ld_acq_cta(&sh.hready[2]));
-            rr = ld_acq_cta(&sh.rready);
-            if (hh >= T && rr > need) break;
-            if (ld_acq_cta(&sh.abort)) {
-              ok = false;
-              break;
-            }
-          }
+      // ---- sync warp: every lane watches one word, one load and one vote a look.
+      // Step T takes halo values up to time T - 1, records up to T + kRecAhead,
+      // and the places of values that the next tile has taken.
+      const int* word = lane < 3 ? &sh.hready[lane] : lane == 3 ? &sh.rready : &sh.taken[lane & 1];
+      const int ahead = lane < 3 ? 0 : lane == 3 ? kRecAhead + 1 : above && lane < 6 ? 1 - kMail : -kDone;
+      const int most = lane == 3 ? Te + 1 : INT_MAX;
+      // Once a wait has run out the remaining steps run through on what is there
+      // (nothing leaves its buffers, and the error word says what came of it).
+      bool drain = false;
+      for (int T = T0 - kRecAhead; T <= Te; ++T) {
+        const int need = min(T + ahead, most);
+        unsigned iter = 0;
+        while (!drain && !__all_sync(0xffffffffu, ld_acq_cta(word) >= need)) {
+          if ((++iter & 31u) != 0) continue;
+          // the waits of the next tile are bounded; it leaves the error word behind
+          if ((iter & 1023u) == 0 && lane == 0 && ld_relaxed(P.err) != 0) st_relaxed_cta(&sh.abort, 1);
+          drain = __any_sync(0xffffffffu, ld_acq_cta(&sh.abort) != 0);
         }
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok && lane == 0) sh.quit = T;
-        __syncwarp();
         step_barrier<(NC + 1) * 32>();
-        if (!ok) break;
-        if (lane == 0) st_rel_cta(&sh.done, T);
+        if (lane == 0) st_relaxed_cta(&sh.done, T);  // behind the barrier: the steps before have read what they need
       }
     } else if (warp < NC + 4) {
       // ---- loader warps: plane p0-2, plane p0-1 (a column per lane), and the
@@ -394,6 +461,9 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       const int e = cg >= G - 2 ? (cg - (G - 2)) * 32 + (c < 2 ? lane : 31) : 64 + cg;
       const typename ML::word* src =  // entry of time 0
           okc ? mail + ((long long)(cw * P.ngrp + cd) * P.F - ct0) * ME + e : mail;
+      const bool near = c < 2 && below;
+      const typename ML::word* box = own_mail + (c & 1) * (kMail * 32) + lane;
+      const unsigned taken = near ? peer_addr(&sh.taken[c], rank - 1) : 0u;
       V* dst = ring + (c < 2 ? c : min(lane, G + 1)) * (kRing * kLanes) + (c < 2 ? lane + 1 : 0);
       // times at which this lane has a point to fetch
       const int t_lo = okc ? SP * pc + SL * Ic : INT_MAX, t_hi = okc ? t_lo + g.nz : INT_MIN;
@@ -402,7 +472,42 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       unsigned iter = 0;
       int ask = 1;  // one step while waiting for the first, a batch once they come
       if (!__any_sync(0xffffffffu, okc)) tau = Te;
-      while (tau < Te) {
+      // the tile below in this cluster: it writes to the own mailbox, a word of
+      // every step at a time
+      unsigned long long t_near = 0;
+      while (near && tau < Te) {
+        const unsigned t1 = (unsigned)tau + 1u;
+        typename ML::word v = ML::value(V(0), t1);
+        if (tau >= t_lo && tau < t_hi) v = ML::get_own(box + (tau & (kMail - 1)) * 32);
+        // one vote on both: a lane may see a later step than its neighbour
+        if (__all_sync(0xffffffffu, ML::ok(v, t1) && tau < ld_acq_cta(&sh.done) + kRing - 4)) {
+          dst[(tau & (kRing - 1)) * kLanes] = ML::val(v);
+          ++tau;
+          __syncwarp();
+          if (lane == 0) {
+            st_rel_cta(&sh.hready[c], tau);
+            if ((tau & 3) == 0) st_peer(taken, tau);
+          }
+          iter = 0;
+          continue;
+        }
+        if ((++iter & 255u) != 0) continue;
+        bool stop = false;
+        if (lane == 0) {
+          const unsigned long long now = globaltimer_ns();
+          if (iter == 256u) t_near = now;
+          else if (now - t_near > P.budget_ns) {
+            atomicCAS(P.err, 0, DEV_ERR_TIMEOUT);
+            stop = true;
+          }
+          stop = stop || ld_relaxed(P.err) != 0 || ld_acq_cta(&sh.abort) != 0;
+        }
+        if (__shfl_sync(0xffffffffu, stop, 0)) {
+          if (lane == 0) st_rel_cta(&sh.abort, 1);
+          break;
+        }
+      }
+      while (!near && tau < Te) {
         // lane 0's view for all: the votes below need every lane
         const int n = __shfl_sync(0xffffffffu, min(min(ld_acq_cta(&sh.done) + kRing - 4, Te) - tau, ask), 0);
         int got = 0;
@@ -450,7 +555,10 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
         else if (n <= 0) __nanosleep(40);
       }
       // the last steps need no more halo
-      if (tau >= Te && lane == 0) st_rel_cta(&sh.hready[c], kDone);
+      if (tau >= Te && lane == 0) {
+        st_rel_cta(&sh.hready[c], kDone);
+        if (near) st_peer(taken, kDone);
+      }
     } else if (warp == NC + 4) {
       // ---- record warp
       // one lane; step f of the tile is one run in every stream
@@ -462,14 +570,14 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
         const V* hv = (const V*)P.h + step0 * (G * 32);
         const V* ov = (const V*)P.old + step0 * (G * 32);
         constexpr unsigned vbytes = G * 32 * sizeof(V);
-        int done = T0 - kRecAhead, issued = 0;
-        for (int f = 0; f < nfill; ++f) {
-          const int T = T0 + f;
-          // the stage's previous occupant (time T - NSTG) is finished
+        int done = T0 - kRecAhead, ch = (int)(base % (unsigned)nch), issued = 0;
+        for (int f = 0; f < nfill; f += C) {
+          // the previous occupants of the chunk, up to time T0 + f + C - 1 - nstg, are finished
+          const int free_at = T0 + f + C - 1 - nstg;
           bool stop = false;
-          while (f >= NSTG && done <= T - NSTG) {
+          while (f >= nstg && done <= free_at) {
             done = ld_acq_cta(&sh.done);
-            if (done > T - NSTG) break;
+            if (done > free_at) break;
             if (ld_acq_cta(&sh.abort)) {
               stop = true;
               break;
@@ -477,40 +585,41 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
             __nanosleep(20);
           }
           if (stop) break;
-          const unsigned slot = (base + f) % NSTG;
-          unsigned long long* bar = &sh.full[slot];
-          char* st = stages + slot * stage_bytes;
-          V* sv = reinterpret_cast<V*>(st + G * R::BYTES);
-          mbar_expect_tx(bar, stage_bytes);
-          bulk_copy_g2s(st, rec + (long long)f * (G * R::BYTES), G * R::BYTES, bar);
-          bulk_copy_g2s(sv, bv + (long long)f * (G * 32), vbytes, bar);
-          if (P.h) bulk_copy_g2s(sv + hoff, hv + (long long)f * (G * 32), vbytes, bar);
-          if (P.relax == 2) bulk_copy_g2s(sv + ooff, ov + (long long)f * (G * 32), vbytes, bar);
-          issued = f + 1;
+          const int n = min(C, nfill - f);
+          unsigned long long* bar = &sh.full[ch];
+          V* sv = vecs + ch * (C * G * 32);
+          mbar_expect_tx(bar, n * (unsigned)(G * R::BYTES + nvec * vbytes));
+          bulk_copy_g2s(stages + ch * (C * G * R::BYTES), rec + (long long)f * (G * R::BYTES), n * G * R::BYTES, bar);
+          bulk_copy_g2s(sv, bv + (long long)f * (G * 32), n * vbytes, bar);
+          if (P.h) bulk_copy_g2s(sv + hoff, hv + (long long)f * (G * 32), n * vbytes, bar);
+          if (P.relax == 2) bulk_copy_g2s(sv + ooff, ov + (long long)f * (G * 32), n * vbytes, bar);
+          ++issued;
+          ch = ch + 1 == nch ? 0 : ch + 1;
         }
         // every copy has landed before the tile is left (at once, unless a wait
         // ran out and the tracker left early)
-        for (int f = max(0, issued - NSTG); f < issued; ++f) {
+        for (int f = max(0, issued - nch); f < issued; ++f) {
           const unsigned a = base + f;
           const unsigned long long t0 = globaltimer_ns();
-          while (!mbar_try_wait(&sh.full[a % NSTG], (a / NSTG) & 1u))
+          while (!mbar_try_wait(&sh.full[a % nch], (a / nch) & 1u))
             if (globaltimer_ns() - t0 > kCopyWaitNs) break;
         }
       }
     } else if (lane == 0) {
       // ---- tracker warp, one lane
       bool stop = false;
-      for (int T = T0; T <= Te && !stop; ++T) {
-        const unsigned f = base + (T - T0);
+      int ch = (int)(base % (unsigned)nch);
+      unsigned parity = (base / (unsigned)nch) & 1u;
+      for (int T = T0; T <= Te && !stop; T += C) {
         unsigned long long t0 = 0;
-        while (!mbar_try_wait(&sh.full[f % NSTG], (f / NSTG) & 1u)) {
+        while (!mbar_try_wait(&sh.full[ch], parity)) {
           if (ld_acq_cta(&sh.abort)) {
             stop = true;
             break;
           }
           // the record warp waits for the steps, the steps for the halo: only
           // a copy that is due counts against the bound
-          if (T > ld_acq_cta(&sh.done) + NSTG - 2) {
+          if (T + C > ld_acq_cta(&sh.done) + nstg - 1) {
             t0 = 0;
             continue;
           }
@@ -523,12 +632,12 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
             break;
           }
         }
-        if (!stop) st_rel_cta(&sh.rready, T + 1);
+        if (!stop) st_rel_cta(&sh.rready, T + C);
+        ch = ch + 1 == nch ? 0 : ch + 1;
+        parity ^= ch == 0;
       }
     }
-    base += (unsigned)(Te - T0 + 1);
-    __syncthreads();
-    if (sh.abort) break;
+    base += (unsigned)((Te - T0 + C) / C);
   }
   if (threadIdx.x == 0) {
     __threadfence();
@@ -544,25 +653,20 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
 }
 
 template <int PK, int NS, bool HD, int G, int H, int NSTG>
-cudaError_t launch_tri_kernel(const TriParams& P, cudaStream_t st) {
+cudaError_t launch_tri_kernel(int CL, const TriParams& P, cudaStream_t st) {
   using SM = TriSmem<PK, NS, HD, G, H>;
   const int nvec = 1 + (P.h != nullptr) + (P.relax == 2);
-  const size_t smem = SM::head + NSTG * SM::stage(nvec);
-  auto kern = k_tri<PK, NS, HD, G, H, NSTG>;
-  int dev = 0, nsm = 0, per = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, tri_threads<G, H>(), smem);
-  if (e != cudaSuccess) return e;
-  const int grid = std::min(P.ntiles, nsm * std::max(1, per));
-  kern<<<grid, tri_threads<G, H>(), smem, st>>>(P);
-  return cudaGetLastError();
+  // as many stages as fit, whole chunks of them
+  constexpr int C = kChunk<NSTG>, kMaxSmem = 227 * 1024;
+  TriParams Q = P;
+  Q.nstg = (int)std::min<size_t>(NSTG, (kMaxSmem - SM::head - 1024) / SM::stage(nvec)) / C * C;
+  const size_t smem = SM::head + Q.nstg * SM::stage(nvec);
+  return launch_clusters(k_tri<PK, NS, HD, G, H, NSTG>, CL, P.nunits, tri_threads<G, H>(), smem, Q, st);
 }
 
 }  // namespace tri
 
 // One entry per working precision, each compiled in its own translation unit.
-cudaError_t tri_launch_k64(int ns, bool hd, int G, bool helpers, const tri::TriParams& P, cudaStream_t st);
-cudaError_t tri_launch_k32(int ns, bool hd, const tri::TriParams& P, cudaStream_t st);
-cudaError_t tri_launch_kbf(int ns, bool hd, const tri::TriParams& P, cudaStream_t st);
+cudaError_t tri_launch_k64(int ns, bool hd, const TriShape& t, bool helpers, const tri::TriParams& P, cudaStream_t st);
+cudaError_t tri_launch_k32(int ns, bool hd, const TriShape& t, const tri::TriParams& P, cudaStream_t st);
+cudaError_t tri_launch_kbf(int ns, bool hd, const TriShape& t, const tri::TriParams& P, cudaStream_t st);
