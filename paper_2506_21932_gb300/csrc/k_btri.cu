@@ -580,7 +580,7 @@ cudaError_t go(int CL, const BtriParams& P, cudaStream_t st) {
   constexpr int G = kPlanes<V>;
   const int nvec = 1 + (P.h != nullptr) + (P.relax == 2);
   const size_t smem = ring_bytes<V>(G) + mail_bytes<V>() + (size_t)kStages * stage_size<V>(G, nvec);
-  return launch_clusters(k_btri<V>, CL, P.nunits, threads_of(G), smem, P, st);
+  return launch_clusters(k_btri<V>, CL, P.nunits, threads_of(G), 1, smem, P, st);
 }
 
 }  // namespace

@@ -152,28 +152,32 @@ template <> struct Mail<float> {
   static __device__ __forceinline__ float val(const word& w) { return __uint_as_float((unsigned)w); }
 };
 
-// Launch in clusters of CL CTAs, one per unit of CL tiles but no more than are
-// resident at once.
+// Launch in clusters of CL CTAs, one per unit of CL tiles but no more than the
+// SMs hold (per: CTAs per SM the registers are cut for).  Units are claimed by
+// ticket, so a cluster that finds no room waits and then finds no unit left:
+// the number need not be exact, and asking the runtime for it costs more than
+// the launch.
 template <typename Kern, typename Params>
-cudaError_t launch_clusters(Kern kern, int CL, int nunits, int threads, size_t smem, const Params& P,
+cudaError_t launch_clusters(Kern kern, int CL, int nunits, int threads, int per, size_t smem, const Params& P,
                             cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  constexpr size_t kSmSmem = 228 * 1024, kCtaSmem = 2048;  // what an SM has; a CTA's static part
+  if (per * (smem + kCtaSmem) > kSmSmem) per = 1;
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = CL;
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CL);
+  cfg.gridDim = dim3(CL * std::min(nunits, std::max(1, nsm * per / CL)));
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  int n = 0;
-  e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-  if (e != cudaSuccess) return e;
-  cfg.gridDim = dim3(CL * std::min(nunits, std::max(1, n)));
   e = cudaLaunchKernelEx(&cfg, kern, P);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }

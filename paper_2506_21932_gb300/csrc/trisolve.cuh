@@ -661,7 +661,8 @@ cudaError_t launch_tri_kernel(int CL, const TriParams& P, cudaStream_t st) {
   TriParams Q = P;
   Q.nstg = (int)std::min<size_t>(NSTG, (kMaxSmem - SM::head - 1024) / SM::stage(nvec)) / C * C;
   const size_t smem = SM::head + Q.nstg * SM::stage(nvec);
-  return launch_clusters(k_tri<PK, NS, HD, G, H, NSTG>, CL, P.nunits, tri_threads<G, H>(), smem, Q, st);
+  return launch_clusters(k_tri<PK, NS, HD, G, H, NSTG>, CL, P.nunits, tri_threads<G, H>(),
+                         tri_ctas<G, H>(), smem, Q, st);
 }
 
 }  // namespace tri
