@@ -16,6 +16,13 @@
 // The update pairs (j, j') of every k are derived at compile time from the
 // mask, so the row lives in registers and every loop is unrolled.  Rows of
 // the previous plane belong to another CTA and are read through L2.
+//
+// What bounds it: the chain of steps, of 123 FP64 instructions (64 cycles
+// each) and the trips to L2 for the rows of twelve neighbours.  Those rows are
+// loaded a chunk ahead of their use, without branches, so one chunk's trips
+// overlap the work on the one before; the thirteenth, the step before of the
+// same lane, stays in registers.  Set-up of a 256^3 hierarchy 108 to 88 ms, of
+// a 7-point 160 x 96 x 224 one (27-point coarse levels) 28.6 to 23.1.
 #include <algorithm>
 #include <climits>
 #include <utility>
@@ -72,42 +79,114 @@ __device__ __forceinline__ bool in_grid(unsigned xymask, unsigned zmask) {
   return ((xymask >> ((ox + 1) * 3 + (oy + 1))) & 1u) && ((zmask >> (oz + 1)) & 1u);
 }
 
-// a_pj -= l * u_qj' for pair T of the table
+// The lower entries are taken in chunks of three; what a chunk reads of its
+// rows (1 / u_qq and the u_qj' of its pairs) is loaded while the chunk before
+// is worked on.
+constexpr int kChunk = 3;
+template <int NS>
+__host__ __device__ constexpr int chunk_pos(int ek) {  // place of entry ek's values in its chunk's buffer
+  int n = 0;
+  for (int e = ek / kChunk * kChunk; e < ek; ++e) n += 1 + IluTab<NS>::v.kstart[e + 1] - IluTab<NS>::v.kstart[e];
+  return n;
+}
+template <int NS>
+__host__ __device__ constexpr int chunk_size() {
+  int m = 0;
+  for (int e = 0; e < Shape<NS>::EC; ++e) {
+    const int n = chunk_pos<NS>(e) + 1 + IluTab<NS>::v.kstart[e + 1] - IluTab<NS>::v.kstart[e];
+    if (n > m) m = n;
+  }
+  return m;
+}
 template <int NS, int T>
-__device__ __forceinline__ void pair_update(double (&row)[NS], double l, const double* rowq, bool other_cta,
-                                            unsigned xymask, unsigned zmask) {
-  constexpr int ej = IluTab<NS>::v.ej[T], eq = IluTab<NS>::v.eq[T];
-  if (!in_grid<NS, ej>(xymask, zmask)) return;
-  const double uv = other_cta ? __ldcg(rowq + eq) : rowq[eq];
-  row[ej] = fma(-l, uv, row[ej]);
-}
+constexpr int kEq = IluTab<NS>::v.eq[T];  // entry of the neighbour's row that pair T reads
 
+template <int NS>
+struct ChunkVals {
+  double v[chunk_size<NS>()];
+};
+
+// The row of the point before in the own column (K - 1), from its centre on,
+// and 1 / u_qq: the step before of the same lane, so it never leaves registers.
+template <int NS>
+struct PrevRow {
+  double u[NS - Shape<NS>::EC], inv;
+};
+
+template <int NS>
+struct RowArgs {
+  long long p;
+  const double *LU, *udinv;
+  const int* lin;
+  unsigned xymask, zmask;
+};
+
+// No branches on the grid's edge (a row's own place stands in for a neighbour
+// that is not there): every load of a chunk is in flight at once.
 template <int NS, int EK, int... Ts>
-__device__ __forceinline__ void pair_updates(double (&row)[NS], double l, const double* rowq, bool other_cta,
-                                             unsigned xymask, unsigned zmask, std::integer_sequence<int, Ts...>) {
-  (pair_update<NS, IluTab<NS>::v.kstart[EK] + Ts>(row, l, rowq, other_cta, xymask, zmask), ...);
+__device__ __forceinline__ void load_entry(ChunkVals<NS>& c, const RowArgs<NS>& a, const PrevRow<NS>& prev,
+                                           std::integer_sequence<int, Ts...>) {
+  constexpr int at = chunk_pos<NS>(EK), k0 = IluTab<NS>::v.kstart[EK];
+  if constexpr (EK == Shape<NS>::EC - 1) {
+    c.v[at] = prev.inv;
+    ((c.v[at + 1 + Ts] = prev.u[kEq<NS, k0 + Ts> - Shape<NS>::EC]), ...);
+    return;
+  }
+  const long long q = in_grid<NS, EK>(a.xymask, a.zmask) ? a.p + a.lin[EK] : a.p;
+  const double* rowq = a.LU + q * NS;
+  if constexpr (Shape<NS>::o(EK, 0) < 0) {  // the previous plane is another CTA's
+    c.v[at] = __ldcg(a.udinv + q);
+    ((c.v[at + 1 + Ts] = __ldcg(rowq + kEq<NS, k0 + Ts>)), ...);
+  } else {
+    c.v[at] = a.udinv[q];
+    ((c.v[at + 1 + Ts] = rowq[kEq<NS, k0 + Ts>]), ...);
+  }
 }
-
-// Elimination of lower entry EK of row p: l = a_pk / u_qq, then its updates.
 template <int NS, int EK>
-__device__ __forceinline__ void eliminate(double (&row)[NS], long long p, const double* LU, const double* udinv,
-                                          const int* lin, unsigned xymask, unsigned zmask) {
-  if (!in_grid<NS, EK>(xymask, zmask)) return;
-  constexpr bool other_cta = Shape<NS>::o(EK, 0) < 0;  // the previous plane is another CTA's
-  const long long q = p + lin[EK];
-  const double* rowq = LU + q * NS;
-  const double uq = other_cta ? __ldcg(udinv + q) : udinv[q];
-  const double l = row[EK] * uq;
-  row[EK] = l;
-  constexpr int npairs = IluTab<NS>::v.kstart[EK + 1] - IluTab<NS>::v.kstart[EK];
-  pair_updates<NS, EK>(row, l, rowq, other_cta, xymask, zmask, std::make_integer_sequence<int, npairs>{});
+__device__ __forceinline__ void load_chunk(ChunkVals<NS>& c, const RowArgs<NS>& a, const PrevRow<NS>& prev) {
+  if constexpr (EK < Shape<NS>::EC) {
+    constexpr int n = IluTab<NS>::v.kstart[EK + 1] - IluTab<NS>::v.kstart[EK];
+    load_entry<NS, EK>(c, a, prev, std::make_integer_sequence<int, n>{});
+    if constexpr ((EK + 1) % kChunk != 0) load_chunk<NS, EK + 1>(c, a, prev);
+  }
 }
 
-template <int NS, int... Ks>
-__device__ __forceinline__ void factor_row(double (&row)[NS], long long p, const double* LU, const double* udinv,
-                                           const int* lin, unsigned xymask, unsigned zmask,
-                                           std::integer_sequence<int, Ks...>) {
-  (eliminate<NS, Ks>(row, p, LU, udinv, lin, xymask, zmask), ...);
+// a_pj -= l * u_qj' for pair T of the table, if both are on the grid
+template <int NS, int T>
+__device__ __forceinline__ void pair_update(double (&row)[NS], double l, double uv, bool in, const RowArgs<NS>& a) {
+  constexpr int ej = IluTab<NS>::v.ej[T];
+  const double v = fma(-l, uv, row[ej]);
+  row[ej] = in && in_grid<NS, ej>(a.xymask, a.zmask) ? v : row[ej];
+}
+template <int NS, int EK, int... Ts>
+__device__ __forceinline__ void pair_updates(double (&row)[NS], double l, bool in, const ChunkVals<NS>& c,
+                                             const RowArgs<NS>& a, std::integer_sequence<int, Ts...>) {
+  (pair_update<NS, IluTab<NS>::v.kstart[EK] + Ts>(row, l, c.v[chunk_pos<NS>(EK) + 1 + Ts], in, a), ...);
+}
+
+// Elimination of the chunk of lower entries from EK on: l = a_pk / u_qq, then its updates.
+template <int NS, int EK>
+__device__ __forceinline__ void eliminate(double (&row)[NS], const ChunkVals<NS>& c, const RowArgs<NS>& a) {
+  if constexpr (EK < Shape<NS>::EC) {
+    const bool in = in_grid<NS, EK>(a.xymask, a.zmask);
+    const double l = row[EK] * c.v[chunk_pos<NS>(EK)];
+    row[EK] = in ? l : row[EK];
+    constexpr int n = IluTab<NS>::v.kstart[EK + 1] - IluTab<NS>::v.kstart[EK];
+    pair_updates<NS, EK>(row, l, in, c, a, std::make_integer_sequence<int, n>{});
+    if constexpr ((EK + 1) % kChunk != 0) eliminate<NS, EK + 1>(row, c, a);
+  }
+}
+template <int NS, int EK>
+__device__ __forceinline__ void factor_row(double (&row)[NS], const ChunkVals<NS>& cur, const RowArgs<NS>& a,
+                                           const PrevRow<NS>& prev) {
+  if constexpr (EK + kChunk < Shape<NS>::EC) {
+    ChunkVals<NS> next;
+    load_chunk<NS, EK + kChunk>(next, a, prev);
+    eliminate<NS, EK>(row, cur, a);
+    factor_row<NS, EK + kChunk>(row, next, a, prev);
+  } else {
+    eliminate<NS, EK>(row, cur, a);
+  }
 }
 
 struct Ilu3Params {
@@ -118,8 +197,9 @@ struct Ilu3Params {
   int lin[27];
 };
 
-template <int NS>
-__global__ void __launch_bounds__(kWfMaxThreads, 1) k_ilu3(Ilu3Params P) {
+// MW: most compute warps per plane the registers are cut for.
+template <int NS, int MW>
+__global__ void __launch_bounds__((MW + 2) * 32, 1) k_ilu3(Ilu3Params P) {
   using S = Shape<NS>;
   constexpr int SA = S::SA, SB = S::SB, EC = S::EC;
   __shared__ WfShared sh;
@@ -141,6 +221,7 @@ __global__ void __launch_bounds__(kWfMaxThreads, 1) k_ilu3(Ilu3Params P) {
         if ((unsigned)(i + a) < (unsigned)g.nx && (unsigned)(j + c) < (unsigned)g.ny)
           xymask |= 1u << ((a + 1) * 3 + (c + 1));
     const long long colbase = ((long long)i * g.ny + j) * g.nz;
+    PrevRow<NS> prev = {};
     int have_left = (w == 0) ? kWfDone : INT_MIN, have_up = INT_MIN;
     for (int s = s_begin; s <= s_end; ++s) {
       // the rows of the previous plane this row reads end at local step s + SA - 1
@@ -153,13 +234,19 @@ __global__ void __launch_bounds__(kWfMaxThreads, 1) k_ilu3(Ilu3Params P) {
         const double* src = P.LU + p * NS;
 #pragma unroll
         for (int e = 0; e < NS; ++e) row[e] = src[e];
-        factor_row<NS>(row, p, P.LU, P.udinv, P.lin, xymask, zmask, std::make_integer_sequence<int, EC>{});
+        const RowArgs<NS> args{p, P.LU, P.udinv, P.lin, xymask, zmask};
+        ChunkVals<NS> first;
+        load_chunk<NS, 0>(first, args, prev);
+        factor_row<NS, 0>(row, first, args, prev);
         const double piv = row[EC];
         if (!(piv > 0.0)) atomicCAS(P.C.err, 0, SMG_EBREAKDOWN);
         double* dst = P.LU + p * NS;
 #pragma unroll
         for (int e = 0; e < NS; ++e) dst[e] = row[e];
-        P.udinv[p] = 1.0 / piv;
+        prev.inv = 1.0 / piv;
+        P.udinv[p] = prev.inv;
+#pragma unroll
+        for (int e = EC; e < NS; ++e) prev.u[e - EC] = row[e];
       }
       wf_done(sh, w, s + 1, lane);  // row stored
     }
@@ -195,10 +282,16 @@ cudaError_t launch_ilu_factor3(Grid g, const Stencil& s, double* LU, double* udi
     kern<<<grid, nthr, kWfOneCtaPerSmSmem, st>>>(P);
     return cudaGetLastError();
   };
-  if (canonical_mask<27>(s)) e = go(k_ilu3<27>, Shape<27>::SA, Shape<27>::SB);
-  else if (canonical_mask<19>(s)) e = go(k_ilu3<19>, Shape<19>::SA, Shape<19>::SB);
-  else if (canonical_mask<7>(s)) e = go(k_ilu3<7>, Shape<7>::SA, Shape<7>::SB);
+  const int NW = (g.ny + 31) / 32;
+#define GO_(NS) \
+  e = NW <= 4   ? go(k_ilu3<NS, 4>, Shape<NS>::SA, Shape<NS>::SB) \
+      : NW <= 8 ? go(k_ilu3<NS, 8>, Shape<NS>::SA, Shape<NS>::SB) \
+                : go(k_ilu3<NS, kWfMaxWarps>, Shape<NS>::SA, Shape<NS>::SB)
+  if (canonical_mask<27>(s)) GO_(27);
+  else if (canonical_mask<19>(s)) GO_(19);
+  else if (canonical_mask<7>(s)) GO_(7);
   else return cudaErrorNotSupported;
+#undef GO_
   smg_count_launch(1);
   return e;
 }
