@@ -15,8 +15,10 @@
 //  (3) k_update, all SMs: A = A + N W (pivot rows: N W alone).
 // The rows end up as those of the inverse of P A; k_unpermute undoes P on the
 // columns.  Measured: a set-up with n = 2048 went from 76 to 29.5 ms, with
-// n = 768 from 36.5 to 28.6 ms.  What is left is the panels' chain: a search,
-// a cluster barrier and a step over the panel per column.
+// n = 768 from 36.5 to 28.6 ms; with candidates compared as integers and pushed
+// to the peers before the barrier, and one division a CTA, n = 2048 to 26.9.
+// What is left is the panels' chain, 4 us a column: a search, a cluster barrier,
+// a division and a step over the panel.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -40,22 +42,41 @@ struct Moves {
   int from[kNb], to[kNb];
 };
 
-// Larger magnitude first, the lower row among equals.
-__device__ __forceinline__ void better(double& v, int& r, double v2, int r2) {
+// Pivot candidates are compared as integers (the bits of |v| order like |v|; a
+// comparison of doubles takes the FP64 pipe 64 cycles a warp): larger first, the
+// lower row among equals.  NaN is no candidate.
+__device__ __forceinline__ long long pivot_key(double v) {
+  const long long k = __double_as_longlong(v) & 0x7fffffffffffffffLL;
+  return k > 0x7ff0000000000000LL ? -1 : k;
+}
+__device__ __forceinline__ void better(long long& v, int& r, long long v2, int r2) {
   if (v2 > v || (v2 == v && r2 < r)) {
     v = v2;
     r = r2;
+  }
+}
+template <int W>
+__device__ __forceinline__ void best_of(long long& v, int& r) {  // of W neighbouring lanes
+#pragma unroll
+  for (int o = W / 2; o > 0; o >>= 1) {
+    const long long v2 = __shfl_xor_sync(0xffffffffu, v, o);
+    const int r2 = __shfl_xor_sync(0xffffffffu, r, o);
+    better(v, r, v2, r2);
   }
 }
 
 __global__ void __launch_bounds__(kThreads) k_panel(int n, int k0, double* __restrict__ M, Moves* moves,
                                                     int* __restrict__ perm, int* err) {
   extern __shared__ double a[];  // [rows of this CTA][kNb + 1]
-  constexpr int LD = kNb + 1;
-  __shared__ double c_val[2], c_row[2][kNb];
-  __shared__ int c_idx[2];
-  __shared__ double w_val[kThreads / 32], prow[kNb], best_val;
-  __shared__ int w_idx[kThreads / 32], best_idx;
+  constexpr int LD = kNb + 1, kWarps = kThreads / 32;
+  // every CTA's candidate of a column: its key, row and values, written by its owner
+  __shared__ long long c_key[2][kCluster];
+  __shared__ int c_idx[2][kCluster];
+  __shared__ double c_row[2][kCluster][kNb];
+  __shared__ long long w_key[kWarps];
+  __shared__ int w_idx[kWarps];
+  __shared__ double prow[kNb], pinv;
+  __shared__ int pivot;
   __shared__ Moves mv;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
@@ -67,71 +88,58 @@ __global__ void __launch_bounds__(kThreads) k_panel(int n, int k0, double* __res
     a[r * LD + c] = c < nb ? M[(long long)(r0 + r) * n + k0 + c] : 0.0;
   }
   for (int r = tid; r < rows; r += kThreads) used[r] = 0;
-  __syncthreads();
+  cl.sync();  // every CTA runs before its candidates are written to
   bool singular = false;
   for (int t = 0; t < nb; ++t) {
     const int buf = t & 1;
-    double bv = -1.0;
+    long long bv = -1;
     int bi = n;
     for (int r = tid; r < rows; r += kThreads)
-      if (r0 + r >= k0 && !used[r]) better(bv, bi, fabs(a[r * LD + t]), r0 + r);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double v2 = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int r2 = __shfl_xor_sync(0xffffffffu, bi, o);
-      better(bv, bi, v2, r2);
-    }
+      if (r0 + r >= k0 && !used[r]) better(bv, bi, pivot_key(a[r * LD + t]), r0 + r);
+    best_of<32>(bv, bi);
     if (lane == 0) {
-      w_val[wp] = bv;
+      w_key[wp] = bv;
       w_idx[wp] = bi;
     }
     __syncthreads();
     if (wp == 0) {
-      bv = lane < kThreads / 32 ? w_val[lane] : -1.0;
-      bi = lane < kThreads / 32 ? w_idx[lane] : n;
+      bv = w_key[lane % kWarps];
+      bi = w_idx[lane % kWarps];
+      best_of<kWarps>(bv, bi);  // the same in every lane
+      // to every CTA of the cluster, two at a time
 #pragma unroll
-      for (int o = 4; o > 0; o >>= 1) {
-        const double v2 = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int r2 = __shfl_xor_sync(0xffffffffu, bi, o);
-        better(bv, bi, v2, r2);
+      for (int h = 0; h < kCluster; h += 2) {
+        const int to = h + lane / kNb, c = lane % kNb;
+        cl.map_shared_rank(&c_row[buf][rank][0], to)[c] = bi < n ? a[(bi - r0) * LD + c] : 0.0;
       }
-      bv = __shfl_sync(0xffffffffu, bv, 0);
-      bi = __shfl_sync(0xffffffffu, bi, 0);
-      if (lane == 0) {
-        c_val[buf] = bv;
-        c_idx[buf] = bi;
+      if (lane < kCluster) {
+        *cl.map_shared_rank(&c_key[buf][rank], lane) = bv;
+        *cl.map_shared_rank(&c_idx[buf][rank], lane) = bi;
       }
-      if (lane < kNb && bi < n) c_row[buf][lane] = a[(bi - r0) * LD + lane];
     }
     cl.sync();
     if (wp == 0) {
-      double gv = lane < kCluster ? *cl.map_shared_rank(&c_val[buf], lane) : -1.0;
-      int gi = lane < kCluster ? *cl.map_shared_rank(&c_idx[buf], lane) : n;
-#pragma unroll
-      for (int o = kCluster / 2; o > 0; o >>= 1) {
-        const double v2 = __shfl_xor_sync(0xffffffffu, gv, o);
-        const int r2 = __shfl_xor_sync(0xffffffffu, gi, o);
-        better(gv, gi, v2, r2);
-      }
-      gv = __shfl_sync(0xffffffffu, gv, 0);
-      gi = __shfl_sync(0xffffffffu, gi, 0);
-      if (gv > 0.0 && lane < kNb) {
-        const double* pr = cl.map_shared_rank(&c_row[buf][0], gi / per);
-        prow[lane] = pr[lane];
+      bv = c_key[buf][lane % kCluster];
+      bi = c_idx[buf][lane % kCluster];
+      best_of<kCluster>(bv, bi);
+      if (bv > 0) {
+        const double* pr = c_row[buf][bi / per];
+        if (lane < kNb) prow[lane] = pr[lane];
+        const double inv = 1.0 / pr[t];
+        if (lane == 0) pinv = inv;
       }
       if (lane == 0) {
-        best_val = gv;
-        best_idx = gi;
-        mv.piv[t] = gi;
+        pivot = bv > 0 ? bi : -1;
+        mv.piv[t] = bi;
       }
     }
     __syncthreads();
-    if (!(best_val > 0.0)) {  // the same in every CTA
+    const int p = pivot;
+    if (p < 0) {  // the same in every CTA
       singular = true;
       break;
     }
-    const int p = best_idx;
-    const double inv = 1.0 / prow[t];
+    const double inv = pinv;
     for (int r = tid; r < rows; r += kThreads) {
       double* row = a + r * LD;
       if (r0 + r == p) {
@@ -146,7 +154,7 @@ __global__ void __launch_bounds__(kThreads) k_panel(int n, int k0, double* __res
     }
     __syncthreads();
   }
-  cl.sync();  // no CTA leaves while another may read its candidates
+  cl.sync();
   if (singular) {
     if (rank == 0 && tid == 0) atomicCAS(err, 0, SMG_EBREAKDOWN);
     return;
