@@ -119,25 +119,54 @@ __global__ void __launch_bounds__(256) k_shear_copy(Line ln, int to_stream, cons
   }
 }
 
-// Stream out = b - A x, x and b in natural order.
+// Stream out = b - A x, x and b in natural order.  A warp takes 32 points of a
+// column.  Its rows of A, read lane by lane, are evicted from L1 before their
+// last entry is used when too many warps do so, and too few registers keep too
+// few loads in flight: residual at 384^3 in ms with 6, 8, 5, 4, 3 blocks per SM
+//   FP64 3.98 5.69 3.02 2.94 3.00 (2.48 of multiply-adds).
+// FP32 rows go through shared memory in whole lines (256^3: 0.72 to 0.52 ms; FP64
+// rows that way: 6.2 ms at 384^3); BF16 208 x 144 x 176: 0.139 with 8 blocks,
+// 0.125 with 5.
 template <int PK, int NS>
-__global__ void __launch_bounds__(256) k_shear_residual(Line ln, Stencil s, const typename Prec<PK>::val* __restrict__ A,
-                                                        const float* __restrict__ scale,
-                                                        const typename Prec<PK>::vec* __restrict__ x,
-                                                        const typename Prec<PK>::vec* __restrict__ b,
-                                                        typename Prec<PK>::vec* __restrict__ out) {
+struct ResidualCfg {
+  using Val = typename Prec<PK>::val;
+  static constexpr bool STAGE = PK == K32;
+  static constexpr int blocks = PK == K64 ? 4 : PK == K32 ? 8 : 5;  // per SM
+  static constexpr size_t rows = STAGE ? sizeof(Val) * 8 * 32 * NS : 0;
+};
+template <int PK, int NS>
+__global__ void __launch_bounds__(256, ResidualCfg<PK, NS>::blocks)
+    k_shear_residual(Line ln, Stencil s, const typename Prec<PK>::val* __restrict__ A, const float* __restrict__ scale,
+                     const typename Prec<PK>::vec* __restrict__ x, const typename Prec<PK>::vec* __restrict__ b,
+                     typename Prec<PK>::vec* __restrict__ out) {
   using V = typename Prec<PK>::vec;
+  using Val = typename Prec<PK>::val;
   __shared__ V t[32][33];
+  extern __shared__ __align__(16) unsigned char rows_raw[];
   ln.w = blockIdx.x;
   ln.pr = blockIdx.z;
   const Grid g = ln.g;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k0 = blockIdx.y * 32;
   long long p;
   int i, j, k, kk;
+  Val* mine = reinterpret_cast<Val*>(rows_raw) + wp * (32 * NS);
 #pragma unroll 1
   for (int c = 0; c < 4; ++c) {
-    if (!ln.at(wp + 8 * c, k0 + lane, p, i, j, k)) continue;
-    const typename Prec<PK>::val* a = A + p * NS;
+    const bool ok = ln.at(wp + 8 * c, k0 + lane, p, i, j, k);
+    if (!__any_sync(0xffffffffu, ok)) continue;
+    const Val* a = A + p * NS;
+    if constexpr (ResidualCfg<PK, NS>::STAGE) {
+      // forward stream: lanes are consecutive k, lane 0 of a column is on the grid
+      const int n = min(32, g.nz - k0) * NS;
+      const Val* run = A + __shfl_sync(0xffffffffu, p, 0) * NS;
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < NS; ++q)
+        if (q * 32 + lane < n) mine[q * 32 + lane] = run[q * 32 + lane];
+      __syncwarp();
+      a = mine + lane * NS;
+    }
+    if (!ok) continue;
     V acc = V(0);
 #pragma unroll
     for (int e = 0; e < NS; ++e) {
@@ -286,9 +315,16 @@ cudaError_t launch_shear_residual(const LevelView& L, const TriShape& t, const v
   const int ns = L.s.ns, pk = L.pk;
   const Line ln = line_of(L.g, t, +1);
   const dim3 nb = tiles(t, ln.g.nz, 32, ln.g.ny);
-#define F_(PK, NS)                                                                            \
-  k_shear_residual<PK, NS><<<nb, 256, 0, st>>>(ln, L.s, (const Prec<PK>::val*)L.A, L.scale,   \
-                                               (const Prec<PK>::vec*)x, (const Prec<PK>::vec*)b, (Prec<PK>::vec*)out)
+#define F_(PK, NS)                                                                                        \
+  do {                                                                                                    \
+    constexpr size_t sm = ResidualCfg<PK, NS>::rows;                                                     \
+    const cudaError_t e =                                                                                 \
+        cudaFuncSetAttribute(k_shear_residual<PK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
+    if (e != cudaSuccess) return e;                                                                       \
+    k_shear_residual<PK, NS><<<nb, 256, sm, st>>>(ln, L.s, (const Prec<PK>::val*)L.A, L.scale,            \
+                                                  (const Prec<PK>::vec*)x, (const Prec<PK>::vec*)b,       \
+                                                  (Prec<PK>::vec*)out);                                   \
+  } while (0)
   BY_PK(F_);
 #undef F_
   smg_count_launch(1);
