@@ -28,12 +28,13 @@ struct Line {
   __device__ __forceinline__ bool at(int il, int K, long long& p, int& i, int& j, int& k) const {
     return point(il, K + SL * il, p, i, j, k);
   }
-  // Row q (0 <= q < 32 + 31 SL) of the tile of K = k0 .. k0 + 31: whether lane
-  // has a point there, and its K offset kk and slot.
+  // Row q (0 <= q < KC + 31 SL) of the tile of K = k0 .. k0 + KC - 1: whether
+  // lane has a point there, and its K offset kk and slot.
+  template <int KC = 32>
   __device__ __forceinline__ bool slot(int lane, int k0, int q, int& kk, long long& s) const {
     kk = q - SL * lane;
     const int J = pr - lane;
-    if (kk < 0 || kk > 31 || k0 + kk >= g.nz || 32 * w + lane >= g.nx || J < 0 || J >= g.ny) return false;
+    if (kk < 0 || kk >= KC || k0 + kk >= g.nz || 32 * w + lane >= g.nx || J < 0 || J >= g.ny) return false;
     s = row(k0 + q) * 32 + lane;
     return true;
   }
@@ -90,32 +91,42 @@ __global__ void __launch_bounds__(256) k_records(Line ln, int whole_scale, const
   if constexpr (HD) reinterpret_cast<Vec*>(rec + R::D_OFF)[lane] = (Vec)dinv[p];
 }
 
-template <typename T>
+// Tiles of KC points of 32 columns.  A row of a tile holds 32 lanes' points only
+// where all their columns have one there, KC - 31 SL of KC + 31 SL rows, so a
+// long tile wastes less: 27-point FP64 pack / unpack / add in ms with KC = 32, 64
+// and 128 0.39 / 0.44 / 0.51, 0.31 / 0.33 / 0.40 and 0.28 / 0.31 / 0.43 at 384^3,
+// 0.021 / 0.025 / 0.027, 0.019 / 0.020 / 0.025 and 0.021 / 0.023 / 0.031 at 128^3.
+template <typename T, int KC>
 __global__ void __launch_bounds__(256) k_shear_copy(Line ln, int to_stream, const T* __restrict__ src,
                                                     T* __restrict__ dst, int add) {
-  __shared__ T t[32][33];
+  __shared__ T t[KC][33];
   ln.w = blockIdx.x;
   ln.pr = blockIdx.z;
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k0 = blockIdx.y * 32, rows = 32 + 31 * ln.SL;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k0 = blockIdx.y * KC, rows = KC + 31 * ln.SL;
   long long p;
   int i, j, k, kk;
   if (to_stream) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-      if (ln.at(wp + 8 * c, k0 + lane, p, i, j, k)) t[lane][wp + 8 * c] = src[p];
+    for (int c = 0; c < KC / 8; ++c) {
+      const int il = wp + 8 * (c & 3), kl = (c >> 2) * 32 + lane;
+      if (ln.at(il, k0 + kl, p, i, j, k)) t[kl][il] = src[p];
+    }
     __syncthreads();
     for (int q = wp; q < rows; q += 8)
-      if (ln.slot(lane, k0, q, kk, p)) dst[p] = t[kk][lane];
+      if (ln.template slot<KC>(lane, k0, q, kk, p)) dst[p] = t[kk][lane];
   } else {
+#pragma unroll 4
     for (int q = wp; q < rows; q += 8)
-      if (ln.slot(lane, k0, q, kk, p)) t[kk][lane] = src[p];
+      if (ln.template slot<KC>(lane, k0, q, kk, p)) t[kk][lane] = src[p];
     __syncthreads();
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-      if (ln.at(wp + 8 * c, k0 + lane, p, i, j, k)) {
-        const T v = t[lane][wp + 8 * c];
+    for (int c = 0; c < KC / 8; ++c) {
+      const int il = wp + 8 * (c & 3), kl = (c >> 2) * 32 + lane;
+      if (ln.at(il, k0 + kl, p, i, j, k)) {
+        const T v = t[kl][il];
         dst[p] = add ? dst[p] + v : v;
       }
+    }
   }
 }
 
@@ -303,9 +314,17 @@ cudaError_t launch_tri_records_gs(const Grid& g, const TriShape& t, int pk, cons
 cudaError_t launch_shear_copy(const Grid& g, const TriShape& t, int dir, int vb, bool to_stream, const void* src,
                               void* dst, bool add, cudaStream_t st) {
   const Line ln = line_of(g, t, dir);
-  const dim3 nb = tiles(t, ln.g.nz, 32, ln.g.ny);
-  if (vb == 8) k_shear_copy<double><<<nb, 256, 0, st>>>(ln, to_stream, (const double*)src, (double*)dst, add);
-  else k_shear_copy<float><<<nb, 256, 0, st>>>(ln, to_stream, (const float*)src, (float*)dst, add);
+  constexpr int KCT = 64;
+  const bool tall = ln.SL > 0 && g.nz > 32;  // SL = 0: every row is full
+  const dim3 nb = tiles(t, ln.g.nz, tall ? KCT : 32, ln.g.ny);
+#define C_(T)                                                                                        \
+  do {                                                                                               \
+    if (tall) k_shear_copy<T, KCT><<<nb, 256, 0, st>>>(ln, to_stream, (const T*)src, (T*)dst, add);  \
+    else k_shear_copy<T, 32><<<nb, 256, 0, st>>>(ln, to_stream, (const T*)src, (T*)dst, add);        \
+  } while (0)
+  if (vb == 8) C_(double);
+  else C_(float);
+#undef C_
   smg_count_launch(1);
   return cudaGetLastError();
 }
