@@ -101,8 +101,9 @@ FP64_PROBE = os.path.join(ROOT, "profiles", "fp64_fma_peak_gb300.txt")
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per point of the
 # dominant kernel, from one ncu capture of the current kernel on the same
 # problem family at a smaller size (the traffic grows with the points); keyed
-# by (kernel, smoother, stencil points, precision).  Absent where no capture
-# of the current kernel exists.
+# by (kernel, smoother, stencil points, precision).  Those below are of the
+# plane-per-CTA sweeps, kept to compare with; no entry where no capture of the
+# kernel that runs exists.
 TRAFFIC_PER_POINT = {
     # k_sweep3 ILU lower solve, FP64, 27 points: 268.97 MB for 128^3
     ("k_sweep3", 1, 27, 0): (268.970e6 / 128 ** 3, "profiles/k_sweep3_ilu_lower_aniso27_128cubed.md"),
@@ -419,15 +420,16 @@ def run_ours(args, w, rank, world):
     if w["smoother"] == 2:
         kname = "k_lsweep (line Gauss-Seidel, zero-guess forward, level 0)"
         nz = int(w["dims"][2])
-        m = max(2, -(-nz // 128))
-        fac_pt = 8.0 * ((m - 1) * 5 + 17) * 128 / nz
+        # line factors: 32 chunks of m rows for each of lw solving warps
+        lw, m = (1 if nz <= 64 else 2 if nz <= 128 else 4), (2 if nz <= 256 else 4 if nz <= 512 else 8)
+        fac_pt = 8.0 * ((m - 1) * 5 + 3 + 2 * (4 + lw.bit_length())) * 32 * lw / nz
         flops_pt, bytes_pt = 2 * (nlow - 1) + 10, nlow * cbytes + fac_pt + 2 * vbytes
     elif w["smoother"] == 1:
-        kfile = "k_sweep3h" if lvl0_warps == 2 else "k_sweep3"
+        kfile = "k_tri" if lvl0_warps else "k_sweep2"
         kname = "%s (ILU(0) lower solve, level 0)" % kfile
         flops_pt, bytes_pt = 2 * nlow + 1, nlow * cbytes + 2 * vbytes + sbytes
     else:
-        kfile = {2: "k_sweep3h", 1: "k_sweep3"}.get(lvl0_warps, "k_sweep2") if B == 1 else "k_bsweep3"
+        kfile = ("k_tri" if lvl0_warps else "k_sweep2") if B == 1 else "k_btri"
         kname = "%s (Gauss-Seidel zero-guess forward, level 0)" % kfile
         flops_pt = (2 * nlow + 2) * B * B
         bytes_pt = nlow * cbytes * B * B + vbytes * B * B + 2 * vbytes * B + sbytes
@@ -577,7 +579,7 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true", help="skip the host-buffer pass (profiling runs)")
     ap.add_argument("--sweep-warps", type=int, default=0, choices=[0, 1, 2],
-                    help="warps per strip of the wavefront sweeps (0: the library's choice)")
+                    help="1: the wavefront sweeps without helper warps (0: the library's choice)")
     args = ap.parse_args()
     w = WORKLOADS[args.workload]
     rank = int(os.environ.get("RANK", 0))

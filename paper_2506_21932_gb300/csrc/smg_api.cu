@@ -1237,7 +1237,7 @@ extern "C" int smg_level_copy(smg_t h, int l, int which, void* dst, size_t bytes
 }
 
 // Whether a level operation runs the sheared wavefront: on FP64 levels only
-// where smg_sweep_noalloc's natural-order kernel (sweep3.cuh) takes the same
+// where smg_sweep_noalloc's natural-order kernel (k_sweep3.cu) takes the same
 // sweep and forms the same sums, so the two entry points agree to the bit.
 static bool level_op_sheared(smg_ctx* h, const Level& L, int kind) {
   return sheared(L) && (h->pk != K64 || L.B == 3 || sweep3_supported(view(h, L, true), kind));
