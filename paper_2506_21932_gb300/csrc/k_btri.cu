@@ -55,8 +55,8 @@ struct BtriParams {
 
 struct BtriShared {
   unsigned long long full[kStages];
-  int hready[2];  // plane p0 - 1, the lane left of the strip
-  int taken;      // the next tile has taken every time < taken of the last plane
+  int hready[2];      // plane p0 - 1, the lane left of the strip
+  PeerCounter taken;  // the next tile has taken every time < taken of the last plane
   int rready, done, abort, tile;
 };
 
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       sh.rready = T0;
       sh.done = T0 - 1;
       sh.abort = 0;
-      sh.taken = T0;
+      sh.taken.v = T0;
     }
     cluster_sync();
     if (dg >= ntile) continue;  // a unit may end early
@@ -200,14 +200,14 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       }
     } else if (warp == NC) {
       // ---- sync warp (as in trisolve.cuh)
-      const int* word = lane < 2 ? &sh.hready[lane] : lane == 2 ? &sh.rready : &sh.taken;
+      const int* word = lane < 2 ? &sh.hready[lane] : lane == 2 ? &sh.rready : &sh.taken.v;
       const int ahead = lane < 2 ? 0 : lane == 2 ? 2 : above && lane == 3 ? 1 - kMail : -kDone;
       const int most = lane == 2 ? Te + 1 : INT_MAX;
       bool drain = false;
       for (int T = T0 - 1; T <= Te; ++T) {
         const int need = min(T + ahead, most);
         unsigned iter = 0;
-        while (!drain && !__all_sync(0xffffffffu, ld_acq_cta(word) >= need)) {
+        while (!drain && !__all_sync(0xffffffffu, ld_acq_cluster(word) >= need)) {
           if ((++iter & 31u) != 0) continue;
           if ((iter & 1023u) == 0 && lane == 0 && ld_relaxed(P.err) != 0) st_relaxed_cta(&sh.abort, 1);
           drain = __any_sync(0xffffffffu, ld_acq_cta(&sh.abort) != 0);

@@ -81,10 +81,16 @@ __device__ __forceinline__ int ld_peer(unsigned a) {
   asm volatile("ld.relaxed.cluster.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
   return v;
 }
-// A word of this CTA's shared memory that a peer writes.
-__device__ __forceinline__ int ld_own(const int* p) {
+// A counter in this CTA's shared memory that a CTA of the cluster writes while
+// this one runs: a type of its own, so that it is not read at CTA scope (such a
+// load does not pair with a store from outside the CTA).
+struct PeerCounter {
   int v;
-  asm volatile("ld.relaxed.cluster.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+};
+// A load at cluster scope pairs with the stores of either kind of counter.
+__device__ __forceinline__ int ld_acq_cluster(const int* p) {
+  int v;
+  asm volatile("ld.acquire.cluster.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
   return v;
 }
 
