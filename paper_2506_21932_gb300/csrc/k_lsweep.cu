@@ -495,8 +495,21 @@ __global__ void __launch_bounds__((NWS + kHelpers + 2 + (NWS < 4 ? 2 - NWS : 0))
           bv[q] = k < nz ? P.b[col * nz + k] : 0.0;
         }
         const int need = I == 0 || P.T.ne == 0 ? 0 : min(J + 1 + P.T.dep, g.ny);
+        // Nothing else bounds a copy in flight (plane 0 has no loader), so once
+        // the rest is there a copy that is due counts against the budget.
+        unsigned long long t_wait = 0;
         const bool ok = wait_for(sh, [&] {
-          return ld_acq_cta(&sh.hready) >= need && ld_acq_cta(&sh.done) >= J - 1 && landed(J);
+          if (ld_acq_cta(&sh.hready) < need || ld_acq_cta(&sh.done) < J - 1) return false;
+          if (landed(J)) return true;
+          if (ld_acq_cta(&sh.done) + (int)stages > J) {
+            const unsigned long long now = globaltimer_ns();
+            if (t_wait == 0) t_wait = now;
+            else if (now - t_wait > P.budget_ns) {
+              atomicCAS(P.err, 0, DEV_ERR_TIMEOUT);
+              st_rel_cta(&sh.abort, 1);
+            }
+          }
+          return false;
         });
         if (!ok) break;
         const double* rec = stage(J);
