@@ -41,7 +41,7 @@ __host__ __device__ constexpr int entries_of(int G) { return 32 + G - 1; }
 
 struct BtriParams {
   Grid g;
-  int nunits, ngrp, F;
+  int nunits, ngrp, rows;
   const int* tiles;
   int flip, relax;
   unsigned long long budget_ns;
@@ -92,18 +92,9 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
   V* ev = (V*)P.emit;
   typename ML::word* mail = (typename ML::word*)P.mail;
   const unsigned tag = (unsigned)P.ws->epoch + 1u;
-  // slot of unknown 0 of point (I, p, time T) in the result's stream: column(I, p) + dstep * T
-  const int dstep = P.flip ? -G * 96 : G * 96;
-  auto column = [&](int I, int p) -> long long {
-    int c = I, q = p, k0 = -p;  // K = T + k0
-    if (P.flip) {
-      c = g.nx - 1 - I;
-      q = g.nx + g.ny - 2 - p;
-      k0 = g.nz - 1 - k0;
-    }
-    const int cw = c >> 5, cl = c & 31, pr = q - 32 * cw, cd = pr / G, cg = pr % G;
-    return (((long long)(cw * P.ngrp + cd) * P.F + cg + k0) * G + cg) * 96 + cl;
-  };
+  // first stored step of group d of strip w, and the stored step of time T
+  auto group = [&](int w, int d) { return (long long)(w * P.ngrp + d % P.ngrp) * P.rows; };
+  auto fold = [&](int T) { return T < 0 ? P.rows - 1 : T % P.rows; };  // T >= -1
   if (threadIdx.x == 0) {
     for (int t = 0; t < kStages; ++t) mbar_init(&sh.full[t], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -149,13 +140,26 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       auto vec_of = [&](int T, int which) {
         return reinterpret_cast<const V*>(stage(T)) + G * 32 * kTerms + which + pl * 96 + q * 32 + lane;
       };
-      long long at = colok ? column(I, p) + (long long)dstep * (T0 - 1) + 32 * q : 0;
+      // The lane's results: column (rc, rp) of the result's stream, whose time is T
+      // or (mirrored) Tm - T; the stored steps run out at time tw (mailbox: mw).
+      int rc = I, rp = p, row = fold(T0 - 1), tw = T0 - 1 + P.rows - row;
+      const int dstep = P.flip ? -G * 96 : G * 96, mrow = row;
+      int mw = tw;
+      if (P.flip) {
+        rc = g.nx - 1 - I;
+        rp = g.nx + g.ny - 2 - p;
+        row = fold(g.nx + g.ny - 2 + g.nz - T0);
+        tw = T0 + row;
+      }
+      const int cw = rc >> 5, cp = rp - 32 * cw;
+      const long long at = colok ? ((group(cw, cp / G) + row) * G + cp % G) * 96 + (rc & 31) + 32 * q : 0;
+      V* up = u + at;
+      V* ep = ev + at;
       // every lane of the last plane, lane 31 of the others; inside the cluster
       // the next tile's own mailbox
       const bool near = above && pl == G - 1, post = (pl == G - 1 && !above) || lane == 31;
       const unsigned peer = near ? peer_addr(own_mail + q * 32 + lane, rank + 1) : 0u;
-      typename ML::word* mb = mail + (((long long)(w * P.ngrp + dg) * P.F - T0) * kEntries +
-                                      (pl == G - 1 ? lane : 32 + pl)) * 3 + q;
+      typename ML::word* mb = mail + ((group(w, dg) + mrow) * kEntries + (pl == G - 1 ? lane : 32 + pl)) * 3 + q;
       const V wv = (V)P.w;
       // operands in the ring at time T - 1: (I-1, P-1), (I, P-1), (I, P), three unknowns each
       constexpr int CS = (G + 1) * kRing * kLanes;
@@ -170,7 +174,7 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       };
       const int Tb = T0 - 1;
       fetch(Tb);
-      for (int T = Tb; T <= Te; ++T) {
+      auto step = [&](int T) {
         asm volatile("bar.sync 1, %0;" ::"n"((NC + 1) * 32) : "memory");
         const int K = T - p;
         const bool ok = colok && K >= 0 && K < g.nz;
@@ -191,12 +195,26 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
         if (ok) {
           if (near)
             ML::put_peer(peer + (T & (kMail - 1)) * (96 * (unsigned)sizeof(typename ML::word)), r, (unsigned)T + 1u);
-          if (post) ML::put(mb + (long long)T * (3 * kEntries), r, tag);
-          u[at] = r;
-          if (ev) ev[at] = P.h ? a + *vec_of(T, hoff) : a;
+          if (post) ML::put(mb, r, tag);
+          *up = r;
+          if (ev) *ep = P.h ? a + *vec_of(T, hoff) : a;
         }
-        at += dstep;
+        up += dstep;
+        ep += dstep;
+        mb += 3 * kEntries;
         fetch(T + 1);
+      };
+      for (int T = Tb; T <= Te;) {
+        for (const int end = min(min(tw, mw), Te + 1); T < end; ++T) step(T);
+        if (T == tw) {
+          up -= (long long)P.rows * dstep;
+          ep -= (long long)P.rows * dstep;
+          tw += P.rows;
+        }
+        if (T == mw) {
+          mb -= (long long)P.rows * (3 * kEntries);
+          mw += P.rows;
+        }
       }
     } else if (warp == NC) {
       // ---- sync warp (as in trisolve.cuh)
@@ -227,12 +245,11 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       const int cd = !c ? dg - 1 : lane < 1 ? dg + SG - 1 : dg + SG;
       const int cg = !c || lane < 1 ? G - 1 : lane - 1;
       const int e = cg == G - 1 ? (c ? 31 : lane) : 32 + cg;
-      const typename ML::word* src =
-          okc ? mail + (((long long)(cw * P.ngrp + cd) * P.F - (32 * cw + G * cd)) * kEntries + e) * 3 : mail;
+      const typename ML::word* src = okc ? mail + (group(cw, cd) * kEntries + e) * 3 : mail;
       V* dst = ring + (c ? min(lane, G) : 0) * (kRing * kLanes) + (c ? 0 : lane + 1);
       constexpr int CS = (G + 1) * kRing * kLanes;
       const int t_lo = okc ? pc : INT_MAX, t_hi = okc ? pc + g.nz : INT_MIN;
-      int tau = T0 - 1;
+      int tau = T0 - 1, row = fold(tau);  // row: its stored step
       unsigned long long t_wait = 0;
       unsigned iter = 0;
       int ask = 1;
@@ -280,7 +297,8 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       }
       while (!near && tau < Te) {
         // lane 0's view for all: the votes below need every lane
-        const int n = __shfl_sync(0xffffffffu, min(min(ld_acq_cta(&sh.done) + kRing - 1, Te) - tau, ask), 0);
+        const int n = min(P.rows - row,
+                          __shfl_sync(0xffffffffu, min(min(ld_acq_cta(&sh.done) + kRing - 1, Te) - tau, ask), 0));
         int got = 0;
         if (n > 0) {
           typename ML::word val[kBatch][3];
@@ -290,7 +308,7 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
             for (int r = 0; r < 3; ++r) {
               val[m][r] = ML::value(V(0), tag);
               if (m < n && tau + m >= t_lo && tau + m < t_hi)
-                val[m][r] = ML::get(src + (long long)(tau + m) * (3 * kEntries) + r);
+                val[m][r] = ML::get(src + (long long)(row + m) * (3 * kEntries) + r);
             }
 #pragma unroll
           for (int m = 0; m < kBatch; ++m)
@@ -304,6 +322,7 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
         }
         if (got > 0) {
           tau += got;
+          row = row + got == P.rows ? 0 : row + got;
           __syncwarp();
           if (lane == 0) st_rel_cta(&sh.hready[c], tau);
           t_wait = 0;
@@ -339,13 +358,13 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
       // ---- record warp, one lane
       if (lane == 0) {
         const int nfill = Te - T0 + 1;
-        const long long step0 = (long long)(w * P.ngrp + dg) * P.F;
+        const long long step0 = group(w, dg);
         constexpr int RL = G * 32 * kTerms, VL = G * 96;
         const V* rec = (const V*)P.rec + step0 * RL;
         const V* bv = (const V*)P.b + step0 * VL;
         const V* hv = (const V*)P.h + step0 * VL;
         const V* ov = (const V*)P.old + step0 * VL;
-        int done = T0 - 1, issued = 0;
+        int done = T0 - 1, issued = 0, row = fold(T0);
         for (int f = 0; f < nfill; ++f) {
           const int T = T0 + f;
           bool stop = false;
@@ -362,10 +381,11 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
           unsigned long long* bar = &sh.full[(base + f) % kStages];
           V* st = reinterpret_cast<V*>(stages + ((base + f) % kStages) * stage_bytes);
           mbar_expect_tx(bar, stage_bytes);
-          bulk_copy_g2s(st, rec + (long long)f * RL, RL * sizeof(V), bar);
-          bulk_copy_g2s(st + RL, bv + (long long)f * VL, VL * sizeof(V), bar);
-          if (P.h) bulk_copy_g2s(st + RL + hoff, hv + (long long)f * VL, VL * sizeof(V), bar);
-          if (P.relax == 2) bulk_copy_g2s(st + RL + ooff, ov + (long long)f * VL, VL * sizeof(V), bar);
+          bulk_copy_g2s(st, rec + (long long)row * RL, RL * sizeof(V), bar);
+          bulk_copy_g2s(st + RL, bv + (long long)row * VL, VL * sizeof(V), bar);
+          if (P.h) bulk_copy_g2s(st + RL + hoff, hv + (long long)row * VL, VL * sizeof(V), bar);
+          if (P.relax == 2) bulk_copy_g2s(st + RL + ooff, ov + (long long)row * VL, VL * sizeof(V), bar);
+          row = row + 1 == P.rows ? 0 : row + 1;
           issued = f + 1;
         }
         // every copy has landed before the tile is left
@@ -424,7 +444,15 @@ __global__ void __launch_bounds__(threads_of(kPlanes<V>), 1) k_btri(BtriParams P
 // Point of lane il and row r (r = K) of plane pr of strip w, direction dir.
 struct BLine {
   Grid g;
-  int G, F, groups, dir, w, pr;
+  int G, groups, rows, dir, w, pr;
+  int t0;          // time of K = 0, folded
+  long long base;  // first stream row of the plane
+  __device__ __forceinline__ void enter(int strip, int plane) {
+    w = strip;
+    pr = plane;
+    t0 = (32 * w + pr) % rows;
+    base = (long long)(w * groups + pr / G % groups) * rows * G + pr % G;
+  }
   __device__ __forceinline__ bool point(int il, int K, long long& p) const {
     const int I = 32 * w + il, J = pr - il;
     if (I >= g.nx || J < 0 || J >= g.ny || K >= g.nz) return false;
@@ -433,8 +461,8 @@ struct BLine {
     return true;
   }
   __device__ __forceinline__ long long row(int K) const {
-    const int d = pr / G, gg = pr % G;
-    return ((long long)(w * groups + d) * F + gg + K) * G + gg;
+    const int f = t0 + K;
+    return base + (long long)(f < rows ? f : f - rows) * G;
   }
 };
 
@@ -442,8 +470,7 @@ struct BLine {
 template <typename V>
 __global__ void __launch_bounds__(256) k_brecords(BLine ln, const double* __restrict__ A,
                                                   const double* __restrict__ dinv, V* __restrict__ rec) {
-  ln.w = blockIdx.x;
-  ln.pr = blockIdx.z;
+  ln.enter(blockIdx.x, blockIdx.z);
   const int lane = threadIdx.x & 31, K = blockIdx.y * 8 + (threadIdx.x >> 5);
   long long p;
   if (!ln.point(lane, K, p)) return;
@@ -464,8 +491,7 @@ template <typename V>
 __global__ void __launch_bounds__(256) k_bcopy(BLine ln, int to_stream, const V* __restrict__ src,
                                                const V* __restrict__ dinv, V* __restrict__ dst) {
   __shared__ V t[3][32][33];
-  ln.w = blockIdx.x;
-  ln.pr = blockIdx.z;
+  ln.enter(blockIdx.x, blockIdx.z);
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k0 = blockIdx.y * 32;
   long long p;
   if (to_stream) {
@@ -520,8 +546,7 @@ __global__ void __launch_bounds__(256) k_bhalf(BLine ln, const V* __restrict__ A
                                                const V* __restrict__ x, const V* __restrict__ b, V* __restrict__ cs,
                                                V* __restrict__ hs) {
   __shared__ V t[3][32][33];
-  ln.w = blockIdx.x;
-  ln.pr = blockIdx.z;
+  ln.enter(blockIdx.x, blockIdx.z);
   const Grid g = ln.g;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k0 = blockIdx.y * 32;
   const long long step[3] = {(long long)g.ny * g.nz, g.nz, 1};
@@ -573,7 +598,7 @@ __global__ void __launch_bounds__(256) k_bhalf(BLine ln, const V* __restrict__ A
   }
 }
 
-BLine line_of(const Grid& g, const TriShape& t, int dir) { return BLine{g, t.G, t.F, t.groups, dir, 0, 0}; }
+BLine line_of(const Grid& g, const TriShape& t, int dir) { return BLine{g, t.G, t.groups, t.rows, dir, 0, 0, 0, 0}; }
 
 template <typename V>
 cudaError_t go(int CL, const BtriParams& P, cudaStream_t st) {
@@ -598,15 +623,15 @@ TriShape btri_shape(const Grid& g, int pk) {
   t.ns = 7;
   t.G = pk == K64 ? kPlanes<double> : kPlanes<float>;
   t.strips = (g.nx + 31) / 32;
-  t.groups = (g.ny + 31 + t.G - 1) / t.G;
-  t.F = t.G - 1 + g.nz;
+  t.groups = (g.ny + t.G - 1) / t.G;
+  t.rows = g.nz;
   t.CL = tri_cluster(t, g, pk);
   return t;
 }
 
 size_t btri_rec_bytes(const TriShape& t, int pk) { return tri_slots(t) * kTerms * (pk == K64 ? 8 : 4); }
 size_t btri_mail_bytes(const TriShape& t, int pk) {
-  return (size_t)t.strips * t.groups * t.F * entries_of(t.G) * 3 * (pk == K64 ? 16 : 8);
+  return (size_t)t.strips * t.groups * t.rows * entries_of(t.G) * 3 * (pk == K64 ? 16 : 8);
 }
 
 cudaError_t launch_btri_records(const Grid& g, const TriShape& t, int pk, const double* A, const double* dinv,
@@ -653,7 +678,7 @@ cudaError_t launch_btri(const LevelView& L, const TriShape& t, const TriCall& c,
   P.g = L.g;
   P.nunits = tri_unit_count(L.g, t);
   P.ngrp = t.groups;
-  P.F = t.F;
+  P.rows = t.rows;
   P.tiles = tiles;
   P.flip = c.flip;
   P.relax = c.relax;

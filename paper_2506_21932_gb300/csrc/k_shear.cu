@@ -13,7 +13,15 @@ namespace {
 // One plane of a strip in a stream: w the strip, pr = P - 32 w the plane.
 struct Line {
   Grid g;
-  int SP, SL, G, F, groups, dir, w, pr;
+  int SP, SL, G, groups, rows, dir, w, pr;
+  int t0;          // time of row 0, folded
+  long long base;  // first stream row of the plane
+  __device__ __forceinline__ void enter(int strip, int plane) {
+    w = strip;
+    pr = plane;
+    t0 = (SP * (32 * w + pr) + SL * 32 * w) % rows;
+    base = (long long)(w * groups + pr / G % groups) * rows * G + pr % G;
+  }
   // Whether lane il has a point at row r (K = r - SL il), and its natural
   // index and coordinates.
   __device__ __forceinline__ bool point(int il, int r, long long& p, int& i, int& j, int& k) const {
@@ -40,8 +48,10 @@ struct Line {
   }
   // Stream row (32 slots) of row r.
   __device__ __forceinline__ long long row(int r) const {
-    const int d = pr / G, gg = pr % G;
-    return ((long long)(w * groups + d) * F + SP * gg + r) * G + gg;
+    int f = t0 + r;
+    if (f >= rows) f -= rows;
+    if (f >= rows) f %= rows;  // short columns
+    return base + (long long)f * G;
   }
 };
 
@@ -63,8 +73,7 @@ __global__ void __launch_bounds__(256) k_records(Line ln, int whole_scale, const
   using Vec = typename Prec<PK>::vec;
   constexpr int EC = Shape<NS>::EC;
   const int lane = threadIdx.x & 31, r = blockIdx.y * 8 + (threadIdx.x >> 5), dir = ln.dir;
-  ln.w = blockIdx.x;
-  ln.pr = blockIdx.z;
+  ln.enter(blockIdx.x, blockIdx.z);
   long long p;
   int i, j, k;
   if (!ln.point(lane, r, p, i, j, k)) return;
@@ -100,8 +109,7 @@ template <typename T, int KC>
 __global__ void __launch_bounds__(256) k_shear_copy(Line ln, int to_stream, const T* __restrict__ src,
                                                     T* __restrict__ dst, int add) {
   __shared__ T t[KC][33];
-  ln.w = blockIdx.x;
-  ln.pr = blockIdx.z;
+  ln.enter(blockIdx.x, blockIdx.z);
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k0 = blockIdx.y * KC, rows = KC + 31 * ln.SL;
   long long p;
   int i, j, k, kk;
@@ -135,14 +143,15 @@ __global__ void __launch_bounds__(256) k_shear_copy(Line ln, int to_stream, cons
 // last entry is used when too many warps do so, and too few registers keep too
 // few loads in flight: residual at 384^3 in ms with 6, 8, 5, 4, 3 blocks per SM
 //   FP64 3.98 5.69 3.02 2.94 3.00 (2.48 of multiply-adds).
-// FP32 rows go through shared memory in whole lines (256^3: 0.72 to 0.52 ms; FP64
-// rows that way: 6.2 ms at 384^3); BF16 208 x 144 x 176: 0.139 with 8 blocks,
-// 0.125 with 5.
+// FP32 rows go through shared memory in whole lines (FP64 rows that way: 6.2 ms at
+// 384^3), 32 KB a block on 27 points, so at most seven fit; seven or eight leave
+// too few registers (256^3: 0.44 ms with 6 blocks, 0.81 with 7 or 8; without
+// shared memory 0.72).  BF16 208 x 144 x 176: 0.139 with 8 blocks, 0.125 with 5.
 template <int PK, int NS>
 struct ResidualCfg {
   using Val = typename Prec<PK>::val;
   static constexpr bool STAGE = PK == K32;
-  static constexpr int blocks = PK == K64 ? 4 : PK == K32 ? 8 : 5;  // per SM
+  static constexpr int blocks = PK == K64 ? 4 : PK == K32 ? 6 : 5;  // per SM
   static constexpr size_t rows = STAGE ? sizeof(Val) * 8 * 32 * NS : 0;
 };
 template <int PK, int NS>
@@ -154,8 +163,7 @@ __global__ void __launch_bounds__(256, ResidualCfg<PK, NS>::blocks)
   using Val = typename Prec<PK>::val;
   __shared__ V t[32][33];
   extern __shared__ __align__(16) unsigned char rows_raw[];
-  ln.w = blockIdx.x;
-  ln.pr = blockIdx.z;
+  ln.enter(blockIdx.x, blockIdx.z);
   const Grid g = ln.g;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k0 = blockIdx.y * 32;
   long long p;
@@ -233,8 +241,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_shear_split(Line ln, const T* __restrict__ f, const T* __restrict__ h,
                                                      T* __restrict__ d0, T* __restrict__ d1) {
   __shared__ T tf[32][33], th[32][33];
-  ln.w = blockIdx.x;
-  ln.pr = blockIdx.z;
+  ln.enter(blockIdx.x, blockIdx.z);
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k0 = blockIdx.y * 32;
   long long p;
   int i, j, k, kk;
@@ -256,7 +263,7 @@ __global__ void __launch_bounds__(256) k_shear_split(Line ln, const T* __restric
 Line line_of(const Grid& g, const TriShape& t, int dir) {
   const int SP = t.ns == 27 ? Shear<27>::SP : t.ns == 19 ? Shear<19>::SP : Shear<7>::SP;
   const int SL = t.ns == 27 ? Shear<27>::SL : t.ns == 19 ? Shear<19>::SL : Shear<7>::SL;
-  return Line{g, SP, SL, t.G, t.F, t.groups, dir, 0, 0};
+  return Line{g, SP, SL, t.G, t.groups, t.rows, dir, 0, 0, 0, 0};
 }
 
 // Strips by chunks of steps by planes of a strip.

@@ -75,14 +75,12 @@ int tri_cluster(const TriShape& t, const Grid& g, int pk) {
 }
 
 TriShape tri_shape(const Grid& g, int ns, int pk) {
-  const int SB = ns == 27 ? Shape<27>::SB : ns == 19 ? Shape<19>::SB : Shape<7>::SB;
-  const int SA = ns == 27 ? Shape<27>::SA : ns == 19 ? Shape<19>::SA : Shape<7>::SA;
   TriShape t;
   t.ns = ns;
   t.G = planes_per_tile(g, ns, pk);
   t.strips = (g.nx + 31) / 32;
-  t.groups = (g.ny + 31 + t.G - 1) / t.G;
-  t.F = SB * (t.G - 1) + 31 * (SA - SB) + g.nz;
+  t.groups = (g.ny + t.G - 1) / t.G;
+  t.rows = g.nz;
   t.CL = tri_cluster(t, g, pk);
   return t;
 }
@@ -93,7 +91,7 @@ bool tri_supported(const LevelView& L) {
 
 size_t tri_mail_bytes(const TriShape& t, int pk) {
   const size_t word = pk == K64 ? 16 : 8;
-  return word * (size_t)t.strips * t.groups * t.F * (64 + std::max(0, t.G - 2));
+  return word * (size_t)t.strips * t.groups * tri_mail_rows(t, pk) * (64 + std::max(0, t.G - 2));
 }
 
 size_t tri_rec_bytes(const TriShape& t, int pk, bool hd) {
@@ -134,7 +132,11 @@ cudaError_t launch_tri(const LevelView& L, const TriShape& t, const TriCall& c, 
   P.g = L.g;
   P.nunits = tri_unit_count(L.g, t);
   P.ngrp = t.groups;
-  P.F = t.F;
+  P.rows = t.rows;
+  P.mrows = tri_mail_rows(t, L.pk);
+  const int SA = t.ns == 27 ? Shape<27>::SA : t.ns == 19 ? Shape<19>::SA : Shape<7>::SA;
+  const int SB = t.ns == 27 ? Shape<27>::SB : t.ns == 19 ? Shape<19>::SB : Shape<7>::SB;
+  P.last_row = (SA * (L.g.nx - 1) + SB * (L.g.ny - 1) + L.g.nz - 1) % t.rows;
   P.tiles = tiles;
   P.flip = c.flip;
   P.budget_ns = budget_ns;

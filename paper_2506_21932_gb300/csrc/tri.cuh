@@ -18,13 +18,20 @@
 // consecutive P, all planes one time step at a time.  Vectors and records are
 // stored in that order, tile by tile and step by step, so a step of a tile is
 // one contiguous run and one bulk copy per array:
-//   tile t = w * groups + d: I = 32 w + lane, P = 32 w + G d + g,
-//   step f = SP*g + SL*lane + K, 0 <= f < F = SP (G - 1) + 31 SL + nz,
-//   slot = ((t*F + f)*G + g)*32 + lane
-// (steps at which a lane has no point are left out: F - nz of F steps, and
-// the corners of the strip).  The forward stream of a level uses I = i, J = j,
-// K = k, the backward stream the mirrored coordinates; a solve reads its
-// right-hand side in its own stream and writes its result to either.
+//   tile (w, d): I = 32 w + lane, P = 32 w + G d + g, SP (G - 1) + 31 SL + nz steps.
+// A lane has a point in only nz of these steps, one after another, and in only
+// ny of its strip's planes, so times and tiles are stored modulo nz and modulo
+// groups = ceil(ny / G), and no two points meet:
+//   slot = (((w * groups + d mod groups) * nz + T mod nz)*G + g)*32 + lane.
+// What is left of padding is a last strip of less than 32 I, and ny rounded up to
+// G.  (With a slot for every step and tile the FP64 ILU(0) hierarchy of 1024 x
+// 1024 x 8 took 3,850 bytes a point and that of 2048 x 1024 x 1 23,800; now 980 in
+// both.)  A row thus holds values of several steps and tiles, each lane's of one:
+// a tile copies whole rows, and a lane without a point at that step does not use
+// its value.  The forward stream of a level uses I = i, J = j, K = k, the
+// backward stream the mirrored coordinates; a solve reads its right-hand side in
+// its own stream and writes its result to either (time T of one is Tmax - T of
+// the other, so all lanes and tiles reach the end of the stored steps at once).
 // A record is the strictly lower coefficients in sweep order, each 32 lanes
 // wide, negated (an FP64 negation in the kernel would be an FP64 instruction),
 // for BF16 plain and in pairs, then the FP32 row scale (BF16), then the
@@ -54,13 +61,20 @@ struct TriRec {
 struct TriShape {
   int ns, G;              // mask, planes per tile
   int CL;                 // consecutive tiles of a strip taken by one cluster
-  int strips, groups, F;  // strips of I, groups of planes per strip, steps per tile
+  int strips;             // strips of I
+  int groups, rows;       // groups of planes stored per strip, steps stored per group
 };
 TriShape tri_shape(const Grid& g, int ns, int pk);
 int tri_cluster(const TriShape& t, const Grid& g, int pk);  // CL of a shape
 
+// Steps that a loader asks the mailbox for at once, and steps per group stored in it,
+// no fewer (2048 x 1024 x 1 FP32: a cycle of 41 ms with one, 26 with eight).
+__host__ __device__ constexpr int tri_mail_batch(int pk) { return pk == K64 ? 4 : 8; }
+inline int tri_mail_rows(const TriShape& t, int pk) {
+  return t.rows < tri_mail_batch(pk) ? tri_mail_batch(pk) : t.rows;
+}
 // Slots of a stream (values of one vector).
-inline size_t tri_slots(const TriShape& t) { return (size_t)t.strips * t.groups * t.F * t.G * 32; }
+inline size_t tri_slots(const TriShape& t) { return (size_t)t.strips * t.groups * t.rows * t.G * 32; }
 // Mailbox bytes of a level (zeroed once; shared by its solves).
 size_t tri_mail_bytes(const TriShape& t, int pk);
 // Bytes of all records of one solve on a level.

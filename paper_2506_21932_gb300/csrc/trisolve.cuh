@@ -48,6 +48,7 @@
 #pragma once
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "mailbox.cuh"
 #include "tri.cuh"
@@ -86,7 +87,9 @@ __host__ __device__ constexpr int stage_of(int e) {
 struct TriParams {
   Grid g;
   int nstg;             // record stages (steps)
-  int nunits, ngrp, F;  // units of CL tiles; groups of planes per strip; steps per tile
+  int nunits, ngrp;     // units of CL tiles; groups of planes stored per strip
+  int rows, last_row;   // steps stored per group; stored step of the solve's last time
+  int mrows;            // steps of a group in the mailbox
   const int* tiles;     // strip << 16 | first group of a unit, in the order they are claimed
   int flip;
   unsigned long long budget_ns;
@@ -107,6 +110,7 @@ struct TriShared {
   int done;                     // every step < done is finished
   int abort;                    // a wait ran out (or another CTA's did)
   int tile;
+  int row, mrow;                // stored step of the tile's first time, in streams and mailbox
 };
 
 template <int G, int H>
@@ -217,17 +221,15 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   V* u = (V*)P.u;
   V* ev = (V*)P.emit;
-  // Slot of point (I, p, time T) in the result's stream: column(I, p) + dstep * T.
-  const int dstep = P.flip ? -G * 32 : G * 32;
-  auto column = [&](int I, int p) -> long long {
-    int c = I, q = p, k0 = -(SP * p + SL * I);  // K = T + k0
-    if (P.flip) {
-      c = g.nx - 1 - I;
-      q = g.nx + g.ny - 2 - p;
-      k0 = g.nz - 1 - k0;  // the mirrored K at T = 0
-    }
-    const int cw = c >> 5, cl = c & 31, pr = q - 32 * cw, cd = pr / G, cg = pr % G;
-    return (((long long)(cw * P.ngrp + cd) * P.F + SP * cg + SL * cl + k0) * G + cg) * 32 + cl;
+  // Store of group d of strip w (d < ngrp + 32, few subtractions), and a stored step
+  // of rows counted back below the first.
+  auto group = [&](int w, int d) -> long long {
+    while (d >= P.ngrp) d -= P.ngrp;
+    return w * P.ngrp + d;
+  };
+  auto back = [&](int row, int rows) {
+    while (row < 0) row += rows;
+    return row;
   };
   if (threadIdx.x == 0) {
     for (int t = 0; t < nch; ++t) mbar_init(&sh.full[t], 1);
@@ -267,6 +269,8 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       sh.rready = T0;
       sh.done = T0 - kRecAhead;
       sh.abort = 0;
+      sh.row = T0 % P.rows;
+      sh.mrow = T0 % P.mrows;
     }
     cluster_sync();
     if (!live) continue;
@@ -319,15 +323,28 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       if (role == 0) {
         const int koff = SP * p + SL * I;
         const unsigned nk = colok ? (unsigned)g.nz : 0u;
-        // the lane's results, mailbox entry (every lane of the last two planes,
-        // lane 31 of the others; inside the cluster the next tile's own mailbox)
-        const long long at = colok ? column(I, p) + (long long)dstep * Tb : 0;
+        // The lane's results: column (c, q) of the result's stream, whose time is T or
+        // (mirrored) Tm - T; the stored steps run out at time tw.
+        int c = I, q = p, row = back(sh.row - kRecAhead, P.rows), tw = Tb + P.rows - row;
+        const int dstep = P.flip ? -G * 32 : G * 32;
+        if (P.flip) {
+          c = g.nx - 1 - I;
+          q = g.nx + g.ny - 2 - p;
+          row = back(P.last_row - row, P.rows);
+          tw = Tb + row + 1;
+        }
+        const int cw = c >> 5, cp = q - 32 * cw;
+        const long long at = colok ? ((group(cw, cp / G) * P.rows + row) * G + cp % G) * 32 + (c & 31) : 0;
         V* up = u + at;
         V* ep = ev + at;
+        // mailbox entry (every lane of the last two planes, lane 31 of the others;
+        // inside the cluster the next tile's own mailbox); its steps run out at mw
         const bool near = above && pl >= G - 2, post = (pl >= G - 2 && !above) || lane == 31;
         const unsigned peer = near ? peer_addr(own_mail + (pl - (G - 2)) * (kMail * 32) + lane, rank + 1) : 0u;
-        typename ML::word* mb = mail + ((long long)(w * P.ngrp + dg) * P.F + (Tb - T0)) * ME +
-                                (pl >= G - 2 ? (pl - (G - 2)) * 32 + lane : 64 + pl);
+        const int mrow = back(sh.mrow - kRecAhead, P.mrows);
+        int mw = Tb + P.mrows - mrow;
+        typename ML::word* mb =
+            mail + (group(w, dg) * P.mrows + mrow) * ME + (pl >= G - 2 ? (pl - (G - 2)) * 32 + lane : 64 + pl);
         // H == 0: c1, c2, c3 are the partial sums of T + 1, T + 2, T + 3 before this step's share
         constexpr bool kOlder = H == 0 && nterms<NS>(0) + nterms<NS>(1) + nterms<NS>(2) > 0;
         Terms<PK, NS, 3> k3;
@@ -355,36 +372,56 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
           q4 = next(q4);
         };
         fetch();
-        for (int T = Tb; T <= Te; ++T) {
-          step_barrier<(NC + 1) * 32>();
-          const bool ok = (unsigned)(T - koff) < nk;
-          V a = k3.add(H ? cell(2, T) : c1, rb, T);
-          if (PK == KBF) {
-            a = mul_rn(V(reinterpret_cast<const float*>(rec(q0) + R::S_OFF)[0]), a);
-            a = vec(q0, 0) - a;
+        // Steps between two turns of the stored steps.  Two forms, with and without
+        // weight and emit: with one form for both the ILU(0) solves with helpers, two
+        // planes, took 0.40 / 0.47 ms at 128^3 instead of 0.375 / 0.41.
+        auto run = [&](auto full) {
+          constexpr bool kFull = decltype(full)::value;
+          auto step = [&](int T) {
+            step_barrier<(NC + 1) * 32>();
+            const bool ok = (unsigned)(T - koff) < nk;
+            V a = k3.add(H ? cell(2, T) : c1, rb, T);
+            if (PK == KBF) {
+              a = mul_rn(V(reinterpret_cast<const float*>(rec(q0) + R::S_OFF)[0]), a);
+              a = vec(q0, 0) - a;
+            }
+            V r = a;
+            if (HD) r = a * d;
+            if (kFull && P.relax) r = P.relax == 1 ? wv * r : fma(wv, r, mul_rn(V(1) - wv, vec(q0, ooff)));
+            own[(T & (kRing - 1)) * kLanes] = ok ? r : V(0);
+            if (kTurn) asm volatile("bar.arrive 2, %0;" ::"n"(G * 64) : "memory");
+            if (ok) {
+              if (near)
+                ML::put_peer(peer + (T & (kMail - 1)) * (32 * (unsigned)sizeof(typename ML::word)), r, (unsigned)T + 1u);
+              if (post) ML::put(mb, r, tag);
+              *up = r;
+              if (kFull && ev) *ep = P.h ? a + vec(q0, hoff) : a;
+            }
+            up += dstep;
+            if (kFull) ep += dstep;
+            mb += ME;
+            if (kOlder) {
+              c1 = k2.add(c2, rb, T + 1);
+              c2 = k1.add(c3, rb, T + 2);
+              c3 = k0.add(b3, rb, T + 3);
+            }
+            fetch();
+          };
+          for (int T = Tb; T <= Te;) {
+            for (const int end = min(min(tw, mw), Te + 1); T < end; ++T) step(T);
+            if (T == tw) {
+              up -= (long long)P.rows * dstep;
+              if (kFull) ep -= (long long)P.rows * dstep;
+              tw += P.rows;
+            }
+            if (T == mw) {
+              mb -= (long long)P.mrows * ME;
+              mw += P.mrows;
+            }
           }
-          V r = a;
-          if (HD) r = a * d;
-          if (P.relax) r = P.relax == 1 ? wv * r : fma(wv, r, mul_rn(V(1) - wv, vec(q0, ooff)));
-          own[(T & (kRing - 1)) * kLanes] = ok ? r : V(0);
-          if (kTurn) asm volatile("bar.arrive 2, %0;" ::"n"(G * 64) : "memory");
-          if (ok) {
-            if (near)
-              ML::put_peer(peer + (T & (kMail - 1)) * (32 * (unsigned)sizeof(typename ML::word)), r, (unsigned)T + 1u);
-            if (post) ML::put(mb, r, tag);
-            *up = r;
-            if (ev) *ep = P.h ? a + vec(q0, hoff) : a;
-          }
-          up += dstep;
-          ep += dstep;
-          mb += ME;
-          if (kOlder) {
-            c1 = k2.add(c2, rb, T + 1);
-            c2 = k1.add(c3, rb, T + 2);
-            c3 = k0.add(b3, rb, T + 3);
-          }
-          fetch();
-        }
+        };
+        if (P.relax || ev) run(std::true_type{});
+        else run(std::false_type{});
       } else if (role == 1) {
         Terms<PK, NS, 0> k;
         int q = stage_of_time(Tb + 3);
@@ -451,7 +488,7 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       // column left of the strip (lane q < G + 2: plane p0-2+q)
       const int c = warp - (NC + 1);
       constexpr int SG = 32 / G;
-      constexpr int kBatch = sizeof(V) == 8 ? 4 : 8;  // time steps asked for at once
+      constexpr int kBatch = tri_mail_batch(PK);  // time steps asked for at once
       const int pc = p0 - 2 + (c < 2 ? c : lane), Ic = c < 2 ? I : 32 * w - 1, Jc = pc - Ic;
       const bool mine = c < 2 || lane < G + 2;
       const bool okc = mine && Ic >= 0 && Ic < g.nx && Jc >= 0 && Jc < g.ny;
@@ -459,17 +496,15 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       const int cw = c < 2 ? w : w - 1;
       const int cd = c < 2 ? dg - 1 : lane < 2 ? dg + SG - 1 : dg + SG;
       const int cg = c < 2 ? G - 2 + c : lane < 2 ? G - 2 + lane : lane - 2;
-      const int ct0 = SP * (32 * cw + G * cd) + SL * 32 * cw;
       const int e = cg >= G - 2 ? (cg - (G - 2)) * 32 + (c < 2 ? lane : 31) : 64 + cg;
-      const typename ML::word* src =  // entry of time 0
-          okc ? mail + ((long long)(cw * P.ngrp + cd) * P.F - ct0) * ME + e : mail;
+      const typename ML::word* src = okc ? mail + group(cw, cd) * P.mrows * ME + e : mail;
       const bool near = c < 2 && below;
       const typename ML::word* box = own_mail + (c & 1) * (kMail * 32) + lane;
       const unsigned taken = near ? peer_addr(&sh.taken[c], rank - 1) : 0u;
       V* dst = ring + (c < 2 ? c : min(lane, G + 1)) * (kRing * kLanes) + (c < 2 ? lane + 1 : 0);
       // times at which this lane has a point to fetch
       const int t_lo = okc ? SP * pc + SL * Ic : INT_MAX, t_hi = okc ? t_lo + g.nz : INT_MIN;
-      int tau = T0 - kOldest;
+      int tau = T0 - kOldest, row = back(sh.mrow - kOldest, P.mrows);  // row: its step in the mailbox
       unsigned long long t_wait = 0;
       unsigned iter = 0;
       int ask = 1;  // one step while waiting for the first, a batch once they come
@@ -511,14 +546,15 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       }
       while (!near && tau < Te) {
         // lane 0's view for all: the votes below need every lane
-        const int n = __shfl_sync(0xffffffffu, min(min(ld_acq_cta(&sh.done) + kRing - 4, Te) - tau, ask), 0);
+        const int n = min(P.mrows - row,
+                          __shfl_sync(0xffffffffu, min(min(ld_acq_cta(&sh.done) + kRing - 4, Te) - tau, ask), 0));
         int got = 0;
         if (n > 0) {
           typename ML::word val[kBatch];
 #pragma unroll
           for (int q = 0; q < kBatch; ++q) {
             val[q] = ML::value(V(0), tag);
-            if (q < n && tau + q >= t_lo && tau + q < t_hi) val[q] = ML::get(src + (long long)(tau + q) * ME);
+            if (q < n && tau + q >= t_lo && tau + q < t_hi) val[q] = ML::get(src + (long long)(row + q) * ME);
           }
 #pragma unroll
           for (int q = 0; q < kBatch; ++q)
@@ -529,6 +565,7 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
         }
         if (got > 0) {
           tau += got;
+          row = row + got == P.mrows ? 0 : row + got;
           __syncwarp();
           if (lane == 0) st_rel_cta(&sh.hready[c], tau);
           t_wait = 0;
@@ -563,16 +600,16 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       }
     } else if (warp == NC + 4) {
       // ---- record warp
-      // one lane; step f of the tile is one run in every stream
+      // one lane; consecutive stored steps of the tile are one run in every stream
       if (lane == 0) {
         const int nfill = Te - T0 + 1;
-        const long long step0 = (long long)(w * P.ngrp + dg) * P.F;
+        const long long step0 = group(w, dg) * P.rows;
         const char* rec = (const char*)P.rec + step0 * (G * R::BYTES);
         const V* bv = (const V*)P.b + step0 * (G * 32);
         const V* hv = (const V*)P.h + step0 * (G * 32);
         const V* ov = (const V*)P.old + step0 * (G * 32);
         constexpr unsigned vbytes = G * 32 * sizeof(V);
-        int done = T0 - kRecAhead, ch = (int)(base % (unsigned)nch), issued = 0;
+        int done = T0 - kRecAhead, ch = (int)(base % (unsigned)nch), issued = 0, row = sh.row;
         for (int f = 0; f < nfill; f += C) {
           // the previous occupants of the chunk, up to time T0 + f + C - 1 - nstg, are finished
           const int free_at = T0 + f + C - 1 - nstg;
@@ -589,12 +626,21 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
           if (stop) break;
           const int n = min(C, nfill - f);
           unsigned long long* bar = &sh.full[ch];
+          char* sr = stages + ch * (C * G * R::BYTES);
           V* sv = vecs + ch * (C * G * 32);
           mbar_expect_tx(bar, n * (unsigned)(G * R::BYTES + nvec * vbytes));
-          bulk_copy_g2s(stages + ch * (C * G * R::BYTES), rec + (long long)f * (G * R::BYTES), n * G * R::BYTES, bar);
-          bulk_copy_g2s(sv, bv + (long long)f * (G * 32), n * vbytes, bar);
-          if (P.h) bulk_copy_g2s(sv + hoff, hv + (long long)f * (G * 32), n * vbytes, bar);
-          if (P.relax == 2) bulk_copy_g2s(sv + ooff, ov + (long long)f * (G * 32), n * vbytes, bar);
+          for (int left = n; left > 0;) {  // one run, or up to the last stored step and on from the first
+            const int m = min(left, P.rows - row);
+            const long long at = (long long)row * (G * 32);
+            bulk_copy_g2s(sr, rec + (long long)row * (G * R::BYTES), m * G * R::BYTES, bar);
+            bulk_copy_g2s(sv, bv + at, m * vbytes, bar);
+            if (P.h) bulk_copy_g2s(sv + hoff, hv + at, m * vbytes, bar);
+            if (P.relax == 2) bulk_copy_g2s(sv + ooff, ov + at, m * vbytes, bar);
+            sr += m * (G * R::BYTES);
+            sv += m * (G * 32);
+            left -= m;
+            row = row + m == P.rows ? 0 : row + m;
+          }
           ++issued;
           ch = ch + 1 == nch ? 0 : ch + 1;
         }
