@@ -249,15 +249,12 @@ enum {
 };
 int smg_level_apply(smg_t h, int l, int op, const void* x, const void* b, void* y, void* stream);
 
-/* The number the option sweep_warps stands for on the point sweep `op`
- * (SMG_OP_GS_FORWARD / GS_BACKWARD / GS_ZERO / ILU_LOWER / ILU_UPPER) of level
- * l, by mask, precision and y extent: 2 on 19/27-point levels with ny <= 256
- * (not FP64 Gauss-Seidel with old values), and for the FP64 ILU(0) solves up
- * to ny = 384, unless the option is 1; otherwise 1; 0 where the level has no
- * such sweep or smg_sweep_noalloc's kernel for it is another one.  The rule is
- * that of the option's first kernels; it does not count the warps of the
- * kernel that runs today.  Host-only: launches nothing.  Errors: -SMG_EINVAL
- * for a bad handle, level or op. */
+/* How the V-cycle runs the point sweep `op` (SMG_OP_GS_FORWARD / GS_BACKWARD /
+ * GS_ZERO / ILU_LOWER / ILU_UPPER) of level l: 2 as a sheared wavefront with
+ * helper warps (FP64, 19/27-point masks, one unknown per point, option
+ * sweep_warps not 1), 1 as a sheared wavefront without, 0 another kernel (other
+ * masks), or the level has no such sweep.  Host-only: launches nothing.
+ * Errors: -SMG_EINVAL for a bad handle, level or op. */
 int smg_level_sweep_warps(smg_t h, int l, int op);
 
 /* Number of CUDA kernels this library has enqueued since it was loaded (a

@@ -483,18 +483,17 @@ cudaError_t launch_kind(int kind, int dir, const Sweep3Params& P, cudaStream_t s
 // mask, at most 12 warps of columns (8 for Gauss-Seidel with old values).
 bool sweep3_supported(const LevelView& L, int kind) {
   const int ns = L.s.ns;
-  if (L.B != 1) return false;
+  if (L.B != 1 || L.pk != K64) return false;
   if (!((ns == 27 && canonical<27>(L.s)) || (ns == 7 && canonical<7>(L.s)) || (ns == 19 && canonical<19>(L.s))))
     return false;
   const int NW = (L.g.ny + 31) / 32;
-  const int maxt = L.pk != K64 ? (kMaxWarpsPerPlane + 2) * 32
-                               : (kind == SW_GS_FULL ? max_threads<SW_GS_FULL>() : max_threads<SW_ILU_L>());
+  const int maxt = kind == SW_GS_FULL ? max_threads<SW_GS_FULL>() : max_threads<SW_ILU_L>();
   return (NW + 2) * 32 <= maxt && (size_t)L.g.nx * NW <= (size_t)kProgSlots;
 }
 
 cudaError_t launch_sweep3(const LevelView& L, int kind, int dir, const void* M, const void* dinv, double w,
                           const void* b, void* u, SweepWs* ws, int* err, const SweepCfg& cfg, cudaStream_t st) {
-  if (L.pk != K64 || !sweep3_supported(L, kind)) return cudaErrorNotSupported;
+  if (!sweep3_supported(L, kind)) return cudaErrorNotSupported;
   Sweep3Params P;
   P.g = L.g;
   P.budget_ns = cfg.budget_ns;
@@ -511,15 +510,4 @@ cudaError_t launch_sweep3(const LevelView& L, int kind, int dir, const void* M, 
   else e = launch_kind<19>(kind, dir, P, st);
   smg_count_launch(1);
   return e;
-}
-
-// The number smg_level_sweep_warps reports for a sheared level's sweep: 1 or
-// 2 by mask, precision, width and the option (see smg.h).
-int sweep3_warps(const LevelView& L, int kind, const SweepCfg& cfg) {
-  if (!sweep3_supported(L, kind)) return 0;
-  const int NW = (L.g.ny + 31) / 32;
-  const bool ilu = kind == SW_ILU_L || kind == SW_ILU_U;
-  const bool two = (L.s.ns == 19 || L.s.ns == 27) &&
-                   (NW <= 8 ? !(L.pk == K64 && kind == SW_GS_FULL) : (L.pk == K64 && ilu && NW <= 12));
-  return cfg.warps != 1 && two ? 2 : 1;
 }

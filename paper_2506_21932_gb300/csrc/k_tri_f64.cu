@@ -20,7 +20,6 @@ bool canonical(const Stencil& s) {
 
 template <int NS, bool HD>
 cudaError_t go(const TriShape& t, bool helpers, const TriParams& P, cudaStream_t st) {
-  // the 7-point mask has no terms older than one step to hand over
   if constexpr (NS == 7) {
     return launch_tri_kernel<K64, NS, HD, 4, 0, 16>(t.CL, P, st);
   } else {
@@ -152,7 +151,7 @@ cudaError_t launch_tri(const LevelView& L, const TriShape& t, const TriCall& c, 
   P.ws = ws;
   P.err = err;
   cudaError_t e;
-  if (L.pk == K64) e = tri_launch_k64(t.ns, c.hd, t, c.warps != 1, P, st);
+  if (L.pk == K64) e = tri_launch_k64(t.ns, c.hd, t, tri_helpers(t.ns, L.pk, c.warps), P, st);
   else if (L.pk == K32) e = tri_launch_k32(t.ns, c.hd, t, P, st);
   else e = tri_launch_kbf(t.ns, c.hd, t, P, st);
   if (e == cudaSuccess) smg_count_launch(1);

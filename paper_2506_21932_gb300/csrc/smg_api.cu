@@ -647,7 +647,6 @@ static int setup_level_smoother(smg_ctx* h, Level& L, cudaStream_t st) {
   // (at the price of a G-step larger lag between consecutive planes)
   L.cfg.G = 4;
   L.cfg.budget_ns = (unsigned long long)h->opt.spin_budget_ms * 1000000ull;
-  L.cfg.warps = h->opt.sweep_warps;
   TRY(dalloc(h, &L.ws, 1));
   SMG_CUDA_TRY(cudaMemsetAsync(L.ws, 0, sizeof(SweepWs), st));
   if (h->opt.smoother == SMG_SMOOTHER_LGS) {
@@ -1173,21 +1172,18 @@ extern "C" int smg_level_count(smg_t h) { return h ? h->nlev : 0; }
 
 extern "C" int smg_level_sweep_warps(smg_t h, int l, int op) {
   if (!h || l < 0 || l >= h->nlev) return -SMG_EINVAL;
-  int kind;
+  int smoother;
   switch (op) {
     case SMG_OP_GS_FORWARD:
-    case SMG_OP_GS_BACKWARD: kind = SW_GS_FULL; break;
-    case SMG_OP_GS_ZERO: kind = SW_GS_ZERO; break;
-    case SMG_OP_ILU_LOWER: kind = SW_ILU_L; break;
-    case SMG_OP_ILU_UPPER: kind = SW_ILU_U; break;
+    case SMG_OP_GS_BACKWARD:
+    case SMG_OP_GS_ZERO: smoother = SMG_SMOOTHER_SGS; break;
+    case SMG_OP_ILU_LOWER:
+    case SMG_OP_ILU_UPPER: smoother = SMG_SMOOTHER_ILU0; break;
     default: return -SMG_EINVAL;
   }
-  Level& L = h->L[l];
-  const bool ilu_op = kind == SW_ILU_L || kind == SW_ILU_U;
-  if (ilu_op != (h->opt.smoother == SMG_SMOOTHER_ILU0) || h->opt.smoother == SMG_SMOOTHER_LGS) return 0;
-  const LevelView v = view(h, L, true);
-  if (!sheared(L) || (!ilu_op && !sweep3_supported(v, SW_GS_FULL))) return 0;
-  return sweep3_warps(v, kind, L.cfg);
+  const Level& L = h->L[l];
+  if (smoother != h->opt.smoother || !sheared(L)) return 0;
+  return L.B == 1 && tri_helpers(L.s.ns, h->pk, h->opt.sweep_warps) ? 2 : 1;
 }
 
 extern "C" int smg_level_info(smg_t h, int l, int dims[3], int* nstencil, int* offsets) {

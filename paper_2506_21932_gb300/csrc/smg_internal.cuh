@@ -170,7 +170,6 @@ struct SweepCfg {
   int SA, SB;  // schedule skews: global time t = SA*i + SB*j + k
   int G;       // publish progress every G steps
   unsigned long long budget_ns;
-  int warps = 0;  // option sweep_warps
 };
 cudaError_t launch_sweep(const LevelView& L, int kind, int dir, const void* M, const float* sc1, const float* sc2,
                          const void* dinv, double w, const void* b, void* u, SweepWs* ws, int* err,
@@ -186,7 +185,6 @@ cudaError_t launch_sweep2(const LevelView& L, int kind, int dir, const void* M, 
 // Warp-pipelined variant on natural-order FP64 data (same masks, at most 12
 // warps of columns); cudaErrorNotSupported (nothing launched) otherwise.
 bool sweep3_supported(const LevelView& L, int kind);
-int sweep3_warps(const LevelView& L, int kind, const SweepCfg& cfg);
 cudaError_t launch_sweep3(const LevelView& L, int kind, int dir, const void* M, const void* dinv, double w,
                           const void* b, void* u, SweepWs* ws, int* err, const SweepCfg& cfg, cudaStream_t st);
 

@@ -83,6 +83,10 @@ size_t tri_rec_bytes(const TriShape& t, int pk, bool hd);
 // Whether the sheared wavefront runs a level's sweeps: one unknown per point,
 // a canonical 7/19/27-point mask.
 bool tri_supported(const LevelView& L);
+// Whether helper warps form the older terms: FP64 (a warp issues its FP64
+// instructions one per 64 cycles), not on the 7-point mask, which has no terms older
+// than one step to hand over, and not with option sweep_warps = 1.
+inline bool tri_helpers(int ns, int pk, int warps) { return pk == K64 && ns != 7 && warps != 1; }
 
 // Order in which the units of CL tiles are claimed: tri_unit_count() entries
 // strip << 16 | first group.

@@ -263,7 +263,7 @@ class SMG:
         return tuple(d), [tuple(off[3 * e:3 * e + 3]) for e in range(ns.value)]
 
     def level_sweep_warps(self, l, op):
-        """Warps per strip of the kernel running sweep `op` on level l (0: another kernel)."""
+        """2: the V-cycle runs sweep `op` of level l as a sheared wavefront with helper warps, 1: without, 0: otherwise."""
         rc = self._lib.smg_level_sweep_warps(self.h, l, op)
         if rc < 0:
             raise SmgError(-rc, "smg_level_sweep_warps")

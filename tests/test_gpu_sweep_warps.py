@@ -1,13 +1,12 @@
-"""The two-warp wavefront sweeps (option sweep_warps = 2) against the one-warp
-kernel and the oracle.
+"""The option sweep_warps of the sheared wavefront, against the oracle.
 
-The two-warp kernel hands the early partial sum of every point, formed in the
-same order as the one-warp kernel's, from a helper warp to the warp that
-finishes the point, so a V-cycle must come out bit for bit the same with
-either kernel.  The cases cover 19- and 27-point masks, ILU(0) and symmetric
-Gauss-Seidel (with and without a weight), the three hierarchy precisions,
-one to twelve 32-column strips per plane with a ragged last strip, one and
-two planes per CTA, and a zero wait budget.
+On FP64 19/27-point levels helper warps form the older terms of a point, in the
+same order as the warp that finishes it does with sweep_warps = 1, so a V-cycle
+must come out bit for bit the same with either kernel.  FP32 and BF16 levels
+have one kernel, which every value of the option runs; there the oracle alone
+is compared.  The cases cover 19- and 27-point masks, ILU(0) and symmetric
+Gauss-Seidel (with and without a weight), the three hierarchy precisions, 20 to
+384 y-points, what the level query says of them, and a zero wait budget.
 """
 import numpy as np
 import pytest
@@ -84,14 +83,14 @@ CASES = [
     ((16, 80, 32), 27, "sgs", 0, 1.0), ((16, 80, 32), 27, "sgs", 1, 1.0), ((16, 80, 32), 27, "sgs", 1, 0.8),
     ((16, 44, 24), 19, "ilu", 0, 1.0), ((16, 44, 24), 19, "ilu", 1, 1.0), ((16, 44, 24), 19, "sgs", 2, 1.0),
     ((16, 44, 24), 19, "sgs", 0, 0.8),
-    # 9 to 12 strips: FP64 ILU(0) on the 832-thread instantiation, the rest on one warp
+    # many tiles in a strip
     ((16, 384, 16), 27, "ilu", 0, 1.0), ((16, 384, 16), 27, "ilu", 1, 1.0), ((16, 352, 16), 27, "ilu", 2, 1.0),
     ((16, 384, 16), 27, "sgs", 2, 1.0), ((16, 352, 16), 27, "sgs", 1, 0.8), ((16, 320, 16), 19, "ilu", 0, 1.0),
 ]
 
 
 @pytest.mark.parametrize("d,mask,smoother,prec,w", CASES)
-def test_two_warp_vcycle_equals_one_warp_and_oracle(S, orc, d, mask, smoother, prec, w):
+def test_vcycle_with_helpers_equals_the_one_without_and_the_oracle(S, orc, d, mask, smoother, prec, w):
     off, A = problem(mask, d)
     sm = S.ILU0 if smoother == "ilu" else S.SGS
     r = cu(I.rhs(int(np.prod(d)), 7).numpy())
@@ -100,28 +99,19 @@ def test_two_warp_vcycle_equals_one_warp_and_oracle(S, orc, d, mask, smoother, p
         h = S.SMG(d, off, cu(A), smoother=sm, precision=prec, relax_w=w, sweep_warps=warps)
         ops = (S.OP_ILU_LOWER, S.OP_ILU_UPPER) if smoother == "ilu" else (S.OP_GS_ZERO, S.OP_GS_FORWARD)
         got = [h.level_sweep_warps(0, op) for op in ops]
-        if warps == 1:
-            assert got == [1, 1]
-        else:  # 2, and the library's choice (0), which takes two warps where they apply
-            # FP64 Gauss-Seidel with old values stays on one warp (it would
-            # spill); planes of more than 8 strips take two warps only for the
-            # FP64 ILU(0) solves
-            wide = (d[1] + 31) // 32 > 8
-            if wide:
-                assert got == ([2, 2] if smoother == "ilu" and prec == 0 else [1, 1])
-            else:
-                assert got == ([2, 2] if smoother == "ilu" else [2, 1 if prec == 0 else 2])
+        assert got == ([2, 2] if prec == 0 and warps != 1 else [1, 1])
         zz = torch.empty_like(r)
         h.vcycle(r, zz)
         z[warps] = zz
         h.close()
-    assert torch.equal(z[1], z[2]) and torch.equal(z[0], z[2])
+    if prec == 0:
+        assert torch.equal(z[1], z[2]) and torch.equal(z[0], z[2])
     ref = orc.MG(d, off, A, smoother=orc.ILU0 if smoother == "ilu" else orc.SGS, precision=prec,
                  w=w).vcycle(host(r))
     assert rel2(host(z[2]), ref) < (TOL_VCYCLE if prec == 0 else TOL_LOWP)
 
 
-def test_two_warp_single_sweeps_in_place(S, orc):
+def test_single_sweeps_in_place(S, orc):
     """The level operations run the same kernel: an in-place ILU(0) upper
     solve after the lower one reproduces the dense triangular solves."""
     d = (8, 40, 8)
@@ -140,10 +130,10 @@ def test_two_warp_single_sweeps_in_place(S, orc):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
-def test_two_warp_zero_wait_budget_aborts_and_context_survives(S, orc, prec):
-    """With a zero wait budget the helper and main warps give up at their
-    first unsatisfied wait (error word set, every CTA drains); with the
-    budget restored the same context runs the oracle's V-cycle."""
+def test_zero_wait_budget_aborts_and_context_survives(S, orc, prec):
+    """With a zero wait budget the loader warps give up at their first
+    unsatisfied wait (error word set, every CTA drains); with the budget
+    restored the same context runs the oracle's V-cycle."""
     d = (24, 40, 24)
     off, A = problem(27, d)
     h = S.SMG(d, off, cu(A), smoother=S.ILU0, precision=prec, sweep_warps=2)
@@ -172,3 +162,32 @@ def test_sweep_warps_query_rejects_bad_arguments(S):
     with pytest.raises(S.SmgError):
         h.level_sweep_warps(99, S.OP_ILU_LOWER)
     assert h.level_sweep_warps(0, S.OP_GS_ZERO) == 0  # not this hierarchy's smoother
+
+
+# (dims, mask, block, smoother, precision) -> (sweep_warps 0, 2 and 1) of the ops
+QUERIES = [
+    ((16, 288, 8), 27, 1, "SGS", 0, (2, 2, 1)),   # wider than the natural-order kernel takes
+    ((16, 400, 8), 27, 1, "ILU0", 0, (2, 2, 1)),
+    ((16, 16, 16), 27, 1, "SGS", 1, (1, 1, 1)),
+    ((16, 16, 16), 19, 1, "ILU0", 2, (1, 1, 1)),
+    ((16, 16, 16), 7, 1, "SGS", 0, (1, 1, 1)),    # no older terms to hand over
+    ((16, 16, 16), 7, 3, "SGS", 0, (1, 1, 1)),
+    ((16, 16, 16), 27, 3, "SGS", 0, (0, 0, 0)),   # blocks on 27 points: another kernel
+    ((16, 16, 16), 13, 1, "SGS", 0, (0, 0, 0)),   # not a canonical mask
+]
+
+
+@pytest.mark.parametrize("d,mask,block,smoother,prec,want", QUERIES)
+def test_query_reports_the_kernel_that_runs(S, d, mask, block, smoother, prec, want):
+    off = {7: I.OFF7, 13: I.OFF7 + [(1, 1, 0), (-1, -1, 0), (0, 1, 1), (0, -1, -1), (1, 0, 1), (-1, 0, -1)],
+           19: I.OFF19, 27: I.OFF27}[mask]
+    A = torch.from_numpy(rnd_sym(d, 3, sorted(off))).cuda()
+    if block == 3:
+        A = A[:, :, None, None] * torch.eye(3, dtype=torch.float64, device="cuda")
+    ops = (S.OP_ILU_LOWER, S.OP_ILU_UPPER) if smoother == "ILU0" else (S.OP_GS_ZERO, S.OP_GS_FORWARD,
+                                                                       S.OP_GS_BACKWARD)
+    for warps, w in zip((0, 2, 1), want):
+        h = S.SMG(d, sorted(off), A, smoother=getattr(S, smoother), precision=prec, block=block, krylov=S.FPCG,
+                  transfer=S.C16XY, sweep_warps=warps)
+        assert [h.level_sweep_warps(0, op) for op in ops] == [w] * len(ops)
+        h.close()
