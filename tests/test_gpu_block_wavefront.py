@@ -116,3 +116,32 @@ def test_block_cycle_equals_its_sweeps(S, prec, w):
     # values of the size of u amplify by the row sums, below 2
     assert torch.linalg.norm(z - u.double()) <= 8 * TOL[prec] * torch.linalg.norm(u.double())
     h.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_block_zero_wait_budget_aborts_and_context_survives(S, prec):
+    """With a zero wait budget the block solves give up at their first unsatisfied
+    wait and every CTA drains, those of one cluster with each other's mailboxes
+    half written; with the budget restored the same context runs the cycle of a
+    context that never gave up, to the bit."""
+    d = (40, 40, 12)  # 36 and 24 FP64 tiles, in clusters of eight
+    A = torch.from_numpy(blocks(d, 7)).cuda()
+    new = lambda: S.SMG(d, I.OFF7, A, block=3, transfer=S.PC8C, smoother=S.SGS, precision=prec, krylov=S.FGMRES,
+                        max_levels=2)
+    r = torch.from_numpy(np.random.default_rng(1).normal(size=int(np.prod(d)) * 3)).cuda()
+    want, z = torch.zeros_like(r), torch.zeros_like(r)
+    fresh, h = new(), new()
+    fresh.vcycle(r, want)
+    fresh.close()
+    for _ in range(2):
+        h.set_wait_budget_ns(0)
+        status = S.OK
+        try:
+            h.vcycle(r, z)
+        except S.SmgError as e:
+            status = e.status
+        assert status in (S.OK, S.ETIMEOUT)
+        h.set_wait_budget_ns(10 ** 9)
+        h.vcycle(r, z)
+        assert torch.equal(z, want)
+    h.close()

@@ -1,10 +1,12 @@
 """Tile shapes of the sheared wavefront that only wide grids reach: four planes
 (FP64) and eight planes (FP32) per tile, clusters of two, four and eight tiles,
 units that end early, and more tiles than clusters are resident at once.
-Sequential sweeps and factors of the oracle in FP64; the matrices are small
-integers over powers of two, so reduced precision only rounds values and sums
-(27 terms and a diagonal, contracting by 78/128 a row: 27 * eps / (1 - 78/128),
-with the larger of that and the repository's bounds)."""
+Single sweeps against the oracle's sequential ones in FP64; the matrices are
+small integers over powers of two, so reduced precision only rounds values and
+sums (27 terms and a diagonal, contracting by 78/128 a row: 27 * eps /
+(1 - 78/128), with the larger of that and the repository's bounds).  Cycles, whose
+solves write to the mirrored stream, in place, with sums handed on and with a
+weight, against the same cycle put together from single level operations."""
 import numpy as np
 import pytest
 
@@ -14,7 +16,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 TOL = {0: 1e-12, 1: 2e-5}
-# planes per tile, tiles per cluster
+EPS = {0: 2.3e-16, 1: 1.2e-7, 2: 1.2e-7}
 # planes per tile, tiles per cluster
 CASES = [((200, 200, 2), 27, 0),   # 4, 4
          ((416, 240, 2), 27, 0),   # 4, 2
@@ -40,10 +42,7 @@ def orc():
     return oracle
 
 
-@pytest.mark.parametrize("d,mask,prec", CASES)
-def test_wide_grids_equal_the_sequential_sweeps(S, orc, d, mask, prec):
-    off = {7: I.OFF7, 19: I.OFF19, 27: I.OFF27}[mask]
-    rng = np.random.default_rng(11)
+def matrix(d, off, rng):
     i, j, k = np.meshgrid(*(np.arange(t) for t in d), indexing="ij")
     A = np.zeros((*d, len(off)))
     for e, o in enumerate(off):
@@ -52,7 +51,14 @@ def test_wide_grids_equal_the_sequential_sweeps(S, orc, d, mask, prec):
             ok &= (x + t >= 0) & (x + t < n)
         A[..., e] = np.where(ok, -rng.integers(1, 4, size=d), 0.0)
     A[..., off.index((0, 0, 0))] = 128.0
-    A = A.reshape(-1, len(off))
+    return A.reshape(-1, len(off))
+
+
+@pytest.mark.parametrize("d,mask,prec", CASES)
+def test_wide_grids_equal_the_sequential_sweeps(S, orc, d, mask, prec):
+    off = {7: I.OFF7, 19: I.OFF19, 27: I.OFF27}[mask]
+    rng = np.random.default_rng(11)
+    A = matrix(d, off, rng)
     n = A.shape[0]
     dt = torch.float64 if prec == 0 else torch.float32
     dev = lambda v: torch.from_numpy(v).to(dt).cuda()
@@ -69,4 +75,51 @@ def test_wide_grids_equal_the_sequential_sweeps(S, orc, d, mask, prec):
     x = dev(u0)
     h.level_apply(0, S.OP_GS_BACKWARD, x=x, b=dev(b))
     assert err(x, orc.gs_backward(d, off, A, Dinv, b, u0)) <= TOL[prec]
+    h.close()
+
+
+@pytest.mark.parametrize("smoother,w", [("ILU0", 1.0), ("SGS", 1.0), ("SGS", 0.8)])
+@pytest.mark.parametrize("d,mask,prec", CASES + [((200, 200, 2), 27, 2), ((264, 104, 3), 19, 2)])  # BF16: 4, 4 and 4, 8
+def test_wide_cycles_equal_their_level_operations(S, d, mask, prec, smoother, w):
+    off = {7: I.OFF7, 19: I.OFF19, 27: I.OFF27}[mask]
+    rng = np.random.default_rng(13)
+    h = S.SMG(d, off, torch.from_numpy(matrix(d, off, rng)).cuda(), smoother=getattr(S, smoother), precision=prec,
+              krylov=S.PCG if prec == 0 else S.FPCG, transfer=S.C16XY, relax_w=w)
+    nl = h.stats()["levels"]
+    size = [int(np.prod(h.level_info(l)[0])) for l in range(nl)]
+    dt = torch.float64 if prec == 0 else torch.float32
+    new = lambda m: torch.zeros(m, dtype=dt, device="cuda")
+
+    def cycle(l, f):
+        n, u = size[l], new(size[l])
+        if l == nl - 1:
+            u = u.double()
+            h.level_apply(l, S.OP_COARSE_SOLVE, b=f.double(), y=u)
+            return u.to(dt)
+        t, c = new(n), new(size[l + 1])
+        if smoother == "ILU0":
+            h.level_apply(l, S.OP_ILU_APPLY, b=f, y=u)
+        else:
+            h.level_apply(l, S.OP_GS_ZERO, x=u, b=f)
+            h.level_apply(l, S.OP_GS_BACKWARD, x=u, b=f)
+        h.level_apply(l, S.OP_RESIDUAL, x=u, b=f, y=t)
+        h.level_apply(l, S.OP_RESTRICT, x=t, y=c)
+        h.level_apply(l, S.OP_PROLONG_ADD, x=cycle(l + 1, c), y=u)
+        if smoother == "ILU0":
+            e = new(n)
+            h.level_apply(l, S.OP_RESIDUAL, x=u, b=f, y=t)
+            h.level_apply(l, S.OP_ILU_APPLY, b=t, y=e)
+            u += e
+        else:
+            h.level_apply(l, S.OP_GS_FORWARD, x=u, b=f)
+            h.level_apply(l, S.OP_GS_BACKWARD, x=u, b=f)
+        return u
+
+    r = torch.from_numpy(rng.normal(size=size[0])).cuda()
+    z = torch.zeros_like(r)
+    h.vcycle(r, z)
+    u = cycle(0, r.to(dt)).double()
+    # per level six operations of at most 28 rounded terms each, of stored values
+    # that are the same in both; none amplifies (rows of 77/128)
+    assert torch.linalg.norm(z - u) <= 6 * 28 * EPS[prec] * nl * torch.linalg.norm(z)
     h.close()
