@@ -1,6 +1,6 @@
 // Software-pipelined wavefront sweeps for the standard masks (7, 19 and 27
-// points, one unknown per point): the same exact lexicographic order and the
-// same plane-per-CTA schedule as k_sweep.cu (t = SA*i + SB*j + k), with the
+// points, one unknown per point) in FP64 and natural order, on planes wider than
+// k_sweep3.cu takes: the same exact lexicographic order and the same plane-per-CTA schedule as k_sweep.cu (t = SA*i + SB*j + k), with the
 // per-step critical path cut to the few dependencies produced in the step
 // just before.
 //
@@ -69,12 +69,11 @@ struct Sweep2Params {
   Grid g;
   int G;
   unsigned long long budget_ns;
-  const void* M;
-  const float* scale;  // KBF row scale used by this sweep (A, L or U)
-  const void* dinv;
+  const double* M;
+  const double* dinv;
   double w;
-  const void* b;  // may alias u (in-place ILU solves)
-  void* u;
+  const double* b;  // may alias u (in-place ILU solves)
+  double* u;
   SweepWs* ws;
   int* err;
   int lin[27];  // linear index step of every entry on this grid
@@ -87,23 +86,21 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 constexpr int kMaxThreads = 512;
 constexpr int kPrefetch = 10;  // coefficient records prefetched into L2 this many points ahead
 
-template <int PK, int NS, int KIND, int DIR>
+template <int NS, int KIND, int DIR>
 __global__ void __launch_bounds__(kMaxThreads, 1) k_sweep2(Sweep2Params P) {
-  using V = typename Prec<PK>::vec;
-  using Val = typename Prec<PK>::val;
   using S = Shape<NS>;
   constexpr int SA = S::SA, SB = S::SB;
-  __shared__ V hist[4][kMaxThreads];
+  __shared__ double hist[4][kMaxThreads];
   __shared__ int s_plane, s_abort, s_last;
 
   const Grid g = P.g;
-  const Val* __restrict__ M = (const Val*)P.M;
-  const V* b = (const V*)P.b;
-  V* u = (V*)P.u;
-  const V* __restrict__ dinv = (const V*)P.dinv;
+  const double* __restrict__ M = P.M;
+  const double* b = P.b;
+  double* u = P.u;
+  const double* __restrict__ dinv = P.dinv;
   const int J = threadIdx.x;
   const bool relax = P.w != 1.0;
-  const V w = (V)P.w;
+  const double w = P.w;
 
   for (;;) {
     __syncthreads();
@@ -123,19 +120,17 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sweep2(Sweep2Params P) {
     int last_pub = t0;
 
     // stage B: raw loads for the point two steps ahead
-    Val cB[NS];
-    V mB[NS];
-    V bB = V(0), dB = V(0), uoB = V(0);
-    float sB = 1.0f;
+    double cB[NS];
+    double mB[NS];
+    double bB = 0.0, dB = 0.0, uoB = 0.0;
     // stage A: partial sum and late operands of the next point
-    V accA = V(0), bA = V(0), dA = V(0), uoA = V(0);
-    Val cOwnA = Val(0), cLateA = Val(0);
-    float sA = 1.0f;
-    V carry = V(0);
+    double accA = 0.0, bA = 0.0, dA = 0.0, uoA = 0.0;
+    double cOwnA = 0.0, cLateA = 0.0;
+    double carry = 0.0;
 #pragma unroll
     for (int e = 0; e < NS; ++e) {
-      cB[e] = Val(0);
-      mB[e] = V(0);
+      cB[e] = 0.0;
+      mB[e] = 0.0;
     }
 
     for (int t = t0 - 2; t <= t1; ++t) {
@@ -154,23 +149,22 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sweep2(Sweep2Params P) {
 
       // (1) finish point K
       if (colok && K >= 0 && K < g.nz) {
-        V s = accA;
+        double s = accA;
 #pragma unroll
         for (int e = 0; e < NS; ++e) {
-          if (cls<NS, KIND, DIR>(e) == C_OWN) s = fma((V)to_c(cOwnA), carry, s);
+          if (cls<NS, KIND, DIR>(e) == C_OWN) s = fma(cOwnA, carry, s);
           if (cls<NS, KIND, DIR>(e) == C_LATE) {
             const int kk = K + DIR * S::o(e, 2);  // schedule z of the neighbour
-            const V v = (J > 0 && kk >= 0 && kk < g.nz) ? hist[kk & 3][J - 1] : V(0);
-            s = fma((V)to_c(cLateA), v, s);
+            const double v = (J > 0 && kk >= 0 && kk < g.nz) ? hist[kk & 3][J - 1] : 0.0;
+            s = fma(cLateA, v, s);
           }
         }
-        if (PK == KBF) s = (V)sA * s;
-        V r;
+        double r;
         if (KIND == SW_ILU_L) {
           r = bA - s;
         } else {
           r = (bA - s) * dA;
-          if (KIND != SW_ILU_U && relax) r = (KIND == SW_GS_ZERO) ? w * r : (V(1) - w) * uoA + w * r;
+          if (KIND != SW_ILU_U && relax) r = (KIND == SW_GS_ZERO) ? w * r : (1.0 - w) * uoA + w * r;
         }
         const int k = DIR > 0 ? K : g.nz - 1 - K;
         u[((long long)i * g.ny + j) * g.nz + k] = r;
@@ -181,23 +175,23 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sweep2(Sweep2Params P) {
       // (2) partial sum of point K+1 from stage B and the early ring values
       const int K1 = K + 1;
       if (colok && K1 >= 0 && K1 < g.nz) {
-        V a0 = V(0), a1 = V(0), a2 = V(0), a3 = V(0);
+        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
         int q = 0;
 #pragma unroll
         for (int e = 0; e < NS; ++e) {
           const int c = cls<NS, KIND, DIR>(e);
-          V term_v = V(0);
+          double term_v = 0.0;
           bool has = false;
           if (c == C_MEM) {
             term_v = mB[e];
             has = true;
           } else if (c == C_EARLY) {
             const int kk = K1 + DIR * S::o(e, 2);
-            term_v = (J > 0 && kk >= 0 && kk < g.nz) ? hist[kk & 3][J - 1] : V(0);
+            term_v = (J > 0 && kk >= 0 && kk < g.nz) ? hist[kk & 3][J - 1] : 0.0;
             has = true;
           }
           if (has) {
-            const V cv = (V)to_c(cB[e]);
+            const double cv = cB[e];
             if ((q & 3) == 0) a0 = fma(cv, term_v, a0);
             else if ((q & 3) == 1) a1 = fma(cv, term_v, a1);
             else if ((q & 3) == 2) a2 = fma(cv, term_v, a2);
@@ -210,7 +204,6 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sweep2(Sweep2Params P) {
         accA = (a0 + a1) + (a2 + a3);
         bA = bB;
         dA = dB;
-        sA = sB;
         uoA = uoB;
       }
 
@@ -219,7 +212,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sweep2(Sweep2Params P) {
       if (colok && K2 >= 0 && K2 < g.nz) {
         const int k2 = DIR > 0 ? K2 : g.nz - 1 - K2;
         const long long p2 = ((long long)i * g.ny + j) * g.nz + k2;
-        const Val* a = M + p2 * NS;
+        const double* a = M + p2 * NS;
 #pragma unroll
         for (int e = 0; e < NS; ++e) {
           const int c = cls<NS, KIND, DIR>(e);
@@ -228,17 +221,16 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sweep2(Sweep2Params P) {
             const int ox = S::o(e, 0), oy = S::o(e, 1), oz = S::o(e, 2);
             const bool in = (unsigned)(i + ox) < (unsigned)g.nx && (unsigned)(j + oy) < (unsigned)g.ny &&
                             (unsigned)(k2 + oz) < (unsigned)g.nz;
-            mB[e] = in ? (ox != 0 ? __ldcg(u + p2 + P.lin[e]) : u[p2 + P.lin[e]]) : V(0);
+            mB[e] = in ? (ox != 0 ? __ldcg(u + p2 + P.lin[e]) : u[p2 + P.lin[e]]) : 0.0;
           }
         }
         bB = b[p2];
         if (KIND != SW_ILU_L) dB = dinv[p2];
-        if (PK == KBF) sB = P.scale[p2];
         if (KIND == SW_GS_FULL && relax) uoB = u[p2];
         if (K2 + kPrefetch < g.nz) {
           const char* pf = (const char*)(M + (p2 + DIR * kPrefetch) * NS);
           prefetch_l2(pf);
-          if (NS * sizeof(Val) > 128) prefetch_l2(pf + 128);
+          if (NS * sizeof(double) > 128) prefetch_l2(pf + 128);
         }
       }
     }
@@ -270,24 +262,24 @@ bool canonical(const Stencil& s) {
   return true;
 }
 
-template <int PK, int NS>
+template <int NS>
 void launch_kind(int kind, int dir, const Sweep2Params& P, int grid, int nthr, cudaStream_t st) {
-  if (kind == SW_GS_ZERO) k_sweep2<PK, NS, SW_GS_ZERO, 1><<<grid, nthr, 0, st>>>(P);
-  else if (kind == SW_ILU_L) k_sweep2<PK, NS, SW_ILU_L, 1><<<grid, nthr, 0, st>>>(P);
-  else if (kind == SW_ILU_U) k_sweep2<PK, NS, SW_ILU_U, -1><<<grid, nthr, 0, st>>>(P);
-  else if (dir > 0) k_sweep2<PK, NS, SW_GS_FULL, 1><<<grid, nthr, 0, st>>>(P);
-  else k_sweep2<PK, NS, SW_GS_FULL, -1><<<grid, nthr, 0, st>>>(P);
+  if (kind == SW_GS_ZERO) k_sweep2<NS, SW_GS_ZERO, 1><<<grid, nthr, 0, st>>>(P);
+  else if (kind == SW_ILU_L) k_sweep2<NS, SW_ILU_L, 1><<<grid, nthr, 0, st>>>(P);
+  else if (kind == SW_ILU_U) k_sweep2<NS, SW_ILU_U, -1><<<grid, nthr, 0, st>>>(P);
+  else if (dir > 0) k_sweep2<NS, SW_GS_FULL, 1><<<grid, nthr, 0, st>>>(P);
+  else k_sweep2<NS, SW_GS_FULL, -1><<<grid, nthr, 0, st>>>(P);
 }
 
 }  // namespace
 
 // Returns cudaErrorNotSupported (nothing launched) when the level is not one
-// this kernel handles: 3 unknowns per point, ny > 512, or a mask other than
-// the lexicographic 7-, 19- or 27-point one.
-cudaError_t launch_sweep2(const LevelView& L, int kind, int dir, const void* M, const float* sc1, const float* sc2,
-                          const void* dinv, double w, const void* b, void* u, SweepWs* ws, int* err,
-                          const SweepCfg& cfg, cudaStream_t st) {
-  if (L.B != 1 || L.g.ny > kMaxThreads) return cudaErrorNotSupported;
+// this kernel handles: reduced precision (whose levels with these masks run the
+// sheared wavefront), 3 unknowns per point, ny > 512, or a mask other than the
+// lexicographic 7-, 19- or 27-point one.
+cudaError_t launch_sweep2(const LevelView& L, int kind, int dir, const void* M, const void* dinv, double w,
+                          const void* b, void* u, SweepWs* ws, int* err, const SweepCfg& cfg, cudaStream_t st) {
+  if (L.B != 1 || L.pk != K64 || L.g.ny > kMaxThreads) return cudaErrorNotSupported;
   const int ns = L.s.ns;
   if (!((ns == 27 && canonical<27>(L.s)) || (ns == 7 && canonical<7>(L.s)) || (ns == 19 && canonical<19>(L.s))))
     return cudaErrorNotSupported;
@@ -295,27 +287,19 @@ cudaError_t launch_sweep2(const LevelView& L, int kind, int dir, const void* M, 
   P.g = L.g;
   P.G = cfg.G;
   P.budget_ns = cfg.budget_ns;
-  P.M = M;
-  P.scale = kind == SW_ILU_U ? sc2 : sc1;
-  P.dinv = dinv;
+  P.M = (const double*)M;
+  P.dinv = (const double*)dinv;
   P.w = w;
-  P.b = b;
-  P.u = u;
+  P.b = (const double*)b;
+  P.u = (double*)u;
   P.ws = ws;
   P.err = err;
   for (int e = 0; e < 27; ++e) P.lin[e] = L.s.lin[e];
   const int nthr = ((L.g.ny + 31) / 32) * 32;
   const int grid = L.g.nx;
-#define DISPATCH(PK)                                                        \
-  do {                                                                      \
-    if (ns == 27) launch_kind<PK, 27>(kind, dir, P, grid, nthr, st);       \
-    else if (ns == 7) launch_kind<PK, 7>(kind, dir, P, grid, nthr, st);    \
-    else launch_kind<PK, 19>(kind, dir, P, grid, nthr, st);                \
-  } while (0)
-  if (L.pk == K64) DISPATCH(K64);
-  else if (L.pk == K32) DISPATCH(K32);
-  else DISPATCH(KBF);
-#undef DISPATCH
+  if (ns == 27) launch_kind<27>(kind, dir, P, grid, nthr, st);
+  else if (ns == 7) launch_kind<7>(kind, dir, P, grid, nthr, st);
+  else launch_kind<19>(kind, dir, P, grid, nthr, st);
   smg_count_launch(1);
   return cudaGetLastError();
 }

@@ -176,11 +176,10 @@ cudaError_t launch_sweep(const LevelView& L, int kind, int dir, const void* M, c
                          const SweepCfg& cfg, cudaStream_t st);
 
 // Software-pipelined variant for the lexicographic 7/19/27-point masks with
-// one unknown per point; returns cudaErrorNotSupported (nothing launched) for
-// any other level, which launch_sweep then runs with the generic kernel.
-cudaError_t launch_sweep2(const LevelView& L, int kind, int dir, const void* M, const float* sc1, const float* sc2,
-                          const void* dinv, double w, const void* b, void* u, SweepWs* ws, int* err,
-                          const SweepCfg& cfg, cudaStream_t st);
+// one unknown per point, FP64; returns cudaErrorNotSupported (nothing launched)
+// for any other level, which launch_sweep then runs with the generic kernel.
+cudaError_t launch_sweep2(const LevelView& L, int kind, int dir, const void* M, const void* dinv, double w,
+                          const void* b, void* u, SweepWs* ws, int* err, const SweepCfg& cfg, cudaStream_t st);
 
 // Warp-pipelined variant on natural-order FP64 data (same masks, at most 12
 // warps of columns); cudaErrorNotSupported (nothing launched) otherwise.

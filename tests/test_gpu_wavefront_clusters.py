@@ -23,7 +23,8 @@ CASES = [((200, 200, 2), 27, 0),   # 4, 4
          ((336, 328, 2), 27, 1),   # 8, 4
          ((152, 280, 3), 7, 1),    # 4, 4
          ((96, 88, 4), 19, 1),     # 4, 8
-         ((72, 64, 3), 27, 0)]     # 2, 8
+         ((72, 64, 3), 27, 0),     # 2, 8
+         ((24, 400, 3), 27, 0)]    # 2, 8; its level operations run in natural order
 
 
 @pytest.fixture(scope="module")
