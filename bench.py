@@ -101,14 +101,11 @@ FP64_PROBE = os.path.join(ROOT, "profiles", "fp64_fma_peak_gb300.txt")
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per point of the
 # dominant kernel, from one ncu capture of the current kernel on the same
 # problem family at a smaller size (the traffic grows with the points); keyed
-# by (kernel, smoother, stencil points, precision).  Those below are of the
-# plane-per-CTA sweeps, kept to compare with; no entry where no capture of the
-# kernel that runs exists.
+# by (kernel, smoother, stencil points, precision).  No entry where no capture
+# of the kernel that runs exists.
 TRAFFIC_PER_POINT = {
-    # k_sweep3 ILU lower solve, FP64, 27 points: 268.97 MB for 128^3
-    ("k_sweep3", 1, 27, 0): (268.970e6 / 128 ** 3, "profiles/k_sweep3_ilu_lower_aniso27_128cubed.md"),
-    # k_sweep3h (two warps per strip), same solve: 268.25 MB for 128^3
-    ("k_sweep3h", 1, 27, 0): (268.252e6 / 128 ** 3, "profiles/k_sweep3h_ilu_lower_aniso27_128cubed.md"),
+    # k_tri ILU lower solve, FP64, 27 points: 334.47 MB for 128^3
+    ("k_tri", 1, 27, 0): (334.473e6 / 128 ** 3, "profiles/k_tri_ilu_lower_aniso27_128cubed.md"),
 }
 
 
@@ -425,11 +422,11 @@ def run_ours(args, w, rank, world):
         fac_pt = 8.0 * ((m - 1) * 5 + 3 + 2 * (4 + lw.bit_length())) * 32 * lw / nz
         flops_pt, bytes_pt = 2 * (nlow - 1) + 10, nlow * cbytes + fac_pt + 2 * vbytes
     elif w["smoother"] == 1:
-        kfile = "k_tri" if lvl0_warps else "k_sweep2"
+        kfile = "k_tri" if lvl0_warps else "k_sweep"
         kname = "%s (ILU(0) lower solve, level 0)" % kfile
         flops_pt, bytes_pt = 2 * nlow + 1, nlow * cbytes + 2 * vbytes + sbytes
     else:
-        kfile = ("k_tri" if lvl0_warps else "k_sweep2") if B == 1 else "k_btri"
+        kfile = ("k_tri" if lvl0_warps else "k_sweep") if B == 1 else "k_btri"
         kname = "%s (Gauss-Seidel zero-guess forward, level 0)" % kfile
         flops_pt = (2 * nlow + 2) * B * B
         bytes_pt = nlow * cbytes * B * B + vbytes * B * B + 2 * vbytes * B + sbytes

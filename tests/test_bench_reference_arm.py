@@ -42,8 +42,10 @@ def test_every_workload_has_a_label():
 def test_traffic_constants_trace_to_the_committed_profiles():
     """Every DRAM-bytes-per-point constant bench.py reports as
     roofline.traffic is the dram read + write of the ncu summary it cites,
-    divided by the points of that capture (128^3), and stays within 1.2x of
-    the kernel's algorithmic bytes (a larger figure would mean re-reads)."""
+    divided by the points of that capture (128^3), and stays within the bytes
+    that the kernel copies: a tile of two planes takes 128 + 64 steps for its 128
+    rows, so it reads records and right-hand side at most 1.5 times (a larger
+    figure would mean other re-reads)."""
     import importlib.util
     import re
     spec = importlib.util.spec_from_file_location("bench_mod", os.path.join(ROOT, "bench.py"))
@@ -62,5 +64,6 @@ def test_traffic_constants_trace_to_the_committed_profiles():
         # ILU(0) lower solve: n_low coefficients + b + u per point
         assert smoother == 1 and ns == 27
         c = {0: 8, 1: 4, 2: 2}[prec]
-        algorithmic = 13 * c + 2 * (8 if prec == 0 else 4) + (4 if prec == 2 else 0)
-        assert algorithmic <= per_point <= 1.2 * algorithmic, (src, per_point, algorithmic)
+        v = 8 if prec == 0 else 4
+        algorithmic = 13 * c + 2 * v + (4 if prec == 2 else 0)
+        assert algorithmic <= per_point <= 1.5 * (algorithmic - v) + v, (src, per_point, algorithmic)
