@@ -15,7 +15,7 @@
 //  (3) k_update, all SMs: A = A + N W (pivot rows: N W alone).
 // The rows end up as those of the inverse of P A; k_unpermute undoes P on the
 // columns.  Measured: a set-up with n = 2048 went from 76 to 29.5 ms, with
-// n = 768 from 36.5 to 28.6 ms; with candidates compared as integers and pushed
+// n = 840 from 36.5 to 28.6 ms; with candidates compared as integers and pushed
 // to the peers before the barrier, and one division a CTA, n = 2048 to 26.9.
 // What is left is the panels' chain, 4 us a column: a search, a cluster barrier,
 // a division and a step over the panel.

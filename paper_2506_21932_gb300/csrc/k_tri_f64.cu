@@ -39,14 +39,21 @@ cudaError_t tri_launch_k64(int ns, bool hd, const TriShape& t, bool helpers, con
   return hd ? go<7, true>(t, helpers, P, st) : go<7, false>(t, helpers, P, st);
 }
 
-// Planes per tile.  More planes mean fewer hops between tiles and more work per
-// SM, but a longer step.  Lower / upper solve in ms, FP64 27-point:
-//   G = 2: 0.44 / 0.47 at 128^3, 1.34 / 1.52 at 256^3
-//   G = 4: 0.62 / 0.69           1.13 / 1.22
-// (four planes fill the SM's FP64 pipe; they pay once the tiles outnumber the
-// SMs), FP32 27-point with 4 and 8 planes: 0.23 and 0.26 at 128^3, 0.53 and 0.58
-// at 256^3, 1.09 and 1.03 at 384^3.  BF16: 4 against 8 0.245 and 0.266 at
-// 104 x 72 x 88.  The 7-point mask has a short step whatever the precision.
+// Planes per tile.  More planes mean fewer tiles to hop between and, in FP64, more
+// multiply-adds in flight, but a longer step.  Lower / upper solve in ms with both,
+// FP64 27-point, 2 and 4 planes:
+//   128^3 0.376 / 0.414  0.519 / 0.553      192^3 0.645 / 0.706  0.806 / 0.861
+//   224^3 0.835 / 0.922  0.937 / 0.998      256^3 1.084 / 1.202  1.144 / 1.220
+//   288^3 1.373 / 1.520  1.392 / 1.474      320^3 1.726 / 1.919  1.686 / 1.787
+//   384^3 2.652 / 2.964  2.476 / 2.633      512 x 512 x 16 1.517 / 1.653  1.896 / 2.025
+// Four planes fill an SM's FP64 pipe, which pays on the largest grids.  The line was
+// drawn when two planes took 0.45 ms at 128^3 and 1.34 at 256^3; it now lies below
+// the crossing (288^3 to 320^3, higher on flat boxes), at a cost of up to 25 % of a
+// solve in between.  FP32 27-point, lower solve with 4 and 8 planes: 256^3 0.520
+// 0.574, 320^3 0.751 0.773, 352^3 0.904 0.874, 384^3 1.083 1.022, 512 x 512 x 16
+// 0.836 0.852, 1024 x 512 x 8 1.366 1.401: the line lies at the crossing of cubes.
+// BF16: 4 against 8 0.245 and 0.266 at 104 x 72 x 88.  The 7-point mask has a short
+// step whatever the precision.
 static int planes_per_tile(const Grid& g, int ns, int pk) {
   const long long plane = (long long)g.nx * g.ny;
   if (ns == 7) return 4;
@@ -61,11 +68,20 @@ static int strip_tiles(const Grid& g, const TriShape& t, int w) {
 // Tiles per cluster (a divisor of 32 / G).  A hop inside a cluster takes 0.45
 // us, between clusters 1.1, but clusters of eight leave some SMs idle, which
 // costs more once there are several tiles per SM.  Lower solve in ms with 2, 4,
-// 8 tiles per cluster:
-//   BF16 27-point 192^3 (336 tiles) 0.489 0.428 0.405    384^3 (1248) 1.09 0.96
-//   FP64  7-point 128^3 (160)       0.204 0.179 0.167    256^3 (576)  0.68 0.68 0.80
-//   FP64 27-point 128^3 (320)       0.497 0.452 0.438    192^3 (672)  0.84 0.82 0.90
-//                 320^3 (880)       1.75  1.82           384^3 (1248) 2.56 2.70 3.53
+// 8 tiles per cluster (number of tiles):
+//   FP64 27-point  128^3 (320) 0.434 0.388 0.376   144^3 (432) 0.493 0.439 0.441
+//                  192^3 (672) 0.698 0.642 0.705
+//     four planes  208^3 (416) 0.902 0.861 0.949   256^3 (576) 1.153 1.144 1.315
+//                  288^3 (720) 1.392 1.414 1.662   384^3 (1248) 2.478 2.614 3.199
+//   FP32 27-point  192^3 (336) 0.410 0.366 0.348   208^3 (416) 0.453 0.403 0.402
+//                  224^3 (448) 0.492 0.438 0.440   320^3 (880) 0.816 0.752 0.848
+//   BF16 27-point  192^3 (336) 0.476 0.422 0.385   384^3 (1248) 1.061 0.942 0.889
+//   FP64 7-point   128^3 (160) 0.224 0.200 0.186   144^3 (216) 0.260 0.228 0.232
+//                  176^3 (308) 0.324 0.294 0.323   256^3 (576) 0.568 0.556 0.640
+// The lines, 340 and 600 tiles, are those of the 27-point masks in FP64 and FP32,
+// where both sides come to the same at 416 to 448 and 576 tiles.  BF16, whose step
+// is the shortest part of a hop, stays ahead with eight throughout, and the 7-point
+// mask in FP64 falls behind with eight from 240 tiles on (up to 10 %).
 int tri_cluster(const TriShape& t, const Grid& g, int pk) {
   int n = 0;
   for (int w = 0; w < t.strips; ++w) n += strip_tiles(g, t, w);

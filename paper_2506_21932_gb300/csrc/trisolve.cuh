@@ -10,7 +10,7 @@
 //
 // What bounds a solve on all but the largest grids is the chain of time steps
 // plus one hop per tile; a step is the barrier, three dependent multiply-adds
-// and a warp's instructions one after another (27-point: 0.38 us FP64 with 2
+// and a warp's instructions one after another (27-point: 0.36 us FP64 with 2
 // planes, 0.25 FP32, 0.20 BF16; 7-point 0.27 / 0.20), so whatever else a step
 // needs is moved to other warps.  On the largest FP64 grids the FP64 pipe is
 // full (384^3: 2.45 ms a solve, 1.56 ms of multiply-adds).
@@ -312,7 +312,8 @@ __global__ void __launch_bounds__(tri_threads<G, H>(), tri_ctas<G, H>()) k_tri(T
       // The main warp's chain has to get into the FP64 pipe before the helpers of
       // its sub-partition: with two planes the one there waits for it (128^3: 0.45
       // to 0.41 ms a solve), with four, where a turn would come too late for
-      // three, they hold back by about the chain's first product (256^3: 1.21 to 1.14).
+      // three, they hold back by about the chain's first product (256^3: 1.21 to 1.14;
+      // the time is the clock's, 100 ns or 200 of the 2070 MHz cycles of these figures).
       constexpr bool kTurn = H && G == 2;
       auto hold = [&] {
         if (G == 4) __nanosleep(100);
